@@ -101,20 +101,22 @@ typedef enum {
     STENCIL_KERNEL_TC = 3,         /* tensor cores: tcgen05 where it applies, else warp MMA */
     STENCIL_KERNEL_TC_WARP = 4,    /* tensor cores, warp-MMA engine only             */
     STENCIL_KERNEL_TC_UMMA = 5,    /* tensor cores, tcgen05 engine (UNSUPPORTED where it does not apply) */
-    STENCIL_KERNEL_RESIDENT = 6,   /* small grids: the whole grid in one thread-block cluster's shared
-                                      memory, every step of a run in one launch                        */
+    STENCIL_KERNEL_RESIDENT = 6,   /* small grids: the whole grid on the chip (register tiles on every SM,
+                                      or one cluster's shared memory), every step in one launch        */
     STENCIL_KERNEL_LOWRANK = 7     /* chosen by compute = LOWRANK (reported by stencil_plan_info only) */
 } stencil_kernel_t;
 
 /* Optional plan settings; pass NULL for defaults.  0 means "choose".
- * kernel = AUTO with FP32 arithmetic picks RESIDENT when the grid fits one
- * cluster (two FP32 copies in the shared memory of at most 16 CTAs; roughly up
- * to 700 x 700 for radius 1) and no streaming-kernel option (tb_depth,
- * threads, tile_rows) is set; otherwise STREAM.  With autotune the first run
- * times both (and, for RESIDENT, every cluster size and blocking depth).  With
- * kernel = RESIDENT, tb_depth sets its steps per halo exchange (default 1).
- * stencil_plan_info reports tb_depth = 0 for RESIDENT (one launch per run),
- * ctas = the cluster size and tile_rows = the slab height. */
+ * kernel = AUTO with FP32 arithmetic picks RESIDENT when the grid fits on the
+ * chip, as one register tile per SM (roughly up to 1500 x 1500 for radius 1)
+ * or else in one cluster (two FP32 copies in the shared memory of at most 16
+ * CTAs), and no streaming-kernel option (tb_depth, threads, tile_rows) is set;
+ * otherwise STREAM.  With autotune the first run times them all (for one
+ * cluster, every cluster size and blocking depth).  kernel = RESIDENT asks for
+ * the one-cluster form; tb_depth then sets its steps per halo exchange
+ * (default 1).  stencil_plan_info reports tb_depth = 0 for RESIDENT (one launch
+ * per run), ctas = the cluster size (1 for register tiles, whose CTAs are not
+ * clustered) and tile_rows = the height of a slab or tile. */
 typedef struct {
     int compute;      /* stencil_compute_t                                          */
     int kernel;       /* stencil_kernel_t                                           */
@@ -126,13 +128,13 @@ typedef struct {
                          16, 32 (TF32): one weight row per MMA, 128 x 128 output
                          tiles; 96 or 128: three or four weight rows stacked in one
                          MMA over 32-column N-tiles, 126- or 125-row output tiles   */
-    int timeout_ms;   /* tcgen05 engine and TMA-fed streaming kernel: limit of each
-                         device-side wait in ms (0 = 2000)                             */
+    int timeout_ms;   /* tcgen05 engine, TMA-fed streaming kernel and register tiles: limit
+                         of each device-side wait in ms (0 = 2000)                     */
     int debug_withhold; /* test hook, 0 in normal use: 1 makes CTA 0 of the tcgen05
                            engine withhold its first accumulator-ready signal, and CTA 0
                            of the TMA-fed streaming kernel wait for 16 bytes more than
-                           its first row brings, so a wait runs out and the run
-                           reports TIMEOUT                                             */
+                           its first row brings, and register tile 0 leave its border
+                           unmarked, so a wait runs out and the run reports TIMEOUT    */
     int load;         /* streaming kernel's input rows: stencil_load_t                */
     int rank;         /* compute = LOWRANK: separable terms kept (0 = numerical rank,
                          else 1..2r+1)                                                 */

@@ -22,6 +22,7 @@
 #include "../../include/stencil.h"
 #include "common.cuh"
 #include "stream_depths.h"
+#include "sweep_grid.h"
 #include "sweep_stream.cuh"
 
 namespace gbst {
@@ -110,6 +111,10 @@ struct stencil_plan {
     // cluster-resident kernel (sweep_resident.cu): usable cluster sizes (bit log2 C), the one in use
     const void* res_fn = nullptr;
     int res_ok = 0, res_c = 0, res_rp = 0, res_kb = 1, res_smem = 0, res_max_smem = 0;
+    // chip-resident register tiles (sweep_grid.cuh): usable, in use (kernel == RESIDENT then), scratch
+    int grid_ok = 0, grid_on = 0;
+    GridConfig grid;
+    void* grid_mem = nullptr;
     unsigned smem_set = 0;  // bit 2k+vec: that kernel's shared-memory attribute is set
     int tuned = 0;
     const void* naive = nullptr;
@@ -301,6 +306,7 @@ static stencil_status_t configure_stream(stencil_plan* p, int k, int threads, in
     }
     if (strips * tiles_y > 0x7fffffffLL) return fail(STENCIL_ERR_UNSUPPORTED, "grid too large");
     p->kernel = STENCIL_KERNEL_STREAM;
+    p->grid_on = 0;
     p->k = k;
     p->threads = nt;
     p->H = H;
@@ -454,11 +460,41 @@ static stencil_status_t use_resident(stencil_plan* p, int C, int kb = 1) {
     CK(cudaFuncSetAttribute(p->res_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     if (C > 8) CK(cudaFuncSetAttribute(p->res_fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     p->kernel = STENCIL_KERNEL_RESIDENT;
+    p->grid_on = 0;
     p->res_c = C;
     p->res_rp = rp;
     p->res_kb = kb;
     p->res_smem = smem;
     return STENCIL_OK;
+}
+
+// The chip-resident register-tile kernel: one tile per SM over the whole chip.
+// AUTO takes it wherever a configuration fits, in place of the cluster-resident
+// kernel (at most 16 SMs) and of the streaming kernel (launches).  It was the
+// faster one at every size it takes, from a 4-step run on: 96 steps in us,
+// register tiles | streaming kernel, FP32 on GB300: 5-point star 300^2 47 | 235,
+// 1000^2 83 | 248, 1500^2 (about the largest) 151 | 273; 9-point box 57 | 298,
+// 111 | 322, 212 | 371; 13-point star 97 | 658, 211 | 658, 1400^2 423 | 725; 7x7
+// box 183 | 1478, 433 | 1379, 1400^2 743 | 1575; 4 steps 11-38 | 16-67.  Against
+// the cluster-resident kernel: 512^2 5-point star, 100 steps, 52 | 219 (FP32);
+// 130 x 517 13-point star, 20 steps, 24 | 74.  A plan the caller steers (kernel,
+// tb_depth, threads, tile_rows or load set) keeps what it asked for.
+static bool grid_candidate(stencil_plan* p) {
+    if (p->compute != STENCIL_COMPUTE_FP32 || p->ny > (1 << 20) || p->nx > (1 << 20)) return false;
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, p->device) != cudaSuccess || !coop) {
+        cudaGetLastError();
+        return false;
+    }
+    const int periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
+    if (!grid_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, 0, 0, &p->grid)) return false;
+    p->grid_ok = grid_fits(p->grid, p->R, p->star, p->sms);
+    return p->grid_ok != 0;
+}
+
+static void use_grid(stencil_plan* p) {
+    p->kernel = STENCIL_KERNEL_RESIDENT;
+    p->grid_on = 1;
 }
 
 static stencil_status_t configure_naive(stencil_plan* p) {
@@ -533,6 +569,27 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
         } else {
             CK(cudaLaunchKernel(p->naive, dim3((unsigned)tp.tiles), dim3(256), args, (size_t)p->smem, st));
         }
+        return STENCIL_OK;
+    }
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on) {
+        const size_t vec_bytes = 4 * p->elem;
+        const int vec = p->nx % 4 == 0 && (uintptr_t)src % vec_bytes == 0 && (uintptr_t)dst % vec_bytes == 0;
+        // In place, a tile may only write once its neighbours have read: at least
+        // one exchange (a single step in place is staged by the caller).
+        int k = p->grid.k;
+        if (src == dst) k = std::min(k, (nlev + 1) / 2);
+        const cudaError_t e =
+            launch_grid(p->grid, p->R, p->star, p->dtype, p->boundary == STENCIL_BOUNDARY_PERIODIC, src, dst,
+                        (int)p->ny, (int)p->nx, vec, nlev, k, p->grid_mem, p->status,
+                        (long long)(p->opt.timeout_ms > 0 ? p->opt.timeout_ms : 2000) * 1000000LL,
+                        p->opt.debug_withhold, p->w, st);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs than the device reports (a partition)
+            cudaGetLastError();
+            p->grid_on = p->grid_ok = 0;
+            p->kernel = STENCIL_KERNEL_STREAM;
+            return fail(STENCIL_ERR_UNSUPPORTED, "the chip-resident tiles do not fit at once");
+        }
+        CK(e);
         return STENCIL_OK;
     }
     if (p->kernel == STENCIL_KERNEL_RESIDENT) {
@@ -851,14 +908,16 @@ static stencil_status_t autotune(stencil_plan* p, const void* in, cudaStream_t s
     return STENCIL_OK;
 }
 
-// Small grids (plans that chose the cluster-resident kernel): time that kernel
-// at every usable cluster size (runs of 64 steps from `in` into the workspace)
-// and the autotuned streaming kernel, per step, and keep the faster.  The
+// Small grids (plans that chose a resident kernel): time the chip-resident
+// kernel, the cluster-resident one at every usable cluster size (runs of 64
+// steps from `in` into the workspace) and the autotuned streaming kernel, per step, and keep the faster.  The
 // decision is cached like the streaming kernel's.
-static std::map<TuneKey, int> g_res_tune_cache;  // 16 * kb + log2(C) + 1, or 0 for the streaming kernel
+static std::map<TuneKey, int> g_res_tune_cache;  // 16 * kb + log2(C) + 1, kTuneGrid, or 0 for the streaming kernel
+static const int kTuneGrid = 1 << 20;
 
 static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaStream_t st) {
-    const TuneKey key(p->ny, p->nx, p->R, p->star, p->dtype, p->boundary, p->device);
+    // (plans that asked for the cluster-resident kernel have no chip-resident candidate)
+    const TuneKey key(p->ny, p->nx, p->R + 16 * p->grid_ok, p->star, p->dtype, p->boundary, p->device);
     int decision = -1;
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
@@ -870,6 +929,36 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
         const int reps = (int)std::max(2.0, std::min(16.0, 1e8 / ((double)p->ny * (double)p->nx * S)));
         float best = 1e30f;
         decision = 0;
+        // S steps from `in` into the workspace with the resident kernel in use.
+        auto try_resident = [&](int code) -> stencil_status_t {
+            cudaEvent_t e0, e1;
+            CK(cudaEventCreate(&e0));
+            CK(cudaEventCreate(&e1));
+            stencil_status_t s = launch_once(p, in, p->ws, S, st);  // warm-up
+            if (s == STENCIL_OK) {
+                cudaEventRecord(e0, st);
+                for (int i = 0; i < reps && s == STENCIL_OK; ++i) s = launch_once(p, in, p->ws, S, st);
+                cudaEventRecord(e1, st);
+            }
+            cudaError_t e = cudaEventSynchronize(e1);
+            float ms = 0.f;
+            if (s == STENCIL_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+            cudaEventDestroy(e0);
+            cudaEventDestroy(e1);
+            if (s != STENCIL_OK) return s;
+            if (e != cudaSuccess) return fail(STENCIL_ERR_CUDA, std::string("autotune timing: ") + cudaGetErrorString(e));
+            const float per_step = ms / (float)(reps * S);
+            if (per_step < best) {
+                best = per_step;
+                decision = code;
+            }
+            return STENCIL_OK;
+        };
+        if (p->grid_ok) {
+            use_grid(p);
+            stencil_status_t s = try_resident(kTuneGrid);
+            if (s != STENCIL_OK) return s;
+        }
         for (int lg = 0; (1 << lg) <= resident_max_cluster(); ++lg) {
             if (!((p->res_ok >> lg) & 1)) continue;
             for (int kb = 1; kb <= 8; kb *= 2) {
@@ -879,27 +968,8 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
                     continue;
                 stencil_status_t s = use_resident(p, 1 << lg, kb);
                 if (s != STENCIL_OK) return s;
-                cudaEvent_t e0, e1;
-                CK(cudaEventCreate(&e0));
-                CK(cudaEventCreate(&e1));
-                s = launch_once(p, in, p->ws, S, st);  // warm-up
-                if (s == STENCIL_OK) {
-                    cudaEventRecord(e0, st);
-                    for (int i = 0; i < reps && s == STENCIL_OK; ++i) s = launch_once(p, in, p->ws, S, st);
-                    cudaEventRecord(e1, st);
-                }
-                cudaError_t e = cudaEventSynchronize(e1);
-                float ms = 0.f;
-                if (s == STENCIL_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
+                s = try_resident(16 * kb + lg + 1);
                 if (s != STENCIL_OK) return s;
-                if (e != cudaSuccess) return fail(STENCIL_ERR_CUDA, std::string("autotune timing: ") + cudaGetErrorString(e));
-                const float per_step = ms / (float)(reps * S);
-                if (per_step < best) {
-                    best = per_step;
-                    decision = 16 * kb + lg + 1;
-                }
             }
         }
         stencil_status_t s = autotune(p, in, st);  // configures the best streaming kernel
@@ -911,6 +981,10 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
         if (ms / (float)(sreps * p->k) < best) decision = 0;
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_res_tune_cache[key] = decision;
+    }
+    if (decision == kTuneGrid) {
+        use_grid(p);
+        return STENCIL_OK;
     }
     if (decision > 0) return use_resident(p, 1 << ((decision & 15) - 1), decision >> 4);
     return autotune(p, in, st);
@@ -934,6 +1008,22 @@ const char* stencil_status_string(stencil_status_t s) {
 const char* stencil_last_error(void) { return g_last_error.c_str(); }
 
 int stencil_version(void) { return 100; }
+
+// Clear device memory before returning, without touching the caller's streams:
+// a first run on any stream must see it cleared.
+// (One stream per device, kept for the life of the process: creating one per
+// plan cost more than the rest of the call.)
+static cudaError_t zero_now(int device, void* ptr, size_t bytes) {
+    static std::mutex mu;
+    static std::map<int, cudaStream_t> streams;
+    std::lock_guard<std::mutex> g(mu);
+    cudaStream_t& st = streams[device];
+    cudaError_t e = cudaSuccess;
+    if (!st) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ptr, 0, bytes, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e;
+}
 
 stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t nx, int radius,
                                      const float* weights, int dtype, int boundary,
@@ -998,6 +1088,22 @@ stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t n
         return fail(STENCIL_ERR_CUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
     }
 
+    // Small grids the chip-resident kernel does not take: the cluster-resident
+    // kernel, unless the caller asked for the streaming kernel or set one of its
+    // options.  With kernel = RESIDENT, tb_depth is its number of steps per halo exchange.
+    auto cluster_choice = [&](stencil_status_t st) -> stencil_status_t {
+        const bool stream_opts = o.tb_depth > 0 || o.threads > 0 || o.tile_rows > 0;
+        if (st == STENCIL_OK && (o.kernel == STENCIL_KERNEL_RESIDENT ||
+                                 (o.kernel == STENCIL_KERNEL_AUTO && !stream_opts))) {
+            const int kb = (o.kernel == STENCIL_KERNEL_RESIDENT && o.tb_depth > 0) ? o.tb_depth : 1;
+            const int C = resident_candidates(p, kb);
+            if (C > 0)
+                st = use_resident(p, C, kb);
+            else if (o.kernel == STENCIL_KERNEL_RESIDENT)
+                st = fail(STENCIL_ERR_UNSUPPORTED, "grid too large for the cluster-resident kernel at this depth");
+        }
+        return st;
+    };
     stencil_status_t st;
     const bool tc_kernel = o.kernel == STENCIL_KERNEL_TC || o.kernel == STENCIL_KERNEL_TC_WARP ||
                            o.kernel == STENCIL_KERNEL_TC_UMMA;
@@ -1017,24 +1123,40 @@ stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t n
         const int k0 = std::min(k, stream_kmax(radius, star));
         p->tma = o.load == STENCIL_LOAD_TMA || (o.load == STENCIL_LOAD_AUTO && tma_eligible(p) && kDefaultTma);
         st = configure_stream(p, k0, threads, o.tile_rows);
-        // Small grids: the cluster-resident kernel, unless the caller asked for
-        // the streaming kernel or set one of its options.
-        // With kernel = RESIDENT, tb_depth is its number of steps per halo exchange.
         const bool stream_opts = o.tb_depth > 0 || o.threads > 0 || o.tile_rows > 0;
-        if (st == STENCIL_OK && (o.kernel == STENCIL_KERNEL_RESIDENT ||
-                                 (o.kernel == STENCIL_KERNEL_AUTO && !stream_opts))) {
-            const int kb = (o.kernel == STENCIL_KERNEL_RESIDENT && o.tb_depth > 0) ? o.tb_depth : 1;
-            const int C = resident_candidates(p, kb);
-            if (C > 0)
-                st = use_resident(p, C, kb);
-            else if (o.kernel == STENCIL_KERNEL_RESIDENT)
-                st = fail(STENCIL_ERR_UNSUPPORTED, "grid too large for the cluster-resident kernel at this depth");
-        }
+        const bool may_grid = o.kernel == STENCIL_KERNEL_AUTO && !stream_opts && o.load == STENCIL_LOAD_AUTO;
+        if (st == STENCIL_OK && may_grid && grid_candidate(p)) use_grid(p);
+        if (st == STENCIL_OK && p->grid_on && o.autotune) resident_candidates(p);  // to be timed as well
+        if (!p->grid_on) st = cluster_choice(st);
     }
     if (st != STENCIL_OK) return bail(st);
 
+    // One block: the ping-pong workspace, then the chip-resident kernel's scratch.
     const size_t bytes = (size_t)ny * (size_t)nx * p->elem;
-    e = cudaMalloc(&p->ws, bytes);
+    if (p->grid_ok) {
+        const size_t off = (bytes + 255) / 256 * 256;
+        const size_t scratch = grid_scratch_bytes((int)ny, (int)nx);
+        e = cudaMalloc(&p->ws, off + scratch);
+        if (e == cudaSuccess) {
+            p->grid_mem = static_cast<char*>(p->ws) + off;
+            e = zero_now(p->device, p->grid_mem, scratch);
+            if (e != cudaSuccess) {
+                bail(STENCIL_ERR_CUDA);
+                return fail(STENCIL_ERR_CUDA, std::string("clearing the exchange grids: ") + cudaGetErrorString(e));
+            }
+        } else {  // no room for the exchange grids: the kernels that need none
+            cudaGetLastError();
+            p->ws = nullptr;
+            p->grid_ok = 0;
+            if (p->grid_on) {
+                p->grid_on = 0;
+                p->kernel = STENCIL_KERNEL_STREAM;
+                st = cluster_choice(STENCIL_OK);
+                if (st != STENCIL_OK) return bail(st);
+            }
+        }
+    }
+    if (!p->ws) e = cudaMalloc(&p->ws, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         p->ws = nullptr;
@@ -1111,11 +1233,20 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* p, stencil_plan_info_t*
     i.tile_rows = p->by;
     i.ctas = p->strips * p->tiles_y;
     i.smem_bytes = p->smem;
-    i.workspace_bytes = (int64_t)((size_t)p->ny * p->nx * p->elem);
+    i.workspace_bytes = (int64_t)((size_t)p->ny * p->nx * p->elem) +
+                        (p->grid_mem ? (int64_t)grid_scratch_bytes((int)p->ny, (int)p->nx) : 0);
     i.mma_n = p->umma_n;
     i.load = p->kernel == STENCIL_KERNEL_STREAM ? (p->tma ? STENCIL_LOAD_TMA : STENCIL_LOAD_CP_ASYNC) : 0;
     i.rank = p->kernel == STENCIL_KERNEL_LOWRANK ? p->lr_rank : 0;
-    if (p->kernel == STENCIL_KERNEL_RESIDENT) {
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on) {
+        i.tb_depth = 0;  // every step of a run in one launch
+        i.threads = 32 * p->grid.warps;
+        i.halo_cols = p->grid.H;
+        i.tile_cols = p->grid.bx;
+        i.tile_rows = p->grid.by;
+        i.ctas = 1;  // the cluster size: its CTAs, one per tile, are not clustered
+        i.smem_bytes = 0;
+    } else if (p->kernel == STENCIL_KERNEL_RESIDENT) {
         i.tb_depth = 0;  // every step of a run in one launch
         i.threads = resident_threads();
         i.halo_cols = p->R;
@@ -1169,10 +1300,19 @@ stencil_status_t stencil_run(stencil_plan_t* p, const void* in, void* out, int64
     }
     std::vector<int> depths = launch_depths(p, T);
     const void* src = in;
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && in == out && T == 1) {
+        // a single step in place has no exchange that orders the reads before the writes
+        CK(cudaMemcpyAsync(p->ws, in, bytes, cudaMemcpyDeviceToDevice, st));
+        src = p->ws;
+    }
     if (p->kernel == STENCIL_KERNEL_RESIDENT) {
         // one launch reads all of its input before it writes any output
         for (size_t i = 0; i < depths.size(); ++i) {
             stencil_status_t s = launch_once(p, src, out, depths[i], st);
+            if (s == STENCIL_ERR_UNSUPPORTED && p->kernel == STENCIL_KERNEL_STREAM) {
+                // (nothing was launched: the streaming kernel takes the run)
+                return stencil_run(p, src == p->ws ? in : src, out, T - (int64_t)i * (1 << 30), stream);
+            }
             if (s != STENCIL_OK) return s;
             src = out;
         }

@@ -1,0 +1,143 @@
+"""GPU tests of the chip-resident register-tile kernel (AUTO plans of grids that
+fit the chip as one tile per SM).
+
+It computes the same products in the same order as the streaming kernel, so
+FP32 results are compared bit for bit (periodic widths that are not a multiple
+of 4: to FP32 rounding, as for the streaming kernel's own depths); 16-bit
+storage is rounded only at the end, so its results are the rounded FP32 ones.
+"""
+import numpy as np
+import pytest
+
+from paper_2605_07954_gb300 import inputs
+from _util import fp32_tol, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TDT = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_07954_gb300 import build
+    build.build()
+
+
+def _weights(name):
+    if name in ("star9", "box25"):
+        return inputs.random_weights("star" if name == "star9" else "box", 2)
+    return inputs.pattern_weights(name)
+
+
+def _plan(shape, W, grid=True, **kw):
+    from paper_2605_07954_gb300 import Plan
+    p = Plan(shape[0], shape[1], W, **kw)
+    if grid:
+        i = p.info()
+        assert i["kernel"] == 6 and i["ctas"] == 1 and i["halo_cols"] % 4 == 0, i
+    return p
+
+
+# One tile, one strip, one tile row, chunks and warps cut by the grid's edge,
+# widths around the 128 staged columns, and about the largest grids that fit.
+SHAPES = [(1, 1), (2, 3), (1, 700), (700, 1), (127, 128), (33, 129), (130, 517), (301, 252), (512, 512),
+          (1000, 1022), (1201, 1100)]
+
+
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+@pytest.mark.parametrize("name", ["heat5", "box9", "star9", "box25", "star13", "box49"])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_same_bits_as_streaming_kernel(name, shape, boundary):
+    W = _weights(name)
+    x = torch.from_numpy(inputs.field(*shape)).cuda()
+    p = _plan(shape, W, boundary=boundary)
+    q = _plan(shape, W, grid=False, boundary=boundary, kernel="stream")
+    for T in (1, 2, 7, 33):
+        y, z = p.run(x, T), q.run(x, T)
+        torch.cuda.synchronize()
+        p.status()
+        if boundary == "periodic" and shape[1] % 4:
+            assert rel_l2(y.cpu().numpy(), z.cpu().numpy().astype(np.float64)) <= fp32_tol(T), T
+        else:
+            assert torch.equal(y, z), T
+    p.close()
+    q.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("shape", [(200, 336), (131, 333)])
+def test_16_bit_storage_rounds_once(dtype, shape):
+    W = inputs.pattern_weights("box9")
+    x = torch.from_numpy(inputs.field(*shape)).cuda().to(TDT[dtype])
+    y = _plan(shape, W, dtype=dtype).run(x, 40)
+    z = _plan(shape, W, grid=False, kernel="stream").run(x.float(), 40)
+    assert torch.equal(y, z.to(TDT[dtype]))
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 9, 40])
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+def test_in_place(T, boundary):
+    W = inputs.pattern_weights("star13")
+    p = _plan((300, 420), W, boundary=boundary)
+    x = torch.from_numpy(inputs.field(300, 420)).cuda()
+    z = x.clone()
+    y = p.run(x, T)
+    p.run(z, T, out=z)
+    assert torch.equal(y, z)
+
+
+def test_unaligned_buffers():
+    W = inputs.pattern_weights("box9")
+    p = _plan((64, 256), W)
+    f = torch.from_numpy(inputs.field(64, 256)).cuda()
+    buf = torch.empty(64 * 256 + 1, device="cuda")
+    x = buf[1:].view(64, 256)
+    x.copy_(f)
+    assert torch.equal(p.run(x, 13), p.run(f, 13))
+
+
+def test_replayed_graph_and_two_streams():
+    """Epochs count on from one launch to the next: a captured run replayed
+    several times, and two plans running on two streams at once."""
+    W = inputs.pattern_weights("heat5")
+    p, q = _plan((512, 512), W), _plan((400, 600), W)
+    x, y = torch.from_numpy(inputs.field(512, 512)).cuda(), torch.from_numpy(inputs.field(400, 600)).cuda()
+    want_x, want_y = p.run(x, 50), q.run(y, 70)
+    out = torch.empty_like(x)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s1):
+        p.run(x, 50, out=out)
+    for _ in range(5):
+        out.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s1):
+            g.replay()
+        with torch.cuda.stream(s2):
+            got_y = q.run(y, 70)
+        torch.cuda.synchronize()
+        assert torch.equal(out, want_x) and torch.equal(got_y, want_y)
+    p.status()
+    q.status()
+
+
+def test_expired_wait_reports_timeout_and_plan_recovers():
+    from paper_2605_07954_gb300 import StencilError
+    W = inputs.pattern_weights("heat5")
+    x = torch.from_numpy(inputs.field(512, 512)).cuda()
+    bad = _plan((512, 512), W, timeout_ms=100, debug_withhold=1)
+    bad.run(x, 60)
+    torch.cuda.synchronize()
+    with pytest.raises(StencilError, match="TIMEOUT"):
+        bad.status()
+    bad.run(x, 1)  # no exchange: nothing to wait for
+    bad.status()
+    good = _plan((512, 512), W)
+    ref = _plan((512, 512), W, grid=False, kernel="stream")
+    assert torch.equal(good.run(x, 60), ref.run(x, 60))
+    good.status()
