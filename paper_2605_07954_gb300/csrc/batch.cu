@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(kStreamMaxThreads)
         p.out = g.buf[(item.z + 1) & 1];
         p.ny = g.ny;
         p.nx = g.nx;
-        p.ld = g.ld;
+        p.ld = p.ld_out = g.ld;
+        p.dense_out = 0;
         p.nlev = K;
         p.H = g.H;
         p.bx = g.bx;

@@ -33,7 +33,9 @@ struct StreamParams {
     const void* in;
     void* out;
     long long ny, nx;
-    long long ld;   // row pitch of in and out, in elements (>= nx; a multiple of 4 when vec)
+    long long ld;   // row pitch of in, in elements (>= nx; a multiple of 4 when vec)
+    long long ld_out;  // row pitch of out (a multiple of 4 when vec, unless dense_out)
+    int dense_out;     // vec kernels: rows of out are not 16-byte aligned, stored element by element
     int nlev;      // time levels (Jacobi steps) this launch advances, 1..KMAX
     int H;         // halo columns loaded on each side of a strip (multiple of 4, >= R*nlev)
     int bx;        // output columns per strip (multiple of 4)

@@ -32,6 +32,9 @@ GBST_DECL_STREAM(2, f32) GBST_DECL_STREAM(2, bf16) GBST_DECL_STREAM(2, f16)
 GBST_DECL_STREAM(3, f32) GBST_DECL_STREAM(3, bf16) GBST_DECL_STREAM(3, f16)
 #undef GBST_DECL_STREAM
 StreamKernelRef get_stream_states_kernel(int R, int star, int k);
+StreamKernelRef get_stream_pad_kernel_f32(int R, int star, int k);
+StreamKernelRef get_stream_pad_kernel_bf16(int R, int star, int k);
+StreamKernelRef get_stream_pad_kernel_f16(int R, int star, int k);
 StreamKernelRef get_stream_tma_kernel_r1(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r2(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r3(int star, int k);
@@ -115,6 +118,10 @@ struct stencil_plan {
     int grid_ok = 0, grid_on = 0;
     GridConfig grid;
     void* grid_mem = nullptr;
+    // streaming runs of a width that is not a multiple of 4 (zero rule): two grids of padded rows
+    int64_t pad_ld = 0;
+    unsigned pad_set = 0;  // bit k: that kernel's shared-memory attribute is set
+    void* pad[2] = {nullptr, nullptr};
     unsigned smem_set = 0;  // bit 2k+vec: that kernel's shared-memory attribute is set
     int tuned = 0;
     const void* naive = nullptr;
@@ -267,6 +274,17 @@ static bool stream_tensor_map(CUtensorMap* map, const void* src, int64_t ny, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+static StreamKernelRef pad_kernel(const stencil_plan* p, int k) {
+    return p->dtype == STENCIL_F32    ? get_stream_pad_kernel_f32(p->R, p->star, k)
+           : p->dtype == STENCIL_BF16 ? get_stream_pad_kernel_bf16(p->R, p->star, k)
+                                      : get_stream_pad_kernel_f16(p->R, p->star, k);
+}
+
+// Plans whose ragged rows go through padded grids (see run_padded).
+static bool pad_eligible(const stencil_plan* p) {
+    return p->nx % 4 != 0 && p->boundary == STENCIL_BOUNDARY_ZERO && pad_kernel(p, 1).fn;
+}
+
 // Fill the streaming kernel's tile configuration for depth k and CTA size threads.
 static stencil_status_t configure_stream(stencil_plan* p, int k, int threads, int tile_rows) {
     const int kmax = stream_kmax(p->R, p->star);
@@ -277,7 +295,7 @@ static stencil_status_t configure_stream(stencil_plan* p, int k, int threads, in
     k = stream_depth_at_most(p->R, p->star, k);
     if (threads < 32 || threads > kStreamMaxThreads || threads % 32)
         return fail(STENCIL_ERR_INVALID_ARG, "threads must be a multiple of 32 in 32..256");
-    const int vec = p->nx % 4 == 0;
+    const int vec = p->nx % 4 == 0 || pad_eligible(p);
     const int H = (p->R * k + 3) / 4 * 4;
     const int bx_max = 4 * threads - 2 * H;
     if (bx_max < 4) return fail(STENCIL_ERR_UNSUPPORTED, "CTA too narrow for this depth");
@@ -533,6 +551,26 @@ static stencil_status_t configure_lowrank(stencil_plan* p) {
     return STENCIL_OK;
 }
 
+// A streaming launch's parameters except its grids, pitches and alignment.
+static StreamParams stream_params(const stencil_plan* p, int nlev) {
+    StreamParams sp{};
+    sp.ny = p->ny;
+    sp.nx = p->nx;
+    sp.ld = sp.ld_out = p->nx;
+    sp.nlev = nlev;
+    sp.H = p->H;
+    sp.bx = p->bx;
+    sp.by = p->by;
+    sp.strips = p->strips;
+    sp.periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
+    sp.w = p->w;
+    for (int i = 0; i < kMaxTaps; ++i) sp.w2.w2[i] = make_float2(p->w.w[i], p->w.w[i]);
+    sp.status = p->status;
+    sp.wait_ns = (long long)(p->opt.timeout_ms > 0 ? p->opt.timeout_ms : 2000) * 1000000LL;
+    sp.debug_withhold = p->opt.debug_withhold;
+    return sp;
+}
+
 // One launch advancing `nlev` steps from src to dst.  `first` / `last`: this
 // launch starts / ends a run (the pipelined TF32 engine rounds its input on
 // the first launch and keeps intermediate states TF32-rounded until the last).
@@ -622,26 +660,12 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
         CK(cudaLaunchKernel(p->naive, grid, block, args, 0, st));
         return STENCIL_OK;
     }
-    StreamParams sp{};
+    StreamParams sp = stream_params(p, nlev);
     sp.in = src;
     sp.out = dst;
-    sp.ny = p->ny;
-    sp.nx = p->nx;
-    sp.ld = p->nx;
-    sp.nlev = nlev;
-    sp.H = p->H;
-    sp.bx = p->bx;
-    sp.by = p->by;
-    sp.strips = p->strips;
-    sp.periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
     const size_t vec_bytes = 4 * p->elem;
     sp.vec = (p->nx % 4 == 0) && ((uintptr_t)src % vec_bytes == 0) &&
              ((uintptr_t)dst % vec_bytes == 0);
-    sp.w = p->w;
-    for (int i = 0; i < kMaxTaps; ++i) sp.w2.w2[i] = make_float2(p->w.w[i], p->w.w[i]);
-    sp.status = p->status;
-    sp.wait_ns = (long long)(p->opt.timeout_ms > 0 ? p->opt.timeout_ms : 2000) * 1000000LL;
-    sp.debug_withhold = p->opt.debug_withhold;
     dim3 grid((unsigned)(p->strips * p->tiles_y)), block((unsigned)p->threads);
     const void* fn = nullptr;
     int smem = 0;
@@ -659,6 +683,91 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
         CK(cudaLaunchKernel(fn, grid, block, args, (size_t)smem, st));
     }
     return STENCIL_OK;
+}
+
+// ---- padded rows for ragged widths ---------------------------------------------------
+//
+// A width that is not a multiple of 4 leaves the rows of a dense grid unaligned,
+// and the streaming kernel then loads and stores them element by element.
+// Runs of the zero rule go through two plan-owned grids of padded rows instead:
+// one pass copies the input, every launch streams 16-byte chunks, and only
+// the last one stores element by element into the caller's grid.  (Periodic
+// rows cannot be padded: a wrapped chunk would read the padding.)  Measured on
+// GB300, 64 steps, us padded | element-wise: 4001 x 5003 5-point star FP32 540 |
+// 809, BF16 519 | 849; 9-point box 706 | 871, 683 | 1030; 13-point star 1622 |
+// 2242, 1567 | 2241; 5x5 box BF16 2353 | 2512; 7x7 box BF16 3568 | 3724.  The
+// FP32 boxes of radius 2 and 3 are bound by arithmetic either way and keep the
+// dense grids (5x5 1600 x 1701 830 | 777, 7x7 4001 x 5003 3512 | 3233).
+
+constexpr int kPadElems = 16;  // pitch granularity
+
+template <typename TW>
+__global__ void __launch_bounds__(256)
+    pad_rows_kernel(const TW* __restrict__ in, TW* __restrict__ out, int64_t ny, int64_t nx, int64_t ld) {
+    // one thread per 4 columns; the padding is written as zeros
+    const int64_t chunks = ld / 4, n = ny * chunks;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        const int64_t y = i / chunks, x = (i - y * chunks) * 4;
+        const TW* row = in + y * nx;
+        alignas(4 * sizeof(TW)) TW v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = x + e < nx ? row[x + e] : TW(0);
+        if constexpr (sizeof(TW) == 4)
+            *reinterpret_cast<uint4*>(out + y * ld + x) = *reinterpret_cast<uint4*>(v);
+        else
+            *reinterpret_cast<uint2*>(out + y * ld + x) = *reinterpret_cast<uint2*>(v);
+    }
+}
+
+// One launch from a padded grid to the other, or (dense) to the caller's grid.
+static stencil_status_t launch_padded(stencil_plan* p, const void* src, void* dst, int nlev, bool dense,
+                                      cudaStream_t st) {
+    StreamParams sp = stream_params(p, nlev);
+    sp.in = src;
+    sp.out = dst;
+    sp.ld = p->pad_ld;
+    sp.ld_out = dense ? p->nx : p->pad_ld;
+    sp.dense_out = dense;
+    sp.vec = 1;
+    const StreamKernelRef r = pad_kernel(p, nlev);
+    const int smem = stream_smem_bytes(p->R, nlev, (int)p->elem, true, false, p->threads);
+    if (!((p->pad_set >> nlev) & 1)) {
+        CK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                stream_smem_bytes(p->R, nlev, (int)p->elem, true, false, kStreamMaxThreads)));
+        p->pad_set |= 1u << nlev;
+    }
+    void* args[] = {&sp};
+    CK(cudaLaunchKernel(r.fn, dim3((unsigned)(p->strips * p->tiles_y)), dim3((unsigned)p->threads), args,
+                        (size_t)smem, st));
+    return STENCIL_OK;
+}
+
+static stencil_status_t run_padded(stencil_plan* p, const void* in, void* out, const std::vector<int>& depths,
+                                   cudaStream_t st) {
+    const int64_t chunks = p->ny * (p->pad_ld / 4);
+    const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(chunks, 256), 16LL * p->sms);
+    if (p->elem == 4)
+        pad_rows_kernel<uint32_t><<<blocks, 256, 0, st>>>(static_cast<const uint32_t*>(in),
+                                                          static_cast<uint32_t*>(p->pad[0]), p->ny, p->nx, p->pad_ld);
+    else
+        pad_rows_kernel<uint16_t><<<blocks, 256, 0, st>>>(static_cast<const uint16_t*>(in),
+                                                          static_cast<uint16_t*>(p->pad[0]), p->ny, p->nx, p->pad_ld);
+    CK(cudaGetLastError());
+    int cur = 0;
+    for (size_t i = 0; i < depths.size(); ++i) {
+        const bool last = i + 1 == depths.size();
+        stencil_status_t s = launch_padded(p, p->pad[cur], last ? out : p->pad[cur ^ 1], depths[i], last, st);
+        if (s != STENCIL_OK) return s;
+        cur ^= 1;
+    }
+    return STENCIL_OK;
+}
+
+// Whether a run of these launches goes through the padded grids (a single
+// launch would pay the copy for one pass: 9-point box BF16 4001 x 5003, 4 steps
+// 64 us padded, 63 element-wise; 16 steps 150 against 223).
+static bool use_padded(const stencil_plan* p, size_t launches) {
+    return p->kernel == STENCIL_KERNEL_STREAM && p->pad[0] && launches >= 2;
 }
 
 // Depths of the launches for T steps: full blocks of k, then the remainder
@@ -743,7 +852,7 @@ stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const
         sp.out = outs[i + d - 1];
         sp.ny = p->ny;
         sp.nx = p->nx;
-        sp.ld = p->nx;
+        sp.ld = sp.ld_out = p->nx;
         sp.nlev = d;
         sp.H = H;
         sp.bx = bx;
@@ -783,10 +892,13 @@ static stencil_status_t time_launch(stencil_plan* p, const void* in, int reps, c
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    stencil_status_t s = launch_once(p, in, p->ws, p->k, st);  // warm-up
+    auto once = [&] {
+        return p->pad[0] ? launch_padded(p, p->pad[0], p->pad[1], p->k, false, st) : launch_once(p, in, p->ws, p->k, st);
+    };
+    stencil_status_t s = once();  // warm-up
     if (s == STENCIL_OK) {
         cudaEventRecord(e0, st);
-        for (int i = 0; i < reps && s == STENCIL_OK; ++i) s = launch_once(p, in, p->ws, p->k, st);
+        for (int i = 0; i < reps && s == STENCIL_OK; ++i) s = once();
         cudaEventRecord(e1, st);
     }
     cudaError_t e = cudaEventSynchronize(e1);
@@ -1156,6 +1268,21 @@ stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t n
             }
         }
     }
+    // Ragged widths under the zero rule: two grids of padded rows, the first of
+    // which doubles as the workspace.
+    if (!p->ws && p->kernel == STENCIL_KERNEL_STREAM && pad_eligible(p)) {
+        const int64_t ld = ceil_div(nx, kPadElems) * kPadElems;
+        const size_t grid = ((size_t)ny * (size_t)ld * p->elem + 255) / 256 * 256;
+        e = cudaMalloc(&p->ws, 2 * grid);
+        if (e == cudaSuccess) {
+            p->pad_ld = ld;
+            p->pad[0] = p->ws;
+            p->pad[1] = static_cast<char*>(p->ws) + grid;
+        } else {  // no room: element-wise loads and stores on the dense grids
+            cudaGetLastError();
+            p->ws = nullptr;
+        }
+    }
     if (!p->ws) e = cudaMalloc(&p->ws, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1235,6 +1362,7 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* p, stencil_plan_info_t*
     i.smem_bytes = p->smem;
     i.workspace_bytes = (int64_t)((size_t)p->ny * p->nx * p->elem) +
                         (p->grid_mem ? (int64_t)grid_scratch_bytes((int)p->ny, (int)p->nx) : 0);
+    if (p->pad[0]) i.workspace_bytes = 2 * (int64_t)((size_t)p->ny * p->pad_ld * p->elem);
     i.mma_n = p->umma_n;
     i.load = p->kernel == STENCIL_KERNEL_STREAM ? (p->tma ? STENCIL_LOAD_TMA : STENCIL_LOAD_CP_ASYNC) : 0;
     i.rank = p->kernel == STENCIL_KERNEL_LOWRANK ? p->lr_rank : 0;
@@ -1267,7 +1395,8 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* p, stencil_plan_info_t*
 
 int64_t stencil_run_launches(const stencil_plan_t* p, int64_t T) {
     if (!p || T < 0) return -1;
-    return (int64_t)launch_depths(p, T).size();
+    const int64_t n = (int64_t)launch_depths(p, T).size();
+    return n + (n > 0 && use_padded(p, (size_t)n) ? 1 : 0);  // (the pass that pads the rows)
 }
 
 stencil_status_t stencil_run(stencil_plan_t* p, const void* in, void* out, int64_t T,
@@ -1318,6 +1447,7 @@ stencil_status_t stencil_run(stencil_plan_t* p, const void* in, void* out, int64
         }
         return STENCIL_OK;
     }
+    if (use_padded(p, depths.size())) return run_padded(p, in, out, depths, st);
     if (in == out && depths.size() % 2 == 1) {
         // An odd launch count would make launch 1 write the grid it reads.
         // Split one launch in two when possible, else stage the input.

@@ -517,7 +517,7 @@ __host__ __device__ constexpr int stream_rows_after(int R, int K) {
 // products are still added row by row (dy = -R .. R), own columns before
 // neighbour columns, so the result does not depend on the schedule or on K.
 template <int R, bool STAR, int K, typename TS, bool VEC, bool EDGE, bool TMA = false, bool ALL = false,
-          bool SKIPCOL = false, class WS>
+          bool SKIPCOL = false, bool PAD = false, class WS>
 __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws, char* ring,
                                             float* ebuf, int NT, int tid, int x0, int y0,
                                             TmaRing tma = TmaRing{}) {
@@ -527,7 +527,7 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
     constexpr int CB = 4 * (int)sizeof(TS);  // bytes of one 4-column chunk
     const int SLOT = NT * CB;                // bytes of one ring slot (one row of the strip)
     const int ny = (int)p.ny, nx = (int)p.nx;
-    const size_t ld = (size_t)p.ld;
+    const size_t ld = (size_t)p.ld, ldo = PAD ? (size_t)p.ld_out : ld;
     const int c0 = x0 - p.H + 4 * tid;  // this thread's first column
     const int ybeg = y0 - R * K;
     const int ylast = min(y0 + p.by, ny);  // one past the last output row
@@ -542,9 +542,11 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
     // chunk outside the grid never publishes its edge columns, so its
     // neighbours read the zeros of the edge arrays, and its own values, which
     // nothing else reads or stores, need no mask; only rows outside the grid
-    // are masked.
+    // are masked, and with PAD (widths that are not a multiple of 4) the columns
+    // of the one chunk the right edge cuts.
     static_assert(!SKIPCOL || VEC, "SKIPCOL needs whole 16-byte chunks");
     const bool pub = !(EDGE && SKIPCOL && mask) || (c0 >= 0 && c0 < nx);
+    const bool ragged = PAD && EDGE && mask && (nx & 3) != 0 && x0 - p.H + 4 * NT > nx;
     const bool store_chunk = active && c0 >= x0 && c0 + 4 <= x0 + p.bx && c0 < nx;
 
     float2 acc[K][D][2];
@@ -676,6 +678,13 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                     // Output row (arriving row) - R of level l+1 is complete.
                     Pa = acc[l][cdone][0];
                     Pb = acc[l][cdone][1];
+                    if constexpr (EDGE && PAD) {
+                        if (ragged) {  // (column 0 of a cut chunk lies in the grid)
+                            Pb.x = col_in[1] ? Pb.x : 0.f;
+                            Pa.y = col_in[2] ? Pa.y : 0.f;
+                            Pb.y = col_in[3] ? Pb.y : 0.f;
+                        }
+                    }
                     if constexpr (EDGE && (MR || !SKIPCOL || !stream_row_gate(R))) {
                         if (mask) {
                             const int yo = ybeg - (l + 1) * R + s;
@@ -693,15 +702,15 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                     if constexpr (ALL) {
                         const int yo = ybeg - (l + 1) * R + s;
                         if (l < K - 1 && store_chunk && yo >= y0 && yo < ylast)
-                            Storage<TS>::store4(static_cast<TS*>(p.lvl_out[l]) + (size_t)yo * ld + c0,
+                            Storage<TS>::store4(static_cast<TS*>(p.lvl_out[l]) + (size_t)yo * ldo + c0,
                                                 make_float4(Pa.x, Pb.x, Pa.y, Pb.y));
                     }
                 }
                 const int yo = ybeg - R * K + s;
                 if (store_chunk && yo >= y0 && yo < ylast) {
-                    TS* orow = static_cast<TS*>(p.out) + (size_t)yo * ld;
+                    TS* orow = static_cast<TS*>(p.out) + (size_t)yo * ldo;
                     const float4 o = make_float4(Pa.x, Pb.x, Pa.y, Pb.y);
-                    if (VEC) {
+                    if (VEC && !(PAD && p.dense_out)) {
                         Storage<TS>::store4(orow + c0, o);
                     } else {
                         const float ov[4] = {o.x, o.y, o.z, o.w};
@@ -783,6 +792,16 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                     }
                 }
                 // acc[l][cdone] is level l+1's row ybeg + s - l(R+1) - R, complete.
+                if constexpr (EDGE && PAD) {
+                    if (ragged) {
+                        float2& A0 = acc[l][cdone][0];
+                        float2& A1 = acc[l][cdone][1];
+                        constexpr bool r1 = R == 1;
+                        A0.y = col_in[r1 ? 2 : 1] ? A0.y : 0.f;
+                        A1.x = col_in[r1 ? 1 : 2] ? A1.x : 0.f;
+                        A1.y = col_in[3] ? A1.y : 0.f;
+                    }
+                }
                 if constexpr (EDGE && (MR || !SKIPCOL || !stream_row_gate(R))) {
                     if (mask) {
                         const int yo = ybeg + s - l * (R + 1) - R;
@@ -806,7 +825,7 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                     const int yo = ybeg + s - l * (R + 1) - R;
                     if (l < K - 1 && store_chunk && yo >= y0 && yo < ylast) {
                         const float2 A0 = acc[l][cdone][0], A1 = acc[l][cdone][1];
-                        Storage<TS>::store4(static_cast<TS*>(p.lvl_out[l]) + (size_t)yo * ld + c0,
+                        Storage<TS>::store4(static_cast<TS*>(p.lvl_out[l]) + (size_t)yo * ldo + c0,
                                             make_float4(A0.x, A0.y, A1.x, A1.y));
                     }
                 }
@@ -816,8 +835,8 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                         const float2 A0 = acc[l][cdone][0], A1 = acc[l][cdone][1];
                         const float4 o = R == 1 ? make_float4(A0.x, A1.x, A0.y, A1.y)
                                                 : make_float4(A0.x, A0.y, A1.x, A1.y);
-                        TS* orow = static_cast<TS*>(p.out) + (size_t)yo * ld;
-                        if (VEC) {
+                        TS* orow = static_cast<TS*>(p.out) + (size_t)yo * ldo;
+                        if (VEC && !(PAD && p.dense_out)) {
                             Storage<TS>::store4(orow + c0, o);
                         } else {
                             const float ov[4] = {o.x, o.y, o.z, o.w};
@@ -871,7 +890,12 @@ __host__ __device__ constexpr int stream_min_blocks(int R, bool STAR, int K) {
 // ALL: every time level of the launch is stored (level l+1 to p.lvl_out[l],
 // the last to p.out), for callers that need each state (the adjoint's
 // recomputation of a segment); VEC kernels only.
-template <int R, bool STAR, int K, typename TS, bool VEC, bool ALL = false>
+// PAD: rows of a padded pitch whose last chunk the grid's right edge may cut, and
+// a last launch that stores dense rows element by element; VEC kernels only, a
+// variant of its own because the extra code in the aligned kernels cost them
+// 5-15 % (9-point box 8192^2, 200 steps: 5.72 -> 6.11 ms, 13-point star 10.6 ->
+// 12.5 ms).
+template <int R, bool STAR, int K, typename TS, bool VEC, bool ALL = false, bool PAD = false>
 __global__ void __launch_bounds__(kStreamMaxThreads, stream_min_blocks(R, STAR, K))
     sweep_stream_kernel(const __grid_constant__ StreamParams p) {
     constexpr int PF = stream_prefetch(K);
@@ -899,9 +923,9 @@ __global__ void __launch_bounds__(kStreamMaxThreads, stream_min_blocks(R, STAR, 
     // (edge tiles of 16-byte-chunk kernels: the edge arrays were zeroed above,
     // so chunks outside the grid may leave them alone, SKIPCOL)
     if (interior)
-        stream_tile<R, STAR, K, TS, VEC, false, false, ALL>(p, ws, ring, ebuf, NT, tid, x0, y0);
+        stream_tile<R, STAR, K, TS, VEC, false, false, ALL, false, PAD>(p, ws, ring, ebuf, NT, tid, x0, y0);
     else
-        stream_tile<R, STAR, K, TS, VEC, true, false, ALL, VEC>(p, ws, ring, ebuf, NT, tid, x0, y0);
+        stream_tile<R, STAR, K, TS, VEC, true, false, ALL, VEC, PAD>(p, ws, ring, ebuf, NT, tid, x0, y0);
 }
 
 // The same sweep with the input rows brought in by the tensor-memory-access
