@@ -33,9 +33,7 @@ struct StreamParams {
     const void* in;
     void* out;
     long long ny, nx;
-    long long ld;   // row pitch of in, in elements (>= nx; a multiple of 4 when vec)
-    long long ld_out;  // row pitch of out (a multiple of 4 when vec, unless dense_out)
-    int dense_out;     // vec kernels: rows of out are not 16-byte aligned, stored element by element
+    long long ld;   // row pitch of in (and out), in elements (>= nx; a multiple of 4 when vec)
     int nlev;      // time levels (Jacobi steps) this launch advances, 1..KMAX
     int H;         // halo columns loaded on each side of a strip (multiple of 4, >= R*nlev)
     int bx;        // output columns per strip (multiple of 4)
@@ -49,6 +47,9 @@ struct StreamParams {
     void* lvl_out[8];   // all-states kernels: time level l+1 (l < nlev-1) is also stored to lvl_out[l]
     Weights w;
     WeightPairs w2;
+    // Padded-row kernels only (at the end: the weights keep their place in the constant bank).
+    long long ld_out;  // row pitch of out (a multiple of 4, unless dense_out)
+    int dense_out;     // rows of out are not 16-byte aligned: stored element by element
 };
 
 // Parameters of the cluster-resident kernel (see sweep_resident.cu).

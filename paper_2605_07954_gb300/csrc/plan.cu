@@ -53,6 +53,12 @@ int box49_umma_tile_rows(int nt);
 cudaError_t launch_box49_umma(int tf32, int nt, const void* src, void* dst, int ny, int nx, int ld,
                               int round_out, unsigned* status, const float* w, int ctas, cudaStream_t st,
                               int timeout_ms, int withhold);
+const void* get_box49_phase_kernel(int tf32);
+int box49_phase_smem_bytes(int tf32);
+int box49_phase_rows();
+int box49_phase_cols(int tf32);
+cudaError_t launch_box49_phase(int tf32, const void* src, void* dst, int ny, int nx, int round_out, unsigned* status,
+                               const float* w, int ctas, cudaStream_t st, int timeout_ms, int withhold);
 const void* get_resident_kernel(int radius, int star, int dtype);
 int resident_threads();
 int resident_max_cluster();
@@ -111,6 +117,8 @@ struct stencil_plan {
     int umma_n = 0;     // tcgen05 engine in use: N of one MMA (0: warp-MMA engine)
     int umma_ok = 0;    // usable tcgen05 MMA widths, bit n / 16
     int umma_ctas = 0;
+    int phase_ok = 0, phase = 0;  // tcgen05 kernel with four output rows per MMA row: usable, in use
+    int phase_ctas = 0;
     // cluster-resident kernel (sweep_resident.cu): usable cluster sizes (bit log2 C), the one in use
     const void* res_fn = nullptr;
     int res_ok = 0, res_c = 0, res_rp = 0, res_kb = 1, res_smem = 0, res_max_smem = 0;
@@ -395,6 +403,22 @@ static stencil_status_t configure_umma(stencil_plan* p) {
     const int nt = p->opt.mma_n > 0 ? p->opt.mma_n : kUmmaDefaultN[tf32];
     if (want == STENCIL_KERNEL_TC_UMMA || kUmmaPreferred[tf32]) p->umma_n = (p->umma_ok >> (nt / 16)) & 1 ? nt : 0;
     if (want == STENCIL_KERNEL_TC_UMMA && !p->umma_n) return fail(STENCIL_ERR_UNSUPPORTED, "tcgen05 kernel unusable");
+    // The phase kernel (box49_phase.cu) takes rows in groups of four.  It is the
+    // default wherever it applies: us per step, phase | kUmmaDefaultN above, BF16
+    // 512^2 12.5 | 16.5, 2048^2 12.4 | 18.6, 4096^2 21.5 | 31.8, 16384^2 209.5 |
+    // 293.2; TF32 12.3 | 16.0, 14.8 | 18.4, 32.4 | 43.7, 390 | 509.
+    p->phase_ok = p->phase = 0;
+    if (p->opt.mma_n == 0 && p->umma_n && p->ny % 4 == 0) {
+        const void* fn = get_box49_phase_kernel(tf32);
+        const int smem = box49_phase_smem_bytes(tf32);
+        int per_sm = 0;
+        CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, box49_umma_threads(0), smem));
+        const int64_t tiles = ceil_div(p->ny, box49_phase_rows()) * ceil_div(p->nx, box49_phase_cols(tf32));
+        p->phase_ok = per_sm >= 1;
+        p->phase_ctas = (int)std::min<int64_t>(p->sms, tiles);
+        p->phase = p->phase_ok;
+    }
     p->kernel = p->umma_n ? STENCIL_KERNEL_TC_UMMA : STENCIL_KERNEL_TC;
     return STENCIL_OK;
 }
@@ -593,7 +617,10 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
         for (int i = 0; i < 49; ++i) tp.w[i] = p->w.w[i];
         const int tf32 = p->compute == STENCIL_COMPUTE_TC_TF32;
         if (p->umma_n && !(tf32 && first) && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 16 == 0) {
-            const cudaError_t e = launch_box49_umma(tf32, p->umma_n, src, dst, tp.ny, tp.nx, tp.ld,
+            const cudaError_t e =
+                p->phase ? launch_box49_phase(tf32, src, dst, tp.ny, tp.nx, tf32 && !last, p->status, p->w.w,
+                                              p->phase_ctas, st, p->opt.timeout_ms, p->opt.debug_withhold)
+                         : launch_box49_umma(tf32, p->umma_n, src, dst, tp.ny, tp.nx, tp.ld,
                                                     tf32 && !last, p->status, p->w.w, p->umma_ctas, st,
                                                     p->opt.timeout_ms, p->opt.debug_withhold);
             if (e == cudaSuccess) return STENCIL_OK;
@@ -914,7 +941,8 @@ static stencil_status_t time_launch(stencil_plan* p, const void* in, int reps, c
 // width (one step per launch, `in` into the workspace) and keep the fastest.
 // A plan created with kernel = TC_UMMA, or with mma_n set, keeps that choice.
 typedef std::tuple<int64_t, int64_t, int, int, int> TcTuneKey;
-static std::map<TcTuneKey, int> g_tc_tune_cache;
+static std::map<TcTuneKey, int> g_tc_tune_cache;  // MMA width (0: warp MMAs), + kTunePhase for the phase kernel
+static const int kTunePhase = 1024;
 
 static stencil_status_t autotune_tc(stencil_plan* p, const void* in, cudaStream_t st) {
     if (!p->umma_ok || p->opt.kernel == STENCIL_KERNEL_TC_UMMA || p->opt.mma_n > 0) return STENCIL_OK;
@@ -928,10 +956,12 @@ static stencil_status_t autotune_tc(stencil_plan* p, const void* in, cudaStream_
     if (best_n < 0) {
         const int reps = (int)std::max(2.0, std::min(32.0, 4e9 / ((double)p->ny * (double)p->nx)));
         float best = 1e30f;
-        for (int c = 0; c <= 5; ++c) {
-            const int nt = c ? kUmmaWidths[c - 1] : 0;
+        for (int c = 0; c <= 6; ++c) {
+            const int nt = c == 6 ? kUmmaDefaultN[p->compute == STENCIL_COMPUTE_TC_TF32] : c ? kUmmaWidths[c - 1] : 0;
             if (nt && !((p->umma_ok >> (nt / 16)) & 1)) continue;
+            if (c == 6 && !p->phase_ok) continue;
             p->umma_n = nt;
+            p->phase = c == 6;
             cudaEvent_t e0, e1;
             CK(cudaEventCreate(&e0));
             CK(cudaEventCreate(&e1));
@@ -950,12 +980,14 @@ static stencil_status_t autotune_tc(stencil_plan* p, const void* in, cudaStream_
             if (e != cudaSuccess) return fail(STENCIL_ERR_CUDA, std::string("autotune timing: ") + cudaGetErrorString(e));
             if (ms < best) {
                 best = ms;
-                best_n = nt;
+                best_n = nt + (c == 6 ? kTunePhase : 0);
             }
         }
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_tc_tune_cache[key] = best_n;
     }
+    p->phase = best_n >= kTunePhase;
+    best_n %= kTunePhase;
     p->umma_n = best_n;
     p->kernel = best_n ? STENCIL_KERNEL_TC_UMMA : STENCIL_KERNEL_TC;
     return STENCIL_OK;
@@ -1388,6 +1420,14 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* p, stencil_plan_info_t*
         i.ctas = p->umma_ctas;
         i.smem_bytes = box49_umma_smem_bytes(p->compute == STENCIL_COMPUTE_TC_TF32, p->umma_n);
         i.tile_rows = box49_umma_tile_rows(p->umma_n);
+    }
+    if (p->umma_n && p->phase) {
+        const int tf32 = p->compute == STENCIL_COMPUTE_TC_TF32;
+        i.mma_n = 128;  // the widest MMA: four column blocks of 32
+        i.ctas = p->phase_ctas;
+        i.smem_bytes = box49_phase_smem_bytes(tf32);
+        i.tile_rows = box49_phase_rows();
+        i.tile_cols = box49_phase_cols(tf32);
     }
     *info = i;
     return STENCIL_OK;
