@@ -311,9 +311,10 @@ typedef struct {
 } stencil_grid_desc_t;
 
 typedef struct {
-    int tb_depth;           /* steps per work item k; 0 = 4, capped per radius (8 / 2 / 2) */
-    int threads;            /* CTA size, multiple of 32 in 32..256; 0 = 128            */
-    int tile_rows;          /* rows per tile; 0 = 256 (at least R*k + 2R + 2)          */
+    int tb_depth;           /* steps per work item k; 0 = choose, capped per radius (8 / 2 / 2) */
+    int threads;            /* CTA size, multiple of 32 in 32..256; 0 = one-warp tiles for
+                               radius 1 (threads = 32 in stencil_batch_info), else 128  */
+    int tile_rows;          /* rows per tile; 0 = choose (at least R*k + 2R + 2)       */
     int autotune;           /* 1: time each depth and CTA size on the whole batch at create */
     int timeout_ms;         /* bound of every device-side wait; 0 = 2000 ms             */
     int debug_withhold_item;/* test hook: 1 + index of a work item whose completion is never

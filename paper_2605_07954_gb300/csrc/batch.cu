@@ -38,6 +38,7 @@
 #include "common.cuh"
 #include "stream_depths.h"
 #include "sweep_stream.cuh"
+#include "sweep_warp.cuh"
 
 namespace gbst {
 
@@ -54,7 +55,8 @@ struct BatchParams {
     const BatchGrid* grids;
     const int4* items;  // (grid, tile, global block index, unused)
     int item_begin, item_end;
-    int* ticket;        // next item to pop (this launch's counter)
+    int* ticket;        // next item to pop (this launch's counter; two for one-warp tiles)
+    int split, star_sms;  // one-warp tiles: items [item_begin, split) are boxes, the rest stars; SMs that take stars first
     int* epochs;        // per tile: blocks completed
     unsigned* status;   // STENCIL_ERR_TIMEOUT when a wait ran out
     int* abort_flag;
@@ -179,6 +181,130 @@ __global__ void __launch_bounds__(kStreamMaxThreads)
     }
 }
 
+// Radius 1: every warp of the launch pops its own items and runs each as a
+// one-warp tile (sweep_warp.cuh), with the same epochs and bounded waits.  The
+// launch has two queues, 9-point boxes and 5-point stars, and an SM serves one
+// of them until it is empty: the two unrolled row loops together do not fit the
+// instruction cache (256 grids x 200 steps: one queue 20.5 ms, one launch per
+// shape 16.6, two queues 15.3).
+constexpr int kBatchWarpCols = 4;  // columns per lane
+
+// Warps per SM the registers must allow (256-grid batch: K = 8 at 16 warps 15.3
+// ms, at 12 without spills 15.6; K = 4 at 16 15.5, at 20 16.0).
+__host__ __device__ constexpr int batch_warp_min_blocks(int K) { return K >= 4 ? 16 : 28; }
+
+template <int K, typename TS>
+__global__ void __launch_bounds__(32, batch_warp_min_blocks(K))
+    batch_warp_kernel(const __grid_constant__ BatchParams bp) {
+    constexpr int NC = kBatchWarpCols;
+    __shared__ __align__(16) char ring[warp_ring_bytes<TS, NC>()];
+    const int lane = threadIdx.x;
+    unsigned smid;
+    asm("mov.u32 %0, %%smid;" : "=r"(smid));
+    int queue = (int)smid < bp.star_sms ? 1 : 0, empty = 0;
+    for (;;) {
+        int it = -1;
+        if (lane == 0 && !*(volatile int*)bp.abort_flag) {
+            while (it < 0 && empty < 2) {
+                const int begin = queue ? bp.split : bp.item_begin, end = queue ? bp.item_end : bp.split;
+                const int t = begin < end ? atomicAdd(bp.ticket + queue, 1) + begin : end;
+                if (t < end) {
+                    it = t;
+                } else {  // this queue is empty: serve the other one
+                    queue ^= 1;
+                    ++empty;
+                }
+            }
+        }
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it < 0) break;
+        const int4 item = bp.items[it];
+        const BatchGrid& g = bp.grids[item.x];
+        const int tx = item.y % g.strips, ty = item.y / g.strips;
+        if (bp.deps && lane < 25) {
+            // one neighbour a lane: 3 x 3, or 5 x 5 with wrapping for periodic grids (the
+            // last strip or tile row may be narrower than the halo)
+            int ux = tx + lane % 5 - 2, uy = ty + lane / 5 - 2;
+            bool need = true;
+            if (g.periodic) {
+                ux = (ux % g.strips + g.strips) % g.strips;
+                uy = (uy % g.tiles_y + g.tiles_y) % g.tiles_y;
+            } else {
+                need = abs(ux - tx) <= 1 && abs(uy - ty) <= 1 && ux >= 0 && ux < g.strips && uy >= 0 && uy < g.tiles_y;
+            }
+            const int* e = bp.epochs + g.tile_base + (need ? uy * g.strips + ux : item.y);
+            long long t0 = 0;
+            for (unsigned spins = 0; need && ld_acquire(e) < item.z; ++spins) {
+                if (*(volatile int*)bp.abort_flag) {
+                    it = -1;
+                    break;
+                }
+                if ((spins & 15u) == 15u) {
+                    const long long now = global_ns();
+                    if (t0 == 0) t0 = now;
+                    if (now - t0 > bp.timeout_ns || spins > (1u << 26)) {
+                        atomicCAS(bp.status, 0u, (unsigned)STENCIL_ERR_TIMEOUT);
+                        atomicExch(bp.abort_flag, 1);
+                        it = -1;
+                        break;
+                    }
+                }
+                __nanosleep(64);
+            }
+        }
+        if (__any_sync(0xffffffffu, it < 0)) break;
+        StreamParams p;
+        p.in = g.buf[item.z & 1];
+        p.out = g.buf[(item.z + 1) & 1];
+        p.ny = g.ny;
+        p.nx = g.nx;
+        p.ld = g.ld;
+        p.H = g.H;
+        p.bx = g.bx;
+        p.by = g.by;
+        p.periodic = g.periodic;
+        const int x0 = tx * g.bx, y0 = ty * g.by;
+        const int ylast = min(y0 + g.by, g.ny);
+        const bool interior = y0 - K >= 0 && ylast + warp_rows_after(K) <= g.ny && x0 - g.H >= 0 &&
+                              x0 - g.H + 32 * NC <= g.nx;
+        auto weight = [&](int i) { return g.w2[i].x; };
+        if (g.star) {
+            const WarpWeights<true> ws(weight);
+            if (interior) warp_tile<true, K, TS, NC, false>(p, ws, ring, lane, x0, y0);
+            else warp_tile<true, K, TS, NC, true>(p, ws, ring, lane, x0, y0);
+        } else {
+            const WarpWeights<false> ws(weight);
+            if (interior) warp_tile<false, K, TS, NC, false>(p, ws, ring, lane, x0, y0);
+            else warp_tile<false, K, TS, NC, true>(p, ws, ring, lane, x0, y0);
+        }
+        __syncwarp();  // every lane's stores of this tile are issued
+        if (lane == 0 && it != bp.withhold) {
+            __threadfence();
+            red_release_add(bp.epochs + g.tile_base + item.y, 1);
+        }
+    }
+}
+
+template <int K>
+static const void* batch_warp_dtype(int dtype) {
+    switch (dtype) {
+        case DT_F32: return (const void*)batch_warp_kernel<K, float>;
+        case DT_BF16: return (const void*)batch_warp_kernel<K, __nv_bfloat16>;
+        case DT_F16: return (const void*)batch_warp_kernel<K, __half>;
+        default: return nullptr;
+    }
+}
+
+static const void* batch_warp(int K, int dtype) {
+    switch (K) {
+        case 1: return batch_warp_dtype<1>(dtype);
+        case 2: return batch_warp_dtype<2>(dtype);
+        case 4: return batch_warp_dtype<4>(dtype);
+        case 8: return batch_warp_dtype<8>(dtype);
+        default: return nullptr;
+    }
+}
+
 struct BatchKernelRef {
     const void* fn;
 };
@@ -257,6 +383,9 @@ struct Launch {
     int deps;        // 1: persistent launch with neighbour waits
     int ctas;
     int smem;
+    int threads;
+    int split;       // one-warp tiles: boxes [begin, split), stars [split, end)
+    int star_sms;
     const void* fn;
 };
 
@@ -286,7 +415,7 @@ struct stencil_batch {
     int n_tiles = 0;
     BatchGrid* dgrids = nullptr;
     int4* items = nullptr;
-    int* counters = nullptr;   // [0, nl): per-launch tickets; [nl]: abort flag; then epochs
+    int* counters = nullptr;   // [0, 2 nl): two tickets per launch; [2 nl]: abort flag; then epochs
     int n_counter_ints = 0;
     unsigned* status = nullptr;
     cudaStream_t cap = nullptr;
@@ -308,9 +437,50 @@ void free_device_plan(stencil_batch* b) {
     b->exec = nullptr;
 }
 
+// Depth and height of the one-warp tiles of a batch's radius-1 grids: the cheapest
+// per step by a cost model.  A tile of `by` rows walks by + 2k rows of k levels,
+// ~33 warp instructions each; an SM quarter issues ~0.66 of them per cycle when
+// it holds several warps, one warp alone ~0.45; popping an item, its waits and
+// the pipeline's fill cost ~4000 cycles.  256 grids of sides 64..2048: k = 8 and
+// 256 rows (15.3 ms; 128 rows 15.8, k = 4 15.5); few or small grids get lower
+// tiles, so that their warps fill the SMs.
+void choose_warp_tiles(const stencil_batch* b, int& k, int* rows) {
+    static const int ks[2] = {8, 4}, heights[7] = {256, 192, 128, 96, 64, 48, 32};
+    const int fixed = k;
+    double best = 1e300;
+    for (int kc : ks) {
+        const int kk = fixed > 0 ? batch_depth_at_most(1, fixed) : kc;
+        for (int by : heights) {
+            if (by < kk + 4) continue;
+            double tiles = 0;
+            for (auto& hg : b->grids)
+                if (hg.R == 1 && hg.d.T > 0)
+                    tiles += (double)cdiv(hg.d.nx, 32 * kBatchWarpCols - 2 * ((kk + 3) / 4 * 4)) *
+                             (double)cdiv(hg.d.ny, std::min<long long>(by, hg.d.ny));
+            const double quarter = tiles / (4.0 * b->sms);  // tiles per SM quarter and time block
+            const double walk = (by + 2.0 * kk) * kk * 33.0;
+            const double cost = (std::max(walk / 0.45, quarter * walk / 0.66) + 4000.0 * std::max(1.0, quarter / 4)) / kk;
+            if (cost < best) {
+                best = cost;
+                k = fixed > 0 ? fixed : kk;
+                *rows = by;
+            }
+        }
+        if (fixed > 0) break;
+    }
+}
+
 // Tile every grid for depth k with CTAs of `threads`, and build the block-major
 // item list and the launches.  Host-side only, then uploads.
+// `threads` 0: radius-1 grids as one-warp tiles (and CTAs of 128 for the others);
+// `k` 0: the depth (and, with tile_rows 0, the height of one-warp tiles) by
+// choose_warp_tiles.
 stencil_status_t build_schedule(stencil_batch* b, int k, int threads, int tile_rows) {
+    const bool warp = threads == 0;
+    int warp_rows = 256;
+    if (warp) choose_warp_tiles(b, k, &warp_rows);
+    if (k == 0) k = 4;
+    if (warp) threads = 128;
     free_device_plan(b);
     b->k = k;
     b->threads = threads;
@@ -329,13 +499,15 @@ stencil_status_t build_schedule(stencil_batch* b, int k, int threads, int tile_r
         g.nx = (int)hg.d.nx;
         g.ld = hg.ld;
         g.H = (R * kg + 3) / 4 * 4;
-        const int bx_max = 4 * threads - 2 * g.H;
+        const bool wg = warp && R == 1;
+        const int bx_max = (wg ? 32 * kBatchWarpCols : 4 * threads) - 2 * g.H;
         if (bx_max < 4) return bfail(STENCIL_ERR_UNSUPPORTED, "CTA too narrow for this depth");
         g.strips = (int)cdiv(g.nx, bx_max);
         g.bx = (int)(cdiv(cdiv(g.nx, g.strips), 4) * 4);
+        g.strips = (int)cdiv(g.nx, g.bx);
         // Tiles at least R*k + 2R + 1 rows high keep every dependency in the
         // 3x3 neighbourhood.
-        const int want = tile_rows > 0 ? tile_rows : 256;
+        const int want = tile_rows > 0 ? tile_rows : wg ? warp_rows : 256;
         const int min_rows = R * kg + 2 * R + 2;
         int ty = (int)std::max(1LL, cdiv(g.ny, std::max(want, min_rows)));
         while (ty > 1 && cdiv(g.ny, ty) < min_rows) --ty;
@@ -354,6 +526,7 @@ stencil_status_t build_schedule(stencil_batch* b, int k, int threads, int tile_r
     // Launch groups: per radius, the main depth-k blocks (persistent), then
     // remainder depths (greedy), each a persistent launch of its own.
     for (int R = 1; R <= 3; ++R) {
+        const bool wg = warp && R == 1;
         std::vector<int> members;
         for (int gi = 0; gi < b->n; ++gi)
             if (b->grids[gi].R == R && b->grids[gi].d.T > 0) members.push_back(gi);
@@ -374,17 +547,29 @@ stencil_status_t build_schedule(stencil_batch* b, int k, int threads, int tile_r
             L.begin = (int)b->items_h.size();
             long long nb = 0;
             for (auto& pb : plan_blocks) nb = std::max(nb, pb.second);
-            for (long long blk = 0; blk < nb; ++blk)
-                for (auto& pb : plan_blocks) {
-                    if (blk >= pb.second) continue;
-                    HostGrid& hg = b->grids[pb.first];
-                    const BatchGrid& g = b->dgrids_h[pb.first];
-                    for (int t = 0; t < g.strips * g.tiles_y; ++t)
-                        b->items_h.push_back(make_int4(pb.first, t, (int)(hg.blocks + blk), 0));
-                }
+            // one-warp tiles: the boxes' queue, then the stars'; else one queue (queue = -1)
+            double cost[2] = {0, 0};
+            for (int queue = wg ? 0 : -1; queue < (wg ? 2 : 0); ++queue) {
+                if (queue == 1) L.split = (int)b->items_h.size();
+                for (long long blk = 0; blk < nb; ++blk)
+                    for (auto& pb : plan_blocks) {
+                        if (blk >= pb.second || (queue >= 0 && b->grids[pb.first].star != queue)) continue;
+                        HostGrid& hg = b->grids[pb.first];
+                        if (queue >= 0) cost[queue] += (queue ? 5.0 : 9.0) * (double)hg.d.ny * (double)hg.d.nx;
+                        const BatchGrid& g = b->dgrids_h[pb.first];
+                        for (int t = 0; t < g.strips * g.tiles_y; ++t)
+                            b->items_h.push_back(make_int4(pb.first, t, (int)(hg.blocks + blk), 0));
+                    }
+            }
             for (auto& pb : plan_blocks) b->grids[pb.first].blocks += (int)pb.second;
             L.end = (int)b->items_h.size();
             L.deps = 1;
+            L.threads = threads;
+            if (wg) {
+                L.threads = 32;
+                L.fn = batch_warp(depth, b->dtype);
+                L.star_sms = (int)std::lround(b->sms * cost[1] / std::max(1.0, cost[0] + cost[1]));
+            }
             b->launches.push_back(L);
         };
         std::vector<std::pair<int, long long>> main_blocks;
@@ -406,6 +591,13 @@ stencil_status_t build_schedule(stencil_batch* b, int k, int threads, int tile_r
         }
     }
     for (auto& L : b->launches) {
+        if (L.fn) {  // one-warp tiles: static shared memory only
+            int per_sm = 0;
+            BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, L.fn, 32, 0));
+            if (per_sm < 1) return bfail(STENCIL_ERR_UNSUPPORTED, "batched kernel does not fit on an SM");
+            L.ctas = (int)std::min<long long>((long long)per_sm * b->sms, L.end - L.begin);
+            continue;
+        }
         L.fn = batch_kernel(L.R, L.depth, b->dtype);
         if (!L.fn) return bfail(STENCIL_ERR_UNSUPPORTED, "no batched kernel for this depth");
         L.smem = stream_smem_bytes(L.R, L.depth, (int)b->elem, true, false, kStreamMaxThreads);
@@ -423,7 +615,7 @@ stencil_status_t build_schedule(stencil_batch* b, int k, int threads, int tile_r
     if (!b->items_h.empty())
         BCK(cudaMemcpy(b->items, b->items_h.data(), sizeof(int4) * b->items_h.size(),
                        cudaMemcpyHostToDevice));
-    b->n_counter_ints = (int)b->launches.size() + 1 + tiles;
+    b->n_counter_ints = 2 * (int)b->launches.size() + 1 + tiles;
     BCK(cudaMalloc(&b->counters, sizeof(int) * std::max(1, b->n_counter_ints)));
     return STENCIL_OK;
 }
@@ -448,15 +640,17 @@ stencil_status_t enqueue(stencil_batch* b, cudaStream_t st) {
         bp.items = b->items;
         bp.item_begin = L.begin;
         bp.item_end = L.end;
-        bp.ticket = b->counters + li;
-        bp.abort_flag = b->counters + nl;
-        bp.epochs = b->counters + nl + 1;
+        bp.ticket = b->counters + 2 * li;
+        bp.split = L.split;
+        bp.star_sms = L.star_sms;
+        bp.abort_flag = b->counters + 2 * nl;
+        bp.epochs = b->counters + 2 * nl + 1;
         bp.status = b->status;
         bp.timeout_ns = b->timeout_ns;
         bp.deps = L.deps;
         bp.withhold = b->opt.debug_withhold_item > 0 && li == 0 ? b->opt.debug_withhold_item - 1 : -1;
         void* args[] = {&bp};
-        BCK(cudaLaunchKernel(L.fn, dim3((unsigned)L.ctas), dim3((unsigned)b->threads), args,
+        BCK(cudaLaunchKernel(L.fn, dim3((unsigned)L.ctas), dim3((unsigned)L.threads), args,
                              (size_t)L.smem, st));
     }
     for (auto& hg : b->grids) {
@@ -574,14 +768,13 @@ stencil_status_t stencil_batch_create(stencil_batch_t** out, int n, const stenci
     if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
         return bail(bfail(STENCIL_ERR_CUDA, "cudaStreamCreate failed"));
 
-    const int threads = o.threads ? o.threads : 128;
     if (o.autotune) {
         // Time every instantiated radius-1 depth (and CTA size unless fixed) on the
         // whole batch; keep the fastest.
         const int ks[4] = {1, 2, 4, 8};
-        const int ths[3] = {64, 128, 256};
+        const int ths[4] = {0, 64, 128, 256};  // 0: one-warp tiles
         float best = 1e30f;
-        int bk = 8, bt = threads;
+        int bk = 8, bt = o.threads;
         for (int k : ks) {
             if (o.tb_depth && k != o.tb_depth) continue;
             for (int th : ths) {
@@ -600,9 +793,9 @@ stencil_status_t stencil_batch_create(stencil_batch_t** out, int n, const stenci
         stencil_status_t s = build_schedule(b, bk, bt, o.tile_rows);
         if (s != STENCIL_OK) return bail(s);
     } else {
-        // Default depth 4: the measured best for the 256-grid radius-1 batch on GB300
-        // (deeper items cost more halo rows per tile at these tile heights).
-        stencil_status_t s = build_schedule(b, o.tb_depth ? o.tb_depth : 4, threads, o.tile_rows);
+        // Default depth 4 for CTAs of `threads`: the measured best for the 256-grid radius-1
+        // batch on GB300 (deeper items cost more halo rows per tile at these tile heights).
+        stencil_status_t s = build_schedule(b, o.tb_depth, o.threads, o.tile_rows);
         if (s != STENCIL_OK) return bail(s);
     }
     *out = b;
@@ -646,7 +839,7 @@ stencil_status_t stencil_batch_info(const stencil_batch_t* b, stencil_batch_info
     stencil_batch_info_t i{};
     i.n = b->n;
     i.tb_depth = b->k;
-    i.threads = b->threads;
+    i.threads = b->launches.empty() ? b->threads : b->launches[0].threads;
     i.tiles = b->n_tiles;
     i.items = (int64_t)b->items_h.size();
     i.launches = (int)b->launches.size();

@@ -146,3 +146,36 @@ def test_batched_256_grids_workload(oracle):
         want = oracle.sweep_f64(g["x"].cpu().numpy(), g["weights"], 200)
         assert rel_l2(g["out"].cpu().numpy(), want) <= fp32_tol(200)
     b.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_one_warp_tiles_edges_and_queues(dtype):
+    """Radius-1 grids run as one-warp tiles from two queues (boxes, stars): widths
+    around a tile's 112 and 120 columns, chunks cut by the right edge, periodic
+    grids of several tiles, heights around the tile heights; with one queue empty
+    too.  Against single runs: FP32 bit for bit, BF16 within its rounding (the
+    two round after different numbers of steps)."""
+    from paper_2605_07954_gb300 import Batch
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    shapes = [(300, 111), (97, 121), (33, 240), (129, 226), (64, 1025), (700, 5), (512, 480), (31, 112)]
+    for kinds in (("heat5r", "box9"), ("heat5r",), ("box9",)):
+        for depth in (0, 8, 1):
+            grids = []
+            for i, (ny, nx) in enumerate(shapes):
+                x = torch.from_numpy(inputs.field(ny, nx, stream=700 + i)).cuda().to(td)
+                grids.append(dict(x=x, out=torch.empty_like(x), T=17 + i, boundary="periodic" if nx % 16 == 0 else "zero",
+                                  weights=inputs.batch_grid_weights(kinds[i % len(kinds)], i)))
+            b = Batch(grids, dtype=dtype, tb_depth=depth, tile_rows=0 if depth != 8 else 40)
+            assert b.info()["threads"] == 32
+            for _ in range(2):
+                b.run()
+            torch.cuda.synchronize()
+            b.status()
+            for i, g in enumerate(grids):
+                if dtype == "f32":
+                    assert torch.equal(g["out"], _single(g["x"], g["weights"], g["T"], g["boundary"])), (kinds, depth, i)
+                else:
+                    ref = _single(g["x"].float(), g["weights"], g["T"], g["boundary"]).double()
+                    err = float((g["out"].double() - ref).norm() / ref.norm())
+                    assert err <= 2.0 ** -8, (kinds, depth, i, err)
+            b.close()
