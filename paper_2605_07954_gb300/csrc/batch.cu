@@ -8,7 +8,7 @@
 // from a device queue in block-major order:
 //
 //   item (grid g, tile i, block b) may start once every tile in the 3x3
-//   neighbourhood of i has completed block b-1.
+//   neighbourhood of i (5x5 and wrapped for periodic grids) has completed block b-1.
 //
 // That covers the reads of block b (the neighbours' block b-1 outputs, within
 // the K*R halo) and the overwrite of block b's destination (the same
@@ -109,9 +109,16 @@ __global__ void __launch_bounds__(kStreamMaxThreads)
                 const int tx = item.y % g.strips, ty = item.y / g.strips;
                 const long long t0 = global_ns();
                 unsigned spins = 0;  // second bound, in case the timer were to stall
-                for (int dy = -1; dy <= 1 && it >= 0; ++dy) {
-                    for (int dx = -1; dx <= 1 && it >= 0; ++dx) {
-                        const int ux = tx + dx, uy = ty + dy;
+                // periodic grids wrap, and reach two tiles far: the last strip or tile
+                // row may be narrower than the halo
+                const int reach = g.periodic ? 2 : 1;
+                for (int dy = -reach; dy <= reach && it >= 0; ++dy) {
+                    for (int dx = -reach; dx <= reach && it >= 0; ++dx) {
+                        int ux = tx + dx, uy = ty + dy;
+                        if (g.periodic) {
+                            ux = (ux % g.strips + g.strips) % g.strips;
+                            uy = (uy % g.tiles_y + g.tiles_y) % g.tiles_y;
+                        }
                         if (ux < 0 || ux >= g.strips || uy < 0 || uy >= g.tiles_y) continue;
                         const int* e = bp.epochs + g.tile_base + uy * g.strips + ux;
                         while (ld_acquire(e) < item.z) {

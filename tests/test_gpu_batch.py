@@ -179,3 +179,23 @@ def test_one_warp_tiles_edges_and_queues(dtype):
                     err = float((g["out"].double() - ref).norm() / ref.norm())
                     assert err <= 2.0 ** -8, (kinds, depth, i, err)
             b.close()
+
+
+@pytest.mark.parametrize("name", ["box9", "star13", "box49"])
+def test_periodic_grids_of_many_tiles(name):
+    """Periodic grids wrap, so a tile at one edge also waits for the tiles at the
+    opposite one: many small tiles, several runs, CTA-wide tiles (threads set)."""
+    from paper_2605_07954_gb300 import Batch
+    W = inputs.pattern_weights(name)
+    grids = []
+    for i, (ny, nx) in enumerate([(400, 1036), (1001, 260), (260, 2100)]):
+        x = torch.from_numpy(inputs.field(ny, nx, stream=900 + i)).cuda()
+        grids.append(dict(x=x, out=torch.empty_like(x), weights=W, T=24, boundary="periodic"))
+    b = Batch(grids, threads=64, tile_rows=24)
+    for _ in range(3):
+        b.run()
+        torch.cuda.synchronize()
+        b.status()
+        for i, g in enumerate(grids):
+            assert torch.equal(g["out"], _single(g["x"], W, 24, "periodic")), i
+    b.close()
