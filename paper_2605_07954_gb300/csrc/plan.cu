@@ -35,6 +35,7 @@ StreamKernelRef get_stream_states_kernel(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_f32(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_bf16(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_f16(int R, int star, int k);
+const void* get_warp_kernel(int star, int dtype, int nc);
 StreamKernelRef get_stream_tma_kernel_r1(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r2(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r3(int star, int k);
@@ -119,6 +120,9 @@ struct stencil_plan {
     int umma_ctas = 0;
     int phase_ok = 0, phase = 0;  // tcgen05 kernel with four output rows per MMA row: usable, in use
     int phase_ctas = 0;
+    // one-warp streaming kernel (sweep_warp.cuh) for launches of kWarpDepth steps: columns per
+    // lane (0: not in use) and its tiles
+    int warp_nc = 0, warp_bx = 0, warp_by = 0, warp_strips = 0, warp_tiles = 0;
     // cluster-resident kernel (sweep_resident.cu): usable cluster sizes (bit log2 C), the one in use
     const void* res_fn = nullptr;
     int res_ok = 0, res_c = 0, res_rp = 0, res_kb = 1, res_smem = 0, res_max_smem = 0;
@@ -288,6 +292,42 @@ static StreamKernelRef pad_kernel(const stencil_plan* p, int k) {
                                       : get_stream_pad_kernel_f16(p->R, p->star, k);
 }
 
+// One-warp tiles for the depth-8 launches of radius-1 plans that leave the
+// streaming kernel's options alone.  Each SM holds 16 warps (8 at NC = 8) and the
+// tiles are cut to one wave of them; a tile needs enough rows to pay for its 16
+// halo rows.  Measured on GB300, 64 steps FP32 in us, one-warp tiles | CTA-wide:
+// 5-point star 16384^2 (NC = 8) 3776 | 4764, 8192^2 1019 | 1252 (NC = 4: 1187),
+// 4096^2 (64-row tiles, NC = 4; NC = 8: 389) 397 | 473, 3500^2 (47 rows) 317 |
+// 338, 3000^2 (34 rows) 312 | 281; 9-point box 16384^2 6712 | 6901, 8192^2 1796 |
+// 1827, 4096^2 561 | 576, 3500^2 439 | 445, 3000^2 476 | 363.
+static bool pad_eligible(const stencil_plan* p);
+constexpr int kWarpDepth = 8;
+constexpr int kWarpMinRows = 44;      // NC = 4
+constexpr int kWarpMinRowsWide = 128;  // NC = 8: fewer warps, so taller tiles before it pays
+
+static void configure_warp(stencil_plan* p, int threads_asked) {
+    p->warp_nc = 0;
+    const stencil_options_t& o = p->opt;
+    const bool vec = p->nx % 4 == 0 || pad_eligible(p);
+    if (p->R != 1 || p->k != kWarpDepth || p->tma || !vec || o.tb_depth > 0 || o.threads > 0 || o.tile_rows > 0 ||
+        o.load != STENCIL_LOAD_AUTO || threads_asked != default_threads(p->R, p->star))
+        return;
+    for (int nc = p->star ? 8 : 4; nc >= 4; nc -= 4) {
+        const int64_t bx_max = 32 * nc - 2 * kWarpDepth;
+        const int64_t bx = ceil_div(ceil_div(p->nx, ceil_div(p->nx, bx_max)), nc) * nc;
+        const int64_t strips = ceil_div(p->nx, bx);
+        const int64_t warps = (int64_t)p->sms * (nc == 8 ? 8 : 16);
+        const int64_t by = ceil_div(p->ny, std::max<int64_t>(1, warps / strips));
+        if (by < (nc == 8 ? kWarpMinRowsWide : kWarpMinRows)) continue;
+        p->warp_nc = nc;
+        p->warp_bx = (int)bx;
+        p->warp_by = (int)by;
+        p->warp_strips = (int)strips;
+        p->warp_tiles = (int)ceil_div(p->ny, by);
+        return;
+    }
+}
+
 // Plans whose ragged rows go through padded grids (see run_padded).
 static bool pad_eligible(const stencil_plan* p) {
     return p->nx % 4 != 0 && p->boundary == STENCIL_BOUNDARY_ZERO && pad_kernel(p, 1).fn;
@@ -342,6 +382,7 @@ static stencil_status_t configure_stream(stencil_plan* p, int k, int threads, in
     p->tiles_y = (int)tiles_y;
     p->smem = smem;
     p->per_sm = per_sm;
+    configure_warp(p, threads);
     return STENCIL_OK;
 }
 
@@ -595,6 +636,18 @@ static StreamParams stream_params(const stencil_plan* p, int nlev) {
     return sp;
 }
 
+// The launch as one-warp tiles (sp: grids and pitches set).
+static stencil_status_t launch_warp(stencil_plan* p, StreamParams& sp, cudaStream_t st) {
+    sp.H = kWarpDepth;
+    sp.bx = p->warp_bx;
+    sp.by = p->warp_by;
+    sp.strips = p->warp_strips;
+    void* args[] = {&sp};
+    CK(cudaLaunchKernel(get_warp_kernel(p->star, p->dtype, p->warp_nc), dim3((unsigned)(p->warp_strips * p->warp_tiles)),
+                        dim3(32), args, 0, st));
+    return STENCIL_OK;
+}
+
 // One launch advancing `nlev` steps from src to dst.  `first` / `last`: this
 // launch starts / ends a run (the pipelined TF32 engine rounds its input on
 // the first launch and keeps intermediate states TF32-rounded until the last).
@@ -693,6 +746,7 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
     const size_t vec_bytes = 4 * p->elem;
     sp.vec = (p->nx % 4 == 0) && ((uintptr_t)src % vec_bytes == 0) &&
              ((uintptr_t)dst % vec_bytes == 0);
+    if (p->warp_nc && nlev == kWarpDepth && sp.vec) return launch_warp(p, sp, st);
     dim3 grid((unsigned)(p->strips * p->tiles_y)), block((unsigned)p->threads);
     const void* fn = nullptr;
     int smem = 0;
@@ -756,6 +810,7 @@ static stencil_status_t launch_padded(stencil_plan* p, const void* src, void* ds
     sp.ld_out = dense ? p->nx : p->pad_ld;
     sp.dense_out = dense;
     sp.vec = 1;
+    if (p->warp_nc && nlev == kWarpDepth && !dense) return launch_warp(p, sp, st);
     const StreamKernelRef r = pad_kernel(p, nlev);
     const int smem = stream_smem_bytes(p->R, nlev, (int)p->elem, true, false, p->threads);
     if (!((p->pad_set >> nlev) & 1)) {
@@ -1398,6 +1453,14 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* p, stencil_plan_info_t*
     i.mma_n = p->umma_n;
     i.load = p->kernel == STENCIL_KERNEL_STREAM ? (p->tma ? STENCIL_LOAD_TMA : STENCIL_LOAD_CP_ASYNC) : 0;
     i.rank = p->kernel == STENCIL_KERNEL_LOWRANK ? p->lr_rank : 0;
+    if (p->kernel == STENCIL_KERNEL_STREAM && p->warp_nc) {
+        i.threads = 32;
+        i.halo_cols = kWarpDepth;
+        i.tile_cols = p->warp_bx;
+        i.tile_rows = p->warp_by;
+        i.ctas = p->warp_strips * p->warp_tiles;
+        i.smem_bytes = 0;
+    }
     if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on) {
         i.tb_depth = 0;  // every step of a run in one launch
         i.threads = 32 * p->grid.warps;

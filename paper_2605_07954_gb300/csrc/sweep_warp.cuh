@@ -102,8 +102,8 @@ __host__ __device__ constexpr int warp_ring_bytes() { return kWarpRing * 32 * NC
 __host__ __device__ constexpr int warp_rows_after(int K) { return K + 3; }
 
 // One tile: outputs [y0, y0 + by) x [x0, x0 + bx).  EDGE: the tile loads rows or
-// columns outside the grid.  p.bx and p.H are multiples of NC.
-template <bool STAR, int K, typename TS, int NC, bool EDGE>
+// columns outside the grid; CUT: the right edge may cut a chunk.  p.bx and p.H are multiples of NC.
+template <bool STAR, int K, typename TS, int NC, bool EDGE, bool CUT = EDGE>
 __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeights<STAR>& ws, char* ring, int lane,
                                           int x0, int y0) {
     constexpr int NP = NC / 2, PF = kWarpRing, NQ = NC / 4;
@@ -118,7 +118,7 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
     const bool per = EDGE && p.periodic != 0;
     const bool mask = EDGE && !per;
     const bool zl = mask && (lane == 0 || c <= 0), zr = mask && (lane == 31 || c + NC >= nx);
-    const bool cut = mask && nx % NC != 0 && x0 - p.H + 32 * NC > nx;  // the right edge cuts a chunk
+    const bool cut = CUT && mask && nx % NC != 0 && x0 - p.H + 32 * NC > nx;  // the right edge cuts a chunk
     const int nsteps = ((ylast - y0) + 2 * K + 2) / 3 * 3;
     const TS* gin = static_cast<const TS*>(p.in);
     char* my = ring + lane * CB;
@@ -144,9 +144,9 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
                 cp_async<PB>(dst + j * PB, o ? gin + (long long)y * ld + pc[j] : gin, o);
             }
         } else {
-            const TS* g = ok ? src + (long long)s * ld : gin;
+            const TS* g = ok ? src + (long long)s * ld : gin;  // (past the tile: zero bytes are copied)
 #pragma unroll
-            for (int j = 0; j < NQ; ++j) cp_async<PB>(dst + j * PB, g + (ok ? 4 * j : 0), ok);
+            for (int j = 0; j < NQ; ++j) cp_async<PB>(dst + j * PB, g + 4 * j, ok);
         }
         cp_async_commit();
     };
@@ -207,7 +207,7 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
                             for (int q = 0; q < NP; ++q) X[q] = make_float2(0.f, 0.f);
                         }
                     }
-                    if (cut) {
+                    if (CUT && cut) {
 #pragma unroll
                         for (int q = 0; q < NP; ++q) {
                             X[q].x = c + q < nx ? X[q].x : 0.f;
@@ -239,6 +239,27 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
         }
     }
     cp_async_wait<0>();
+}
+
+// Warps per SM the registers must allow: the 5-point star at NC = 8 takes 220
+// registers (8 warps), the NC = 4 forms fit 128 (16).
+__host__ __device__ constexpr int warp_min_blocks(int NC) { return NC == 8 ? 8 : 16; }
+
+// A launch of one-warp CTAs over a whole grid: p.strips x tile rows, edge tiles first.
+template <bool STAR, int K, typename TS, int NC>
+__global__ void __launch_bounds__(32, warp_min_blocks(NC)) sweep_warp_kernel(const __grid_constant__ StreamParams p) {
+    __shared__ __align__(16) char ring[warp_ring_bytes<TS, NC>()];
+    const int lane = threadIdx.x;
+    int strip, tile;
+    stream_tile_of(blockIdx.x, p.strips, gridDim.x / p.strips, strip, tile);
+    const int x0 = strip * p.bx, y0 = tile * p.by;
+    const int ny = (int)p.ny, nx = (int)p.nx;
+    const int ylast = min(y0 + p.by, ny);
+    const bool interior = y0 - K >= 0 && ylast + warp_rows_after(K) <= ny && x0 - p.H >= 0 && x0 - p.H + 32 * NC <= nx;
+    const WarpWeights<STAR> ws([&](int i) { return p.w.w[i]; });
+    if (interior) warp_tile<STAR, K, TS, NC, false>(p, ws, ring, lane, x0, y0);
+    else if (nx % NC == 0) warp_tile<STAR, K, TS, NC, true, false>(p, ws, ring, lane, x0, y0);
+    else warp_tile<STAR, K, TS, NC, true>(p, ws, ring, lane, x0, y0);
 }
 
 }  // namespace gbst

@@ -1,0 +1,46 @@
+"""GPU tests of the one-warp streaming kernel of large radius-1 plans: the bits of
+the CTA-wide kernel at widths the right edge cuts, both boundaries, and the three
+storage types (same launches, so the same roundings)."""
+import pytest
+
+from paper_2605_07954_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TDT = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_07954_gb300 import build
+    build.build()
+
+
+# (4 or 8 columns per lane for the star) x (aligned, a chunk cut after 4, padded rows)
+@pytest.mark.parametrize("name", ["heat5", "box9"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("shape,boundary", [((4104, 4096), "zero"), ((4096, 4100), "periodic"), ((3700, 4099), "zero"),
+                                            ((6600, 7012), "zero"), ((6600, 7013), "zero"), ((6600, 7012), "periodic")])
+def test_same_bits_as_cta_wide_kernel(name, dtype, shape, boundary):
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights(name)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    x = torch.rand(shape, generator=g, device="cuda").to(TDT[dtype])
+    p = Plan(shape[0], shape[1], W, dtype=dtype, boundary=boundary)
+    q = Plan(shape[0], shape[1], W, dtype=dtype, boundary=boundary, threads=128 if name == "heat5" else 64)
+    assert p.info()["threads"] == 32 and p.info()["tb_depth"] == q.info()["tb_depth"] == 8
+    for T in (8, 19):
+        y = p.run(x, T)
+        assert torch.equal(y, q.run(x, T)), T
+        z = x.clone()
+        p.run(z, T, out=z)
+        # in place, an odd number of launches is cut otherwise, which 16-bit storage sees
+        if dtype == "f32":
+            assert torch.equal(z, y), T
+    p.close()
+    q.close()
