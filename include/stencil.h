@@ -250,8 +250,9 @@ stencil_status_t stencil_plan_status(stencil_plan_t* plan);
  * their results depend on the launch depths at the rounding level).
  *   residuals  DEVICE, floor(T/m) doubles, written.
  *   m          >= 1.
- * Each checked interval runs m-1 steps temporally blocked and its last step
- * as a single launch into a second buffer (the plan keeps two extra grids).
+ * The last launch of a checked interval stores its last two steps where the
+ * plan has a kernel that can (else m-1 steps run and then one apart); the plan
+ * keeps three extra grids (two where there is no room for three).
  */
 stencil_status_t stencil_run_residual(stencil_plan_t* plan, const void* in, void* out, int64_t T,
                                       int64_t m, double* residuals, stencil_stream_t stream);
@@ -273,8 +274,9 @@ const char* stencil_residual_last_error(void);
  *                  like the rest), or HOST memory (pageable or pinned: the call then
  *                  synchronises `stream` before it returns).  Every entry of the
  *                  square is returned, off-footprint ones included.
- *   ckpt_interval  steps between checkpoints; 0 = ceil(sqrt(T)).  The result does
- *                  not depend on it (same bits).
+ *   ckpt_interval  steps between checkpoints; 0 = choose: T (no checkpoints) while
+ *                  T + 3 grids take at most 1 GiB, else about sqrt(T).  The result
+ *                  does not depend on it (same bits).
  * States are recomputed from checkpoints, not stored: the plan allocates and
  * keeps (ceil(T/s) + s + 2) grids of scratch, s = ckpt_interval.  The weight
  * gradient is reduced deterministically (fixed order, FP64 partials).

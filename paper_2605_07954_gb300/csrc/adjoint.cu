@@ -8,22 +8,21 @@
 //     dL/du_0 = lambda_0.
 //
 // Memory: the states u_t are recomputed, not stored: a checkpoint every s
-// steps (s = ceil(sqrt(T)) by default) is written by a temporally blocked
+// steps (adj_interval: about sqrt(T), or one segment where all states fit) is written by a temporally blocked
 // forward pass; walking the segments backwards, each segment's s states are
 // recomputed from its checkpoint (temporally blocked launches that store every
 // time level), then the adjoint steps of the segment run from its last state
 // down to its first.  Both forward paths use the same per-point arithmetic, so
 // the result does not depend on s.
 //
-// adjoint_step_kernel fuses, for one step, the lambda update and the
-// weight-gradient products: a CTA stages a 32x64 tile of lambda_{t+1} and of
-// u_t with an R-wide halo in shared memory, writes lambda_t for the tile, and
-// adds the tile's (2R+1)^2 products lambda_{t+1} * shifted(u_t) to a per-tile
-// FP64 partial.  Tile t of a launch is always CTA t and launches are ordered,
-// so each partial sums its steps in a fixed order; a last kernel sums the
-// partials over tiles in a fixed order.  The gradient is deterministic.
-// adjoint_stream_kernel does the same step with rows streamed through
-// registers instead of a staged tile (radius 1, widths a multiple of 4).
+// One kernel per reverse step fuses the lambda update and the weight-gradient
+// products: each warp walks down the rows of lambda_{t+1} of its strip with a
+// window of them in registers, writes lambda_t, and adds its (2R+1)^2 products
+// to its CTA's FP64 partial.  Tile t of a launch is always CTA t and launches
+// are ordered, so each partial sums its steps in a fixed order; a last kernel
+// sums the partials over tiles in a fixed order.  The gradient is deterministic.
+// adjoint_stream_kernel is that step for radius 1 and widths a multiple of 4,
+// adjoint_rows_kernel for everything else.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -44,138 +43,161 @@ void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*));
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n,
                                  cudaStream_t st);
 
-constexpr int kAdjTX = 32;          // output tile columns (one per lane)
-constexpr int kAdjTY = 64;          // output tile rows
-constexpr int kAdjRowsPerThread = 8;  // 8 warps x 8 rows
+// One reverse step for any radius and width (radius 1 with widths a multiple of 4
+// has adjoint_stream_kernel below).  A warp owns 120 columns (lanes 1..30, 4 each;
+// lanes 0 and 31 hold halo columns) of kAdrRows output rows and walks down the
+// rows of lambda_{t+1} with the last 2R+1 of them in registers, each extended by
+// R columns per side (shuffles).  Per output row o of the walk:
+//   lambda_t[o][x] = sum_d W[d] lambda_{t+1}[o - dy][x - dx]      (dy-major, then dx)
+//   g[d]          += u_t[o][x] * lambda_{t+1}[o - dy][x - dx]
+// so u_t is read at the warp's own points only (the gradient's terms grouped by
+// the u_t point, as in adjoint_stream_kernel).  The row loop is rolled (7 rows of
+// 300-450 instructions would leave the instruction cache); the window moves down
+// by register copies.  Rows arrive two ahead, 16 bytes a lane, or element by
+// element where rows are not aligned.
+//
+// Gradient sums: two FP32 accumulators per tap and thread (even and odd rows: 16
+// products each), whose 128 sums of a CTA are added without rounding error
+// (TwoSum) before they go into its FP64 partial; that keeps the FP32 part no
+// longer than the staged-tile form's 8 products and 5 levels of lane sums.
+//
+// What bounds it: FMA issue, (13 or 49) + 49 FMAs per point for radius 3.  The
+// staged-tile form it replaces (one point per lane and row, both windows read
+// from shared memory) ran the 13-point star at 1000 x 1022 in 26.4 us a step:
+// now 14.4 (ncu).
+constexpr int kAdrWarps = 4;
+constexpr int kAdrRows = 8;     // output rows per warp
+constexpr int kAdrCols = 120;   // output columns per warp
 
-// One reverse step on a 32 x 64 tile.  Lane tx owns column x0 + tx and warp ty
-// rows y0 + 8 ty .. + 7; it walks its rows keeping the last 2R+1 staged rows
-// of lambda_{t+1} and u_t (its column +- R) in registers, so each row costs
-// 2 (2R+1) shared-memory loads for (2R+1)^2 lambda FMAs and (2R+1)^2 gradient FMAs.
-template <int R>
-__global__ void __launch_bounds__(256)
-    adjoint_step_kernel(const float* __restrict__ lam_in, const float* __restrict__ u,
-                        float* __restrict__ lam_out, double* __restrict__ partials, int ny, int nx,
-                        int periodic, Weights w, int tiles_x) {
-    constexpr int D = 2 * R + 1;
-    constexpr int SY = kAdjTY + 2 * R, SX = kAdjTX + 2 * R;
-    __shared__ float sl[SY][SX + 1];
-    __shared__ float su[SY][SX + 1];
-    __shared__ float red[8][D * D];
-    const int tx = threadIdx.x, ty = threadIdx.y;  // (32, 8)
-    const int x0 = (blockIdx.x % tiles_x) * kAdjTX;
-    const int y0 = (blockIdx.x / tiles_x) * kAdjTY;
-
-    // Stage both tiles with their halo (zero outside, or wrapped).  Every
-    // thread issues all of its loads before its first shared-memory store, so
-    // the DRAM latencies overlap.  Item i = tid + 256 it is staged row i / SX,
-    // column i % SX, advanced without division.
-    {
-        constexpr int ITEMS = SY * SX, ITERS = (ITEMS + 255) / 256;
-        const int tid0 = ty * 32 + tx;
-        int r = tid0 / SX, c = tid0 % SX;
-        float va[ITERS], vb[ITERS];
-        int ra[ITERS], ca[ITERS];
+// Row y of g at the lane's columns c .. c + 3: zero outside the grid, or wrapped.
+__device__ __forceinline__ void adr_load(float (&v)[4], const float* __restrict__ g, int y, int c, int ny, int nx,
+                                         bool per, bool vec) {
+    v[0] = v[1] = v[2] = v[3] = 0.f;
+    if (per) {
+        if ((unsigned)y >= (unsigned)ny) y = (y % ny + ny) % ny;
+    } else if ((unsigned)y >= (unsigned)ny) {
+        return;
+    }
+    const float* row = g + (size_t)y * (size_t)nx;
+    if (vec) {  // nx % 4 == 0: a chunk lies wholly inside or outside, and so does its wrapped image
+        if (per) c = (unsigned)c < (unsigned)nx ? c : (c % nx + nx) % nx;
+        if ((unsigned)c < (unsigned)nx) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(row + c));
+            v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        }
+        return;
+    }
 #pragma unroll
-        for (int it = 0; it < ITERS; ++it) {
-            ra[it] = r;
-            ca[it] = c;
-            va[it] = vb[it] = 0.f;
-            if (r < SY) {
-                int y = y0 - R + r, x = x0 - R + c;
-                bool ok = y >= 0 && y < ny && x >= 0 && x < nx;
-                if (periodic) {
-                    y = (y % ny + ny) % ny;
-                    x = (x % nx + nx) % nx;
-                    ok = true;
-                }
-                if (ok) {
-                    const size_t i = (size_t)y * nx + x;
-                    va[it] = __ldg(lam_in + i);
-                    vb[it] = __ldg(u + i);
-                }
+    for (int e = 0; e < 4; ++e) {
+        int x = c + e;
+        if (per && (unsigned)x >= (unsigned)nx) x = (x % nx + nx) % nx;
+        if ((unsigned)x < (unsigned)nx) v[e] = __ldg(row + x);
+    }
+}
+
+template <int R, bool STAR>
+__global__ void __launch_bounds__(kAdrWarps * 32, 2)
+    adjoint_rows_kernel(const float* __restrict__ lam_in, const float* __restrict__ u, float* __restrict__ lam_out,
+                        double* __restrict__ partials, int ny, int nx, int periodic, Weights w, int tiles_x, int vec) {
+    constexpr int D = 2 * R + 1, E = 4 + 2 * R, NR = kAdrRows + 2 * R;
+    constexpr unsigned FULL = 0xffffffffu;
+    static_assert(NR % 2 == 0, "the row loop runs in pairs");
+    __shared__ float sums[D * D][kAdrWarps * 32 + 1];
+    __shared__ double half[D * D];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = ((int)blockIdx.x % tiles_x) * kAdrCols - 4 + 4 * lane;
+    const int yb = ((int)blockIdx.x / tiles_x) * (kAdrWarps * kAdrRows) + warp * kAdrRows;
+    const bool per = periodic != 0;
+    const bool own = lane >= 1 && lane <= 30 && c < nx;
+    float win[D][E];
+    float g[2][D * D];
+#pragma unroll
+    for (int k = 0; k < D * D; ++k) g[0][k] = g[1][k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+#pragma unroll
+        for (int e = 0; e < E; ++e) win[k][e] = 0.f;
+    float lv[2][4], uv[2][4];  // rows in flight: slot = walked row mod 2
+    auto load = [&](int i) {   // walked row i (lambda row yb - R + i, u row yb + i - 2R)
+        adr_load(lv[i & 1], lam_in, yb - R + i, c, ny, nx, per, vec != 0);
+        const int o = yb + i - 2 * R;
+        uv[i & 1][0] = uv[i & 1][1] = uv[i & 1][2] = uv[i & 1][3] = 0.f;
+        if (own && i >= 2 * R && o < ny) adr_load(uv[i & 1], u, o, c, ny, nx, false, vec != 0);
+    };
+    load(0);
+    load(1);
+#pragma unroll 1
+    for (int i0 = 0; i0 < NR; i0 += 2) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int i = i0 + j;
+#pragma unroll
+            for (int k = 0; k < D - 1; ++k)
+#pragma unroll
+                for (int e = 0; e < E; ++e) win[k][e] = win[k + 1][e];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) win[D - 1][R + e] = lv[j][e];
+#pragma unroll
+            for (int e = 0; e < R; ++e) {
+                win[D - 1][e] = __shfl_up_sync(FULL, lv[j][4 - R + e], 1);
+                win[D - 1][R + 4 + e] = __shfl_down_sync(FULL, lv[j][e], 1);
             }
-            c += 256 % SX;
-            r += 256 / SX;
-            if (c >= SX) {
-                c -= SX;
-                ++r;
+            float uu[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) uu[e] = uv[j][e];
+            if (i + 2 < NR) {  // (j is i's parity: the slot just consumed)
+                adr_load(lv[j], lam_in, yb - R + i + 2, c, ny, nx, per, vec != 0);
+                const int o2 = yb + i + 2 - 2 * R;
+                uv[j][0] = uv[j][1] = uv[j][2] = uv[j][3] = 0.f;
+                if (own && i + 2 >= 2 * R && o2 < ny) adr_load(uv[j], u, o2, c, ny, nx, false, vec != 0);
+            }
+            const int o = yb + i - 2 * R;
+            if (i < 2 * R || o >= ny) continue;
+            // window row k holds lambda row o - R + k, column e of it grid column c - R + e
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int dy = -R; dy <= R; ++dy)
+#pragma unroll
+                for (int dx = -R; dx <= R; ++dx) {
+                    const int t = (dy + R) * D + dx + R;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float l = win[R - dy][R + e - dx];
+                        if (!STAR || dy == 0 || dx == 0) acc[e] = fmaf(w.w[t], l, acc[e]);
+                        g[j][t] = fmaf(uu[e], l, g[j][t]);
+                    }
+                }
+            if (own) {
+                float* row = lam_out + (size_t)o * (size_t)nx + c;
+                if (vec) {
+                    *reinterpret_cast<float4*>(row) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (c + e < nx) row[e] = acc[e];
+                }
             }
         }
+    }
+    // Fixed order: thread (tap, half) adds the 64 sums of two warps, sum and rounding
+    // error apart.
 #pragma unroll
-        for (int it = 0; it < ITERS; ++it) {
-            if (ra[it] < SY) {
-                sl[ra[it]][ca[it]] = va[it];
-                su[ra[it]][ca[it]] = vb[it];
-            }
+    for (int k = 0; k < D * D; ++k) sums[k][threadIdx.x] = g[0][k] + g[1][k];
+    __syncthreads();
+    for (int t = threadIdx.x; t < 2 * D * D; t += kAdrWarps * 32) {
+        const int k = t % (D * D), h = t / (D * D);
+        float s = 0.f, err = 0.f;
+        for (int i = 0; i < 64; ++i) {
+            const float v = sums[k][64 * h + i], n = s + v, z = n - s;
+            err += (s - (n - z)) + (v - z);
+            s = n;
         }
+        const double d = (double)s + (double)err;
+        if (h) half[k] = d;
+        else partials[(size_t)blockIdx.x * D * D + k] += d;
     }
     __syncthreads();
-
-    float g[D * D];
-#pragma unroll
-    for (int k = 0; k < D * D; ++k) g[k] = 0.f;
-    // Register windows: wl[i][e] = lambda staged row (row0 + i), column tx + e;
-    // wu likewise for u.  The output row o = r0 + k needs lambda rows o-R..o+R
-    // (flipped correlation) and u rows o-R..o+R.
-    const int r0 = ty * kAdjRowsPerThread;  // first output row (tile-local)
-    float wl[D][D], wu[D][D];
-#pragma unroll
-    for (int i = 0; i < D - 1; ++i)
-#pragma unroll
-        for (int e = 0; e < D; ++e) {
-            wl[i + 1][e] = sl[r0 + i][tx + e];
-            wu[i + 1][e] = su[r0 + i][tx + e];
-        }
-#pragma unroll
-    for (int k = 0; k < kAdjRowsPerThread; ++k) {
-        // slide: drop the oldest staged row, append staged row r0 + k + 2R
-#pragma unroll
-        for (int i = 0; i < D - 1; ++i)
-#pragma unroll
-            for (int e = 0; e < D; ++e) {
-                wl[i][e] = wl[i + 1][e];
-                wu[i][e] = wu[i + 1][e];
-            }
-#pragma unroll
-        for (int e = 0; e < D; ++e) {
-            wl[D - 1][e] = sl[r0 + k + 2 * R][tx + e];
-            wu[D - 1][e] = su[r0 + k + 2 * R][tx + e];
-        }
-        // window row i holds staged row r0 + k + i, i.e. grid row o - R + i for o = y0 + r0 + k
-        const int y = y0 + r0 + k, x = x0 + tx;
-        if (y >= ny || x >= nx) continue;
-        // lambda_t[o] = sum_d W[d] lambda_{t+1}[o - d], dy-major then dx
-        float acc = 0.f;
-#pragma unroll
-        for (int dy = -R; dy <= R; ++dy)
-#pragma unroll
-            for (int dx = -R; dx <= R; ++dx)
-                acc = fmaf(w.w[(dy + R) * D + (dx + R)], wl[R - dy][R - dx], acc);
-        lam_out[(size_t)y * nx + x] = acc;
-        // dL/dW[d] += lambda_{t+1}[o] * u_t[o + d]
-        const float lp = wl[R][R];
-#pragma unroll
-        for (int dy = -R; dy <= R; ++dy)
-#pragma unroll
-            for (int dx = -R; dx <= R; ++dx)
-                g[(dy + R) * D + (dx + R)] = fmaf(lp, wu[R + dy][R + dx], g[(dy + R) * D + (dx + R)]);
-    }
-    // Fixed-order reduction: butterfly within each warp, then warps in order.
-#pragma unroll
-    for (int k = 0; k < D * D; ++k) {
-        float v = g[k];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (tx == 0) red[ty][k] = v;
-    }
-    __syncthreads();
-    const int tid = ty * 32 + tx;
-    if (tid < D * D) {
-        double s = 0.0;
-        for (int wv = 0; wv < 8; ++wv) s += (double)red[wv][tid];
-        partials[(size_t)blockIdx.x * D * D + tid] += s;
-    }
+    if (threadIdx.x < D * D) partials[(size_t)blockIdx.x * D * D + threadIdx.x] += half[threadIdx.x];
 }
 
 // grad_w[k] = sum over tiles of partials[tile][k] in a fixed order: thread i of
@@ -216,7 +238,7 @@ __global__ void __launch_bounds__(256)
 // term is counted once, by the warp that owns the u_t row, and lambda_{t+1}
 // outside the grid is zero (or wrapped) as in the lambda update, so u_t is
 // read only at the warp's own points, without halo.  Per output the lambda
-// update is adjoint_step_kernel's, in the same order (bit-identical lambda);
+// update adds dy-major, then dx, as adjoint_rows_kernel does (same bits);
 // each thread adds its gradient products row by row, the CTA reduces them in
 // a fixed order into its FP64 partial.
 //
@@ -508,17 +530,15 @@ __global__ void __launch_bounds__(kAdsWarps * 32, 5)
     }
 }
 
-// Radius 1 only: at radius 2 the two register windows (5 rows x 8 columns
-// each) take the kernel to 225 registers, and the staged-tile step is kept.
 static const void* adjoint_stream_kernel_fn(int R) {
     return R == 1 ? (const void*)adjoint_stream_kernel<1> : nullptr;
 }
 
-static const void* adjoint_kernel(int R) {
+static const void* adjoint_rows_kernel_fn(int R, bool star) {
     switch (R) {
-        case 1: return (const void*)adjoint_step_kernel<1>;
-        case 2: return (const void*)adjoint_step_kernel<2>;
-        case 3: return (const void*)adjoint_step_kernel<3>;
+        case 1: return star ? (const void*)adjoint_rows_kernel<1, true> : (const void*)adjoint_rows_kernel<1, false>;
+        case 2: return star ? (const void*)adjoint_rows_kernel<2, true> : (const void*)adjoint_rows_kernel<2, false>;
+        case 3: return star ? (const void*)adjoint_rows_kernel<3, true> : (const void*)adjoint_rows_kernel<3, false>;
         default: return nullptr;
     }
 }
@@ -556,6 +576,27 @@ void adj_scratch_free(void* v) {
     if (sc->base) cudaFree(sc->base);
     if (sc->partials) cudaFree(sc->partials);
     delete sc;
+}
+
+int64_t adj_sqrt(int64_t T) { return (int64_t)std::ceil(std::sqrt((double)T)); }
+
+// Steps between checkpoints.  By default the whole run is one segment while its
+// states take at most 1 GiB: no checkpoint pass is needed then.  Otherwise
+// ceil(sqrt(T)), for radius 1 rounded up to whole launches of 8 steps (Heat 4096^2
+// x 128: 12 steps a segment 3.16 ms of forward launches, 16 steps 2.82 ms).
+int64_t adj_interval(int64_t T, int64_t asked, int R, size_t bytes) {
+    if (asked > 0) return std::min<int64_t>(asked, T);
+    if ((double)(T + 3) * (double)bytes <= (double)(1ull << 30)) return T;
+    const int64_t s = adj_sqrt(T);
+    return std::min<int64_t>(R == 1 ? (s + 7) / 8 * 8 : s, T);
+}
+
+bool adj_star(const Weights& w, int R) {
+    const int D = 2 * R + 1;
+    for (int a = 0; a < D; ++a)
+        for (int c = 0; c < D; ++c)
+            if (a != R && c != R && w.w[a * D + c] != 0.f) return false;
+    return true;
 }
 
 stencil_status_t adj_scratch(stencil_plan_t* plan, size_t grids, size_t grid_bytes, size_t npartials,
@@ -621,23 +662,26 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
 
     // The row-streaming step where it applies (its 16-byte row chunks need
     // nx % 4 == 0, and the buffers below are then 16-byte aligned), else the
-    // staged-tile step.
+    // any-width one.
     const bool streamed = adjoint_stream_kernel_fn(R) != nullptr && nx % 4 == 0;
-    const int tiles_x = streamed ? (nx + kAdsCols - 1) / kAdsCols : (nx + kAdjTX - 1) / kAdjTX;
-    const int tile_rows = streamed ? kAdsWarps * kAdsRows : kAdjTY;
+    const int tiles_x = streamed ? (nx + kAdsCols - 1) / kAdsCols : (nx + kAdrCols - 1) / kAdrCols;
+    const int tile_rows = streamed ? kAdsWarps * kAdsRows : kAdrWarps * kAdrRows;
     const int tiles = tiles_x * ((ny + tile_rows - 1) / tile_rows);
     if (T == 0) {
         if (grad_u0 != grad_uT) ACK(cudaMemcpyAsync(grad_u0, grad_uT, bytes, cudaMemcpyDeviceToDevice, st));
         if (grad_w) ACK(cudaMemsetAsync(grad_w, 0, sizeof(double) * D * D, st));
         return STENCIL_OK;
     }
-    const int64_t sgm = ckpt_interval > 0 ? std::min<int64_t>(ckpt_interval, T)
-                                          : (int64_t)std::ceil(std::sqrt((double)T));
-    const int64_t nseg = (T + sgm - 1) / sgm;
+    int64_t sgm = adj_interval(T, ckpt_interval, R, bytes);
+    int64_t nseg = (T + sgm - 1) / sgm;
     // Buffers: nseg checkpoints, sgm segment states, two adjoint grids.
     AdjScratch* sc = nullptr;
-    const size_t grids = (size_t)nseg + (size_t)sgm + 2;
-    s = adj_scratch(plan, grids, bytes, (size_t)(tiles + 1) * D * D, &sc);
+    s = adj_scratch(plan, (size_t)nseg + (size_t)sgm + 2, bytes, (size_t)(tiles + 1) * D * D, &sc);
+    if (s == STENCIL_ERR_OOM && ckpt_interval == 0 && sgm != adj_sqrt(T)) {  // the least memory, then
+        sgm = adj_sqrt(T);
+        nseg = (T + sgm - 1) / sgm;
+        s = adj_scratch(plan, (size_t)nseg + (size_t)sgm + 2, bytes, (size_t)(tiles + 1) * D * D, &sc);
+    }
     if (s != STENCIL_OK) return s;
     float* ckpt = sc->base;
     float* seg = sc->base + (size_t)nseg * n;
@@ -653,9 +697,11 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
     }
     ACK(cudaMemcpyAsync(lam[0], grad_uT, bytes, cudaMemcpyDeviceToDevice, st));
     int cur = 0;
-    const void* kfn = streamed ? adjoint_stream_kernel_fn(R) : adjoint_kernel(R);
+    // (a star's off-axis weights are zero: the lambda update skips them)
+    const void* kfn = streamed ? adjoint_stream_kernel_fn(R) : adjoint_rows_kernel_fn(R, adj_star(wf, R));
     if (!kfn) return afail(STENCIL_ERR_UNSUPPORTED, "no adjoint kernel for this radius");
-    const dim3 block = streamed ? dim3(kAdsWarps * 32) : dim3(32, 8);
+    const dim3 block = dim3(streamed ? kAdsWarps * 32 : kAdrWarps * 32);
+    int vec = nx % 4 == 0;
     int periodic = info.boundary == STENCIL_BOUNDARY_PERIODIC;
     std::vector<float*> segp((size_t)sgm);
     for (int64_t j = nseg - 1; j >= 0; --j) {
@@ -673,8 +719,8 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
             const float* ut = t == 0 ? state0 : seg + (size_t)t * n;
             const float* lin = lam[cur];
             float* lout = lam[cur ^ 1];
-            void* args[] = {(void*)&lin, (void*)&ut, (void*)&lout, (void*)&partials,
-                            (void*)&ny, (void*)&nx, (void*)&periodic, (void*)&wadj, (void*)&tiles_x};
+            void* args[] = {(void*)&lin, (void*)&ut, (void*)&lout, (void*)&partials, (void*)&ny,
+                            (void*)&nx,  (void*)&periodic, (void*)&wadj, (void*)&tiles_x, (void*)&vec};
             ACK(cudaLaunchKernel(kfn, dim3((unsigned)tiles), block, args, 0, st));
             cur ^= 1;
         }
@@ -702,15 +748,20 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
 int64_t stencil_adjoint_launches(const stencil_plan_t* plan, int64_t T, int64_t ckpt_interval) {
     if (!plan || T < 0 || ckpt_interval < 0) return -1;
     if (T == 0) return 0;
-    const int64_t sgm = ckpt_interval > 0 ? std::min<int64_t>(ckpt_interval, T)
-                                          : (int64_t)std::ceil(std::sqrt((double)T));
-    const int64_t nseg = (T + sgm - 1) / sgm;
-    int64_t L = (nseg - 1) * stencil_run_launches(plan, sgm);  // checkpoints
     stencil_plan_info_t info{};
     const bool fused = stencil_plan_info(plan, &info) == STENCIL_OK && info.dtype == STENCIL_F32 &&
                        info.nx % 4 == 0;
+    const int64_t sgm = adj_interval(T, ckpt_interval, info.radius, (size_t)info.ny * (size_t)info.nx * sizeof(float));
+    const int64_t nseg = (T + sgm - 1) / sgm;
+    int64_t L = (nseg - 1) * stencil_run_launches(plan, sgm);  // checkpoints
+    const bool resident = info.kernel == STENCIL_KERNEL_RESIDENT && info.ctas == 1 && info.threads != 1024 &&
+                          !(info.boundary == STENCIL_BOUNDARY_PERIODIC && info.nx % 4 != 0);
     for (int64_t j = 0; j < nseg; ++j) {  // segment recompute: all-states launches of 8/4/2/1 steps
         int64_t m = std::min<int64_t>(sgm, T - j * sgm) - 1;
+        if (resident) {  // (register tiles: one launch)
+            L += m > 0;
+            continue;
+        }
         if (!fused) {
             L += m * stencil_run_launches(plan, 1);
             continue;

@@ -36,6 +36,7 @@ StreamKernelRef get_stream_pad_kernel_f32(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_bf16(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_f16(int R, int star, int k);
 const void* get_warp_kernel(int star, int dtype, int nc);
+const void* get_warp_states_kernel(int star);
 StreamKernelRef get_stream_tma_kernel_r1(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r2(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r3(int star, int k);
@@ -305,6 +306,20 @@ constexpr int kWarpDepth = 8;
 constexpr int kWarpMinRows = 44;      // NC = 4
 constexpr int kWarpMinRowsWide = 128;  // NC = 8: fewer warps, so taller tiles before it pays
 
+struct WarpTiles {
+    int bx, by, strips, tiles;
+};
+
+// One wave of one-warp tiles with nc columns per lane.
+static WarpTiles warp_tiles(const stencil_plan* p, int nc) {
+    const int64_t bx_max = 32 * nc - 2 * kWarpDepth;
+    const int64_t bx = ceil_div(ceil_div(p->nx, ceil_div(p->nx, bx_max)), nc) * nc;
+    const int64_t strips = ceil_div(p->nx, bx);
+    const int64_t warps = (int64_t)p->sms * (nc == 8 ? 8 : 16);
+    const int64_t by = ceil_div(p->ny, std::max<int64_t>(1, warps / strips));
+    return {(int)bx, (int)by, (int)strips, (int)ceil_div(p->ny, by)};
+}
+
 static void configure_warp(stencil_plan* p, int threads_asked) {
     p->warp_nc = 0;
     const stencil_options_t& o = p->opt;
@@ -313,17 +328,13 @@ static void configure_warp(stencil_plan* p, int threads_asked) {
         o.load != STENCIL_LOAD_AUTO || threads_asked != default_threads(p->R, p->star))
         return;
     for (int nc = p->star ? 8 : 4; nc >= 4; nc -= 4) {
-        const int64_t bx_max = 32 * nc - 2 * kWarpDepth;
-        const int64_t bx = ceil_div(ceil_div(p->nx, ceil_div(p->nx, bx_max)), nc) * nc;
-        const int64_t strips = ceil_div(p->nx, bx);
-        const int64_t warps = (int64_t)p->sms * (nc == 8 ? 8 : 16);
-        const int64_t by = ceil_div(p->ny, std::max<int64_t>(1, warps / strips));
-        if (by < (nc == 8 ? kWarpMinRowsWide : kWarpMinRows)) continue;
+        const WarpTiles t = warp_tiles(p, nc);
+        if (t.by < (nc == 8 ? kWarpMinRowsWide : kWarpMinRows)) continue;
         p->warp_nc = nc;
-        p->warp_bx = (int)bx;
-        p->warp_by = (int)by;
-        p->warp_strips = (int)strips;
-        p->warp_tiles = (int)ceil_div(p->ny, by);
+        p->warp_bx = t.bx;
+        p->warp_by = t.by;
+        p->warp_strips = t.strips;
+        p->warp_tiles = t.tiles;
         return;
     }
 }
@@ -880,9 +891,90 @@ static std::vector<int> launch_depths(const stencil_plan* p, int64_t T) {
 // Each state is the same bits as stencil_run produces (same arithmetic per
 // point, independent of the launch depths).
 
+// One all-states launch of d steps: level l+1 to outs[l] (null: not stored, but the last must be).
+static stencil_status_t launch_states(stencil_plan_t* p, const void* src, float* const* outs, int d, cudaStream_t st) {
+    if (d == kWarpDepth && p->R == 1) {
+        // one-warp tiles where they have enough rows (4096^2 5-point star: 96 us
+        // per launch, 153 CTA-wide)
+        const WarpTiles t = warp_tiles(p, 4);
+        if (t.by >= kWarpMinRows) {
+            StreamParams sp = stream_params(p, d);
+            sp.in = src;
+            sp.out = outs[d - 1];
+            sp.H = kWarpDepth;
+            sp.bx = t.bx;
+            sp.by = t.by;
+            sp.strips = t.strips;
+            sp.vec = 1;
+            for (int l = 0; l < d - 1; ++l) sp.lvl_out[l] = outs[l];
+            void* args[] = {&sp};
+            CK(cudaLaunchKernel(get_warp_states_kernel(p->star), dim3((unsigned)(t.strips * t.tiles)), dim3(32), args, 0,
+                                st));
+            return STENCIL_OK;
+        }
+    }
+    const int threads = 128;
+    const StreamKernelRef r = get_stream_states_kernel(p->R, p->star, d);
+    if (!r.fn) return fail(STENCIL_ERR_UNSUPPORTED, "no all-states kernel");
+    const int H = (p->R * d + 3) / 4 * 4;
+    const int64_t strips = ceil_div(p->nx, 4 * threads - 2 * H);
+    const int bx = (int)(ceil_div(ceil_div(p->nx, strips), 4) * 4);
+    const int nt = (int)(ceil_div(ceil_div(bx + 2 * H, 4), 32) * 32);
+    const int smem = stream_smem_bytes(p->R, d, 4, true, false, nt);
+    const unsigned bit = 1u << d;
+    static std::mutex mu;
+    {
+        std::lock_guard<std::mutex> g(mu);
+        static unsigned set_bits[3][2] = {};
+        if (!(set_bits[p->R - 1][p->star] & bit)) {
+            CK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    stream_smem_bytes(p->R, d, 4, true, false, kStreamMaxThreads)));
+            set_bits[p->R - 1][p->star] |= bit;
+        }
+    }
+    int per_sm = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.fn, nt, smem));
+    if (per_sm < 1) return fail(STENCIL_ERR_UNSUPPORTED, "all-states kernel does not fit on an SM");
+    const int64_t want = std::max<int64_t>(1, (int64_t)per_sm * p->sms / strips);
+    const int64_t by_min = std::max<int64_t>(8, 4LL * p->R * d);
+    int64_t tiles_y = std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(p->ny, by_min)));
+    const int by = (int)ceil_div(p->ny, tiles_y);
+    tiles_y = ceil_div(p->ny, by);
+    StreamParams sp = stream_params(p, d);
+    sp.in = src;
+    sp.out = outs[d - 1];
+    sp.H = H;
+    sp.bx = bx;
+    sp.by = by;
+    sp.strips = (int)strips;
+    sp.vec = 1;
+    for (int l = 0; l < d - 1; ++l) sp.lvl_out[l] = outs[l];
+    void* args[] = {&sp};
+    CK(cudaLaunchKernel(r.fn, dim3((unsigned)(strips * tiles_y)), dim3((unsigned)nt), args, (size_t)smem, st));
+    return STENCIL_OK;
+}
+
 namespace gbst {
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n,
                                  cudaStream_t st) {
+    // Chip-resident plans: every state in one launch (13-point star 1000 x 1022: a
+    // single-step launch per state took 13 us each).  Not for periodic ragged widths,
+    // whose bits depend on how the steps are grouped.
+    bool strided = p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && p->dtype == STENCIL_F32 && n >= 1 &&
+                   n < (1 << 30) && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0);
+    const int64_t stride = n > 1 ? outs[1] - outs[0] : 0;
+    for (int64_t i = 1; i < n && strided; ++i) strided = outs[i] - outs[i - 1] == stride;
+    if (strided) {
+        const int vec = p->nx % 4 == 0 && stride % 4 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)outs[0] % 16 == 0;
+        const cudaError_t e =
+            launch_grid(p->grid, p->R, p->star, p->dtype, p->boundary == STENCIL_BOUNDARY_PERIODIC, in, outs[n - 1],
+                        (int)p->ny, (int)p->nx, vec, (int)n, p->grid.k, p->grid_mem, p->status,
+                        (long long)(p->opt.timeout_ms > 0 ? p->opt.timeout_ms : 2000) * 1000000LL,
+                        p->opt.debug_withhold, p->w, st, outs[0], stride);
+        if (e == cudaSuccess) return STENCIL_OK;
+        if (e != cudaErrorCooperativeLaunchTooLarge) CK(e);
+        cudaGetLastError();  // (fewer SMs than the device reports: the paths below)
+    }
     bool fused = p->dtype == STENCIL_F32 && p->nx % 4 == 0 && (uintptr_t)in % 16 == 0;
     for (int64_t i = 0; i < n && fused; ++i) fused = (uintptr_t)outs[i] % 16 == 0;
     if (!fused) {
@@ -894,65 +986,70 @@ stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const
         }
         return STENCIL_OK;
     }
-    const int threads = 128;
     const void* src = in;
     for (int64_t i = 0; i < n;) {
         int d = 8;
-        StreamKernelRef r{nullptr, 0};
-        for (; d >= 1; d /= 2) {
-            if (d > n - i) continue;
-            r = get_stream_states_kernel(p->R, p->star, d);
-            if (r.fn) break;
-        }
-        if (!r.fn) return fail(STENCIL_ERR_UNSUPPORTED, "no all-states kernel");
-        const int H = (p->R * d + 3) / 4 * 4;
-        const int64_t strips = ceil_div(p->nx, 4 * threads - 2 * H);
-        const int bx = (int)(ceil_div(ceil_div(p->nx, strips), 4) * 4);
-        const int nt = (int)(ceil_div(ceil_div(bx + 2 * H, 4), 32) * 32);
-        const int smem = stream_smem_bytes(p->R, d, 4, true, false, nt);
-        const unsigned bit = 1u << d;
-        static std::mutex mu;
-        {
-            std::lock_guard<std::mutex> g(mu);
-            static unsigned set_bits[3][2] = {};
-            if (!(set_bits[p->R - 1][p->star] & bit)) {
-                CK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        stream_smem_bytes(p->R, d, 4, true, false, kStreamMaxThreads)));
-                set_bits[p->R - 1][p->star] |= bit;
-            }
-        }
-        int per_sm = 0;
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.fn, nt, smem));
-        if (per_sm < 1) return fail(STENCIL_ERR_UNSUPPORTED, "all-states kernel does not fit on an SM");
-        const int64_t want = std::max<int64_t>(1, (int64_t)per_sm * p->sms / strips);
-        const int64_t by_min = std::max<int64_t>(8, 4LL * p->R * d);
-        int64_t tiles_y = std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(p->ny, by_min)));
-        const int by = (int)ceil_div(p->ny, tiles_y);
-        tiles_y = ceil_div(p->ny, by);
-        StreamParams sp{};
-        sp.in = src;
-        sp.out = outs[i + d - 1];
-        sp.ny = p->ny;
-        sp.nx = p->nx;
-        sp.ld = sp.ld_out = p->nx;
-        sp.nlev = d;
-        sp.H = H;
-        sp.bx = bx;
-        sp.by = by;
-        sp.strips = (int)strips;
-        sp.periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
-        sp.vec = 1;
-        sp.status = p->status;
-        sp.wait_ns = (long long)(p->opt.timeout_ms > 0 ? p->opt.timeout_ms : 2000) * 1000000LL;
-        sp.w = p->w;
-        for (int t = 0; t < kMaxTaps; ++t) sp.w2.w2[t] = make_float2(p->w.w[t], p->w.w[t]);
-        for (int l = 0; l < d - 1; ++l) sp.lvl_out[l] = outs[i + l];
-        void* args[] = {&sp};
-        CK(cudaLaunchKernel(r.fn, dim3((unsigned)(strips * tiles_y)), dim3((unsigned)nt), args, (size_t)smem, st));
+        for (; d > 1; d /= 2)
+            if (d <= n - i && get_stream_states_kernel(p->R, p->star, d).fn) break;
+        stencil_status_t s = launch_states(p, src, outs + i, d, st);
+        if (s != STENCIL_OK) return s;
         src = outs[i + d - 1];
         i += d;
     }
     return STENCIL_OK;
+}
+
+// u_{m-1} and u_m (m >= 2, FP32), the last launch storing both, in two of the
+// grids g1, g2 and g0 (*prev, *next).  `in` may be g0, and is then overwritten
+// when launches come before that last one.  STENCIL_ERR_UNSUPPORTED, with nothing
+// enqueued, where the plan has no kernel that stores two steps.
+stencil_status_t plan_run_last_two(stencil_plan_t* p, const void* in, void* g1, void* g2, void* g0, int64_t m,
+                                   cudaStream_t st, const void** prev, const void** next) {
+    if (p->dtype != STENCIL_F32 || m < 2 || (p->opt.autotune && !p->tuned)) return STENCIL_ERR_UNSUPPORTED;
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && m < (1 << 30) &&
+        !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0)) {
+        const int vec = p->nx % 4 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)g1 % 16 == 0 && (uintptr_t)g2 % 16 == 0;
+        const cudaError_t e = launch_grid(p->grid, p->R, p->star, p->dtype, p->boundary == STENCIL_BOUNDARY_PERIODIC, in,
+                                          g2, (int)p->ny, (int)p->nx, vec, (int)m, p->grid.k, p->grid_mem, p->status,
+                                          (long long)(p->opt.timeout_ms > 0 ? p->opt.timeout_ms : 2000) * 1000000LL,
+                                          p->opt.debug_withhold, p->w, st, static_cast<float*>(g1), 0, (int)m - 1);
+        p->last_stream = st;
+        *prev = g1;
+        *next = g2;
+        if (e == cudaSuccess) return STENCIL_OK;
+        if (e != cudaErrorCooperativeLaunchTooLarge) CK(e);
+        cudaGetLastError();
+        return STENCIL_ERR_UNSUPPORTED;
+    }
+    if (p->kernel != STENCIL_KERNEL_STREAM || p->nx % 4 != 0 || ((uintptr_t)in | (uintptr_t)g1 | (uintptr_t)g2 | (uintptr_t)g0) % 16 != 0)
+        return STENCIL_ERR_UNSUPPORTED;
+    // the depth of the last launch that leaves the fewest launches before it
+    int best = 0;
+    size_t fewest = 0;
+    for (int d = 2; d <= 8; d *= 2) {  // (of equals the shallowest: it stores its levels at less cost)
+        if (d > m || !get_stream_states_kernel(p->R, p->star, d).fn) continue;
+        const size_t before = launch_depths(p, m - d).size();
+        if (!best || before < fewest) {
+            best = d;
+            fewest = before;
+        }
+    }
+    // (m = 8 j + 1 and the like: as many launches with the step apart, which stores one grid less)
+    if (!best || launch_depths(p, m - 1).size() <= fewest) return STENCIL_ERR_UNSUPPORTED;
+    void *a = g1, *b = g2;
+    if (m > best) {
+        stencil_status_t s = stencil_run(p, in, g2, m - best, st);
+        if (s != STENCIL_OK) return s;
+        in = g2;
+        b = g0;
+    }
+    p->last_stream = st;
+    float* outs[8] = {};
+    outs[best - 2] = static_cast<float*>(a);
+    outs[best - 1] = static_cast<float*>(b);
+    *prev = a;
+    *next = b;
+    return launch_states(p, in, outs, best, st);
 }
 }  // namespace gbst
 

@@ -11,6 +11,19 @@ GridKernelRef get_grid_kernel_r1(int star, int rb);
 GridKernelRef get_grid_kernel_r2(int star, int rb);
 GridKernelRef get_grid_kernel_r3(int star, int rb);
 
+GridKernelRef get_grid_states_kernel_r1(int star, int rb);
+GridKernelRef get_grid_states_kernel_r2(int star, int rb);
+GridKernelRef get_grid_states_kernel_r3(int star, int rb);
+
+static GridKernelRef grid_states_kernel(int R, int star, int rb) {
+    switch (R) {
+        case 1: return get_grid_states_kernel_r1(star, rb);
+        case 2: return get_grid_states_kernel_r2(star, rb);
+        case 3: return get_grid_states_kernel_r3(star, rb);
+        default: return {nullptr, 0};
+    }
+}
+
 static GridKernelRef grid_kernel(int R, int star, int rb) {
     switch (R) {
         case 1: return get_grid_kernel_r1(star, rb);
@@ -85,9 +98,15 @@ size_t grid_scratch_bytes(int ny, int nx) {
 
 cudaError_t launch_grid(const GridConfig& c, int R, int star, int dtype, int periodic, const void* in, void* out,
                         int ny, int nx, int vec, int T, int k, void* scratch, unsigned* status, long long wait_ns,
-                        int withhold, const Weights& w, cudaStream_t st) {
-    const GridKernelRef ref = grid_kernel(R, star, c.rb);
+                        int withhold, const Weights& w, cudaStream_t st, float* states,
+                        long long state_stride, int state_first) {
+    const GridKernelRef ref = states ? grid_states_kernel(R, star, c.rb) : grid_kernel(R, star, c.rb);
     if (!ref.fn) return cudaErrorInvalidValue;
+    if (states) {  // (plain kernels: set when the plan is made, by grid_fits)
+        const cudaError_t e =
+            cudaFuncSetAttribute(ref.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kGridMaxSmem);
+        if (e != cudaSuccess) return e;
+    }
     GridParams p{};
     p.in = in;
     p.out = out;
@@ -102,6 +121,9 @@ cudaError_t launch_grid(const GridConfig& c, int R, int star, int dtype, int per
     p.status = status;
     p.wait_ns = wait_ns;
     p.withhold = withhold;
+    p.states = states;
+    p.state_stride = state_stride;
+    p.state_first = state_first;
     p.T = T;
     p.k = k;
     p.Hy = c.Hy;

@@ -29,8 +29,10 @@ bool grid_fits(const GridConfig& c, int R, int star, int sms);
 size_t grid_scratch_bytes(int ny, int nx);
 
 // T steps, in one cooperative launch.  k <= c.k: steps per exchange of this launch.
+// states (FP32 runs): the results of steps state_first .. T-1 as well, state_stride floats apart.
 cudaError_t launch_grid(const GridConfig& c, int R, int star, int dtype, int periodic, const void* in, void* out,
                         int ny, int nx, int vec, int T, int k, void* scratch, unsigned* status, long long wait_ns,
-                        int withhold, const Weights& w, cudaStream_t st);
+                        int withhold, const Weights& w, cudaStream_t st, float* states = nullptr,
+                        long long state_stride = 0, int state_first = 1);
 
 }  // namespace gbst

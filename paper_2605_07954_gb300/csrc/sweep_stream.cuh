@@ -701,7 +701,7 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                     }
                     if constexpr (ALL) {
                         const int yo = ybeg - (l + 1) * R + s;
-                        if (l < K - 1 && store_chunk && yo >= y0 && yo < ylast)
+                        if (l < K - 1 && p.lvl_out[l] && store_chunk && yo >= y0 && yo < ylast)
                             Storage<TS>::store4(static_cast<TS*>(p.lvl_out[l]) + (size_t)yo * ldo + c0,
                                                 make_float4(Pa.x, Pb.x, Pa.y, Pb.y));
                     }
@@ -823,7 +823,7 @@ __device__ __forceinline__ void stream_tile(const StreamParams& p, const WS& ws,
                 }
                 if constexpr (ALL) {
                     const int yo = ybeg + s - l * (R + 1) - R;
-                    if (l < K - 1 && store_chunk && yo >= y0 && yo < ylast) {
+                    if (l < K - 1 && p.lvl_out[l] && store_chunk && yo >= y0 && yo < ylast) {
                         const float2 A0 = acc[l][cdone][0], A1 = acc[l][cdone][1];
                         Storage<TS>::store4(static_cast<TS*>(p.lvl_out[l]) + (size_t)yo * ldo + c0,
                                             make_float4(A0.x, A0.y, A1.x, A1.y));
@@ -887,9 +887,9 @@ __host__ __device__ constexpr int stream_min_blocks(int R, bool STAR, int K) {
          : 0;
 }
 
-// ALL: every time level of the launch is stored (level l+1 to p.lvl_out[l],
-// the last to p.out), for callers that need each state (the adjoint's
-// recomputation of a segment); VEC kernels only.
+// ALL: time levels of the launch are stored (level l+1 to p.lvl_out[l] where that
+// is not null, the last to p.out), for callers that need each state (the adjoint's
+// recomputation of a segment) or the last two (residuals); VEC kernels only.
 // PAD: rows of a padded pitch whose last chunk the grid's right edge may cut, and
 // a last launch that stores dense rows element by element; VEC kernels only, a
 // variant of its own because the extra code in the aligned kernels cost them

@@ -102,8 +102,9 @@ __host__ __device__ constexpr int warp_ring_bytes() { return kWarpRing * 32 * NC
 __host__ __device__ constexpr int warp_rows_after(int K) { return K + 3; }
 
 // One tile: outputs [y0, y0 + by) x [x0, x0 + bx).  EDGE: the tile loads rows or
-// columns outside the grid; CUT: the right edge may cut a chunk.  p.bx and p.H are multiples of NC.
-template <bool STAR, int K, typename TS, int NC, bool EDGE, bool CUT = EDGE>
+// columns outside the grid; CUT: the right edge may cut a chunk; ALL: level l+1
+// is also stored to p.lvl_out[l] where that is not null (l < K-1).  p.bx and p.H are multiples of NC.
+template <bool STAR, int K, typename TS, int NC, bool EDGE, bool CUT = EDGE, bool ALL = false>
 __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeights<STAR>& ws, char* ring, int lane,
                                           int x0, int y0) {
     constexpr int NP = NC / 2, PF = kWarpRing, NQ = NC / 4;
@@ -168,6 +169,15 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
         st[j] = cj >= x0 && cj < x0 + p.bx && cj < nx;
     }
     TS* out = static_cast<TS*>(p.out) + c;
+    auto store_row = [&](TS* o, const float2 (&X)[NP]) {
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            float e[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] = 4 * j + i < NP ? X[(4 * j + i) % NP].x : X[(4 * j + i) % NP].y;
+            if (st[j]) Storage<TS>::store4(o + 4 * j, make_float4(e[0], e[1], e[2], e[3]));
+        }
+    };
 
     auto group = [&](int s0, auto mr) {
         [[maybe_unused]] constexpr bool MR = decltype(mr)::value;
@@ -215,18 +225,14 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
                         }
                     }
                 }
-            }
-            const int yo = ybeg - K + s;
-            if (yo >= y0 && yo < ylast) {
-                TS* o = out + (long long)yo * ld;
-#pragma unroll
-                for (int j = 0; j < NQ; ++j) {
-                    float e[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) e[i] = 4 * j + i < NP ? X[(4 * j + i) % NP].x : X[(4 * j + i) % NP].y;
-                    if (st[j]) Storage<TS>::store4(o + 4 * j, make_float4(e[0], e[1], e[2], e[3]));
+                if constexpr (ALL) {
+                    const int yl = ybeg - (l + 1) + s;
+                    if (l < K - 1 && p.lvl_out[l] && yl >= y0 && yl < ylast)
+                        store_row(static_cast<TS*>(p.lvl_out[l]) + c + (long long)yl * ld, X);
                 }
             }
+            const int yo = ybeg - K + s;
+            if (yo >= y0 && yo < ylast) store_row(out + (long long)yo * ld, X);
         });
     };
     for (int s0 = 0; s0 < nsteps; s0 += 3) {
@@ -246,7 +252,8 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
 __host__ __device__ constexpr int warp_min_blocks(int NC) { return NC == 8 ? 8 : 16; }
 
 // A launch of one-warp CTAs over a whole grid: p.strips x tile rows, edge tiles first.
-template <bool STAR, int K, typename TS, int NC>
+// (ALL kernels take widths that are a multiple of NC.)
+template <bool STAR, int K, typename TS, int NC, bool ALL = false>
 __global__ void __launch_bounds__(32, warp_min_blocks(NC)) sweep_warp_kernel(const __grid_constant__ StreamParams p) {
     __shared__ __align__(16) char ring[warp_ring_bytes<TS, NC>()];
     const int lane = threadIdx.x;
@@ -257,9 +264,9 @@ __global__ void __launch_bounds__(32, warp_min_blocks(NC)) sweep_warp_kernel(con
     const int ylast = min(y0 + p.by, ny);
     const bool interior = y0 - K >= 0 && ylast + warp_rows_after(K) <= ny && x0 - p.H >= 0 && x0 - p.H + 32 * NC <= nx;
     const WarpWeights<STAR> ws([&](int i) { return p.w.w[i]; });
-    if (interior) warp_tile<STAR, K, TS, NC, false>(p, ws, ring, lane, x0, y0);
-    else if (nx % NC == 0) warp_tile<STAR, K, TS, NC, true, false>(p, ws, ring, lane, x0, y0);
-    else warp_tile<STAR, K, TS, NC, true>(p, ws, ring, lane, x0, y0);
+    if (interior) warp_tile<STAR, K, TS, NC, false, false, ALL>(p, ws, ring, lane, x0, y0);
+    else if (ALL || nx % NC == 0) warp_tile<STAR, K, TS, NC, true, false, ALL>(p, ws, ring, lane, x0, y0);
+    else warp_tile<STAR, K, TS, NC, true, true, ALL>(p, ws, ring, lane, x0, y0);
 }
 
 }  // namespace gbst
