@@ -58,3 +58,41 @@ def test_fullsize_residuals_nonincreasing():
     assert len(r) == 10 and np.all(r > 0)
     assert np.all(r[1:] <= r[:-1] * (1 + 1e-6))
     p.close()
+
+
+@pytest.mark.parametrize("name,shape,boundary", [("box9", (1700, 1600), "zero"), ("heat5", (1604, 1800), "periodic"),
+                                                 ("star13", (1600, 1504), "zero"), ("box49", (1600, 1504), "periodic"),
+                                                 ("box9", (300, 333), "zero"), ("star13", (300, 332), "periodic")])
+@pytest.mark.parametrize("m", [1, 2, 3, 6, 8, 9, 13])
+def test_last_two_steps_of_every_interval(name, shape, boundary, m):
+    """Intervals whose last launch stores two steps (streaming and chip-resident
+    plans), single steps and remainders: the final state has the bits of a plain
+    run, and every residual is that of the states two runs give."""
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights(name)
+    x = torch.from_numpy(inputs.field(*shape)).cuda()
+    p = Plan(shape[0], shape[1], W, boundary=boundary)
+    T = 3 * m + 1
+    for _ in range(2):
+        y, res = p.run_residual(x, T, m)
+        p.status()
+        assert torch.equal(y, p.run(x, T))
+        want = [torch.linalg.vector_norm(p.run(x, t).double() - p.run(x, t - 1).double()) for t in range(m, T + 1, m)]
+        # FP64 sums of exact differences: rounding at 45 bits and better
+        assert torch.allclose(res, torch.stack(want), rtol=1e-11, atol=0)
+    p.close()
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e25, float("inf")])
+def test_residual_outside_the_fp32_range(scale):
+    """Differences whose squares leave the FP32 range, and infinities."""
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights("box9")
+    x = torch.from_numpy(inputs.field(60, 68)).cuda() * (scale if scale < 1e30 else 1.0)
+    if scale == float("inf"):
+        x[3, 5] = scale
+    p = Plan(60, 68, W)
+    _, res = p.run_residual(x, 4, 2)
+    want = [torch.linalg.vector_norm(p.run(x, t).double() - p.run(x, t - 1).double()) for t in (2, 4)]
+    assert torch.allclose(res, torch.stack(want), rtol=1e-11, atol=0, equal_nan=True)
+    p.close()
