@@ -894,7 +894,7 @@ static std::vector<int> launch_depths(const stencil_plan* p, int64_t T) {
 // One all-states launch of d steps: level l+1 to outs[l] (null: not stored, but the last must be).
 static stencil_status_t launch_states(stencil_plan_t* p, const void* src, float* const* outs, int d, cudaStream_t st) {
     if (d == kWarpDepth && p->R == 1) {
-        // one-warp tiles where they have enough rows (4096^2 5-point star: 96 us
+        // one-warp tiles where they have enough rows (4096^2 5-point star: 123 us
         // per launch, 153 CTA-wide)
         const WarpTiles t = warp_tiles(p, 4);
         if (t.by >= kWarpMinRows) {
