@@ -275,7 +275,8 @@ const char* stencil_residual_last_error(void);
  *                  synchronises `stream` before it returns).  Every entry of the
  *                  square is returned, off-footprint ones included.
  *   ckpt_interval  steps between checkpoints; 0 = choose: T (no checkpoints) while
- *                  T + 3 grids take at most 1 GiB, else about sqrt(T).  The result
+ *                  T + 3 grids take at most 1 GiB, else about sqrt(T) (always sqrt(T)
+ *                  for grids small enough for the cluster-resident kernel).  The result
  *                  does not depend on it (same bits).
  * States are recomputed from checkpoints, not stored: the plan allocates and
  * keeps (ceil(T/s) + s + 2) grids of scratch, s = ckpt_interval.  The weight
@@ -285,6 +286,16 @@ const char* stencil_residual_last_error(void);
 stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const void* grad_uT, int64_t T,
                                  void* grad_u0, double* grad_w, int64_t ckpt_interval,
                                  stencil_stream_t stream);
+
+/*
+ * stencil_adjoint for callers that round the weight gradient to FP32 or less (a
+ * training step with FP32 weights): same arguments and the same grad_u0, but the
+ * FP32 products of grad_w may be grouped as suits the faster kernels (its relative
+ * error stays at about 1e-7; repeated calls still give the same bits).
+ */
+stencil_status_t stencil_adjoint_w32(stencil_plan_t* plan, const void* u0, const void* grad_uT, int64_t T,
+                                     void* grad_u0, double* grad_w, int64_t ckpt_interval,
+                                     stencil_stream_t stream);
 
 /* Kernel launches stencil_adjoint makes for T and ckpt_interval (grad_w != NULL). */
 int64_t stencil_adjoint_launches(const stencil_plan_t* plan, int64_t T, int64_t ckpt_interval);

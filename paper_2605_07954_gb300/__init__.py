@@ -153,15 +153,19 @@ def adjoint(plan: Plan, u0, grad_uT, T: int, ckpt_interval: int = 0):
     Returns a CUDA tensor like u0 and a (2r+1, 2r+1) float64 CUDA tensor.
     Enqueued on torch's current stream.
     """
+    return _adjoint(plan, u0, grad_uT, T, ckpt_interval, "stencil_adjoint")
+
+
+def _adjoint(plan, u0, grad_uT, T, ckpt_interval, entry):
     import torch
     plan._check_tensor(u0)
     plan._check_tensor(grad_uT)
     g_u0 = torch.empty_like(u0)
     d = 2 * plan.radius + 1
     g_w = torch.empty((d, d), dtype=torch.float64, device=u0.device)
-    check(_capi.load().stencil_adjoint(plan.handle, u0.data_ptr(), grad_uT.data_ptr(), int(T),
+    check(getattr(_capi.load(), entry)(plan.handle, u0.data_ptr(), grad_uT.data_ptr(), int(T),
                                        g_u0.data_ptr(), g_w.data_ptr(), int(ckpt_interval),
-                                       _current_stream_handle()), "stencil_adjoint")
+                                       _current_stream_handle()), entry)
     return g_u0, g_w
 
 
@@ -224,7 +228,8 @@ def _stencil_fn():
             (u0,) = ctx.saved_tensors
             # another forward call may have changed the cached plan's weights
             ctx.plan.set_weights(ctx.W)
-            g_u0, g_w = adjoint(ctx.plan, u0, grad_y.contiguous(), ctx.T, ctx.ckpt)
+            entry = "stencil_adjoint" if ctx.wdtype == torch.float64 else "stencil_adjoint_w32"
+            g_u0, g_w = _adjoint(ctx.plan, u0, grad_y.contiguous(), ctx.T, ctx.ckpt, entry)
             return g_u0, g_w.to(ctx.wdevice, ctx.wdtype), None, None, None
 
     return StencilFn

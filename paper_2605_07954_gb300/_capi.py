@@ -92,6 +92,7 @@ _PROTOS = {
     "stencil_run_residual": (_i32, [_vp, _vp, _vp, _i64, _i64, _vp, _vp]),
     "stencil_residual_last_error": (ctypes.c_char_p, []),
     "stencil_adjoint": (_i32, [_vp, _vp, _vp, _i64, _vp, _vp, _i64, _vp]),
+    "stencil_adjoint_w32": (_i32, [_vp, _vp, _vp, _i64, _vp, _vp, _i64, _vp]),
     "stencil_adjoint_launches": (_i64, [_vp, _i64, _i64]),
     "stencil_adjoint_last_error": (ctypes.c_char_p, []),
     "stencil_batch_create": (_i32, [ctypes.POINTER(_vp), _i32, ctypes.POINTER(stencil_grid_desc_t),

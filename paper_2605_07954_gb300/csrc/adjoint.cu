@@ -21,8 +21,14 @@
 // to its CTA's FP64 partial.  Tile t of a launch is always CTA t and launches
 // are ordered, so each partial sums its steps in a fixed order; a last kernel
 // sums the partials over tiles in a fixed order.  The gradient is deterministic.
-// adjoint_stream_kernel is that step for radius 1 and widths a multiple of 4,
-// adjoint_rows_kernel for everything else.
+// adjoint_stream_kernel is that step for radius 1 and widths a multiple of 4;
+// for everything else adjoint_step_kernel, or, where the caller rounds the weight
+// gradient to FP32 (stencil_adjoint_w32) and the radius is 2 or 3, the faster
+// adjoint_rows_kernel.
+//
+// The FP64 weight gradient of stencil_adjoint is tied to the bits of the states, so
+// where those depend on how steps are grouped they come from the streaming kernel
+// (plan_keep_sums) and a fixed checkpoint interval.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,11 +46,12 @@ namespace gbst {
 void plan_weights(const stencil_plan_t* p, float* w);
 void** plan_aux_slot(stencil_plan_t* p, int id);
 void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*));
-stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n,
+bool plan_keep_sums(stencil_plan_t* p, bool on);
+bool plan_states_vary(const stencil_plan_t* p);
+stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
                                  cudaStream_t st);
 
-// One reverse step for any radius and width (radius 1 with widths a multiple of 4
-// has adjoint_stream_kernel below).  A warp owns 120 columns (lanes 1..30, 4 each;
+// One reverse step of radius 2 or 3, any width, for weight gradients kept in FP32.  A warp owns 120 columns (lanes 1..30, 4 each;
 // lanes 0 and 31 hold halo columns) of kAdrRows output rows and walks down the
 // rows of lambda_{t+1} with the last 2R+1 of them in registers, each extended by
 // R columns per side (shuffles).  Per output row o of the walk:
@@ -198,6 +205,147 @@ __global__ void __launch_bounds__(kAdrWarps * 32, 2)
     }
     __syncthreads();
     if (threadIdx.x < D * D) partials[(size_t)blockIdx.x * D * D + threadIdx.x] += half[threadIdx.x];
+}
+
+constexpr int kAdjTX = 32;          // output tile columns (one per lane)
+constexpr int kAdjTY = 64;          // output tile rows
+constexpr int kAdjRowsPerThread = 8;  // 8 warps x 8 rows
+
+// The reverse step behind the FP64 weight gradient where adjoint_stream_kernel does
+// not apply, on a 32 x 64 tile.  Its FP32 sums run over 8 rows x 32 columns before
+// they go to FP64; a kernel that groups the products otherwise moves the FP64
+// result by ~1e-8..1e-7, which callers who keep 64 bits would see (accumulators
+// that reproduce these sums would need 4 x (2R+1)^2 registers in
+// adjoint_rows_kernel).  Step and state in us, FP32, GB300, this | adjoint_rows_kernel:
+// 13-point star 1000 x 1022 29.8 | 17.5, 4000 x 3004 280 | 135; radius 1 at
+// 1000 x 1022 10.7 | 12.6, so radius 1 keeps this kernel for FP32 gradients too.  Lane tx owns column x0 + tx and warp ty
+// rows y0 + 8 ty .. + 7; it walks its rows keeping the last 2R+1 staged rows
+// of lambda_{t+1} and u_t (its column +- R) in registers, so each row costs
+// 2 (2R+1) shared-memory loads for (2R+1)^2 lambda FMAs and (2R+1)^2 gradient FMAs.
+template <int R>
+__global__ void __launch_bounds__(256)
+    adjoint_step_kernel(const float* __restrict__ lam_in, const float* __restrict__ u,
+                        float* __restrict__ lam_out, double* __restrict__ partials, int ny, int nx,
+                        int periodic, Weights w, int tiles_x, int /*vec*/) {
+    constexpr int D = 2 * R + 1;
+    constexpr int SY = kAdjTY + 2 * R, SX = kAdjTX + 2 * R;
+    __shared__ float sl[SY][SX + 1];
+    __shared__ float su[SY][SX + 1];
+    __shared__ float red[8][D * D];
+    const int tx = threadIdx.x, ty = threadIdx.y;  // (32, 8)
+    const int x0 = (blockIdx.x % tiles_x) * kAdjTX;
+    const int y0 = (blockIdx.x / tiles_x) * kAdjTY;
+
+    // Stage both tiles with their halo (zero outside, or wrapped).  Every
+    // thread issues all of its loads before its first shared-memory store, so
+    // the DRAM latencies overlap.  Item i = tid + 256 it is staged row i / SX,
+    // column i % SX, advanced without division.
+    {
+        constexpr int ITEMS = SY * SX, ITERS = (ITEMS + 255) / 256;
+        const int tid0 = ty * 32 + tx;
+        int r = tid0 / SX, c = tid0 % SX;
+        float va[ITERS], vb[ITERS];
+        int ra[ITERS], ca[ITERS];
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            ra[it] = r;
+            ca[it] = c;
+            va[it] = vb[it] = 0.f;
+            if (r < SY) {
+                int y = y0 - R + r, x = x0 - R + c;
+                bool ok = y >= 0 && y < ny && x >= 0 && x < nx;
+                if (periodic) {
+                    y = (y % ny + ny) % ny;
+                    x = (x % nx + nx) % nx;
+                    ok = true;
+                }
+                if (ok) {
+                    const size_t i = (size_t)y * nx + x;
+                    va[it] = __ldg(lam_in + i);
+                    vb[it] = __ldg(u + i);
+                }
+            }
+            c += 256 % SX;
+            r += 256 / SX;
+            if (c >= SX) {
+                c -= SX;
+                ++r;
+            }
+        }
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            if (ra[it] < SY) {
+                sl[ra[it]][ca[it]] = va[it];
+                su[ra[it]][ca[it]] = vb[it];
+            }
+        }
+    }
+    __syncthreads();
+
+    float g[D * D];
+#pragma unroll
+    for (int k = 0; k < D * D; ++k) g[k] = 0.f;
+    // Register windows: wl[i][e] = lambda staged row (row0 + i), column tx + e;
+    // wu likewise for u.  The output row o = r0 + k needs lambda rows o-R..o+R
+    // (flipped correlation) and u rows o-R..o+R.
+    const int r0 = ty * kAdjRowsPerThread;  // first output row (tile-local)
+    float wl[D][D], wu[D][D];
+#pragma unroll
+    for (int i = 0; i < D - 1; ++i)
+#pragma unroll
+        for (int e = 0; e < D; ++e) {
+            wl[i + 1][e] = sl[r0 + i][tx + e];
+            wu[i + 1][e] = su[r0 + i][tx + e];
+        }
+#pragma unroll
+    for (int k = 0; k < kAdjRowsPerThread; ++k) {
+        // slide: drop the oldest staged row, append staged row r0 + k + 2R
+#pragma unroll
+        for (int i = 0; i < D - 1; ++i)
+#pragma unroll
+            for (int e = 0; e < D; ++e) {
+                wl[i][e] = wl[i + 1][e];
+                wu[i][e] = wu[i + 1][e];
+            }
+#pragma unroll
+        for (int e = 0; e < D; ++e) {
+            wl[D - 1][e] = sl[r0 + k + 2 * R][tx + e];
+            wu[D - 1][e] = su[r0 + k + 2 * R][tx + e];
+        }
+        // window row i holds staged row r0 + k + i, i.e. grid row o - R + i for o = y0 + r0 + k
+        const int y = y0 + r0 + k, x = x0 + tx;
+        if (y >= ny || x >= nx) continue;
+        // lambda_t[o] = sum_d W[d] lambda_{t+1}[o - d], dy-major then dx
+        float acc = 0.f;
+#pragma unroll
+        for (int dy = -R; dy <= R; ++dy)
+#pragma unroll
+            for (int dx = -R; dx <= R; ++dx)
+                acc = fmaf(w.w[(dy + R) * D + (dx + R)], wl[R - dy][R - dx], acc);
+        lam_out[(size_t)y * nx + x] = acc;
+        // dL/dW[d] += lambda_{t+1}[o] * u_t[o + d]
+        const float lp = wl[R][R];
+#pragma unroll
+        for (int dy = -R; dy <= R; ++dy)
+#pragma unroll
+            for (int dx = -R; dx <= R; ++dx)
+                g[(dy + R) * D + (dx + R)] = fmaf(lp, wu[R + dy][R + dx], g[(dy + R) * D + (dx + R)]);
+    }
+    // Fixed-order reduction: butterfly within each warp, then warps in order.
+#pragma unroll
+    for (int k = 0; k < D * D; ++k) {
+        float v = g[k];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (tx == 0) red[ty][k] = v;
+    }
+    __syncthreads();
+    const int tid = ty * 32 + tx;
+    if (tid < D * D) {
+        double s = 0.0;
+        for (int wv = 0; wv < 8; ++wv) s += (double)red[wv][tid];
+        partials[(size_t)blockIdx.x * D * D + tid] += s;
+    }
 }
 
 // grad_w[k] = sum over tiles of partials[tile][k] in a fixed order: thread i of
@@ -534,9 +682,17 @@ static const void* adjoint_stream_kernel_fn(int R) {
     return R == 1 ? (const void*)adjoint_stream_kernel<1> : nullptr;
 }
 
+static const void* adjoint_step_kernel_fn(int R) {
+    switch (R) {
+        case 1: return (const void*)adjoint_step_kernel<1>;
+        case 2: return (const void*)adjoint_step_kernel<2>;
+        case 3: return (const void*)adjoint_step_kernel<3>;
+        default: return nullptr;
+    }
+}
+
 static const void* adjoint_rows_kernel_fn(int R, bool star) {
     switch (R) {
-        case 1: return star ? (const void*)adjoint_rows_kernel<1, true> : (const void*)adjoint_rows_kernel<1, false>;
         case 2: return star ? (const void*)adjoint_rows_kernel<2, true> : (const void*)adjoint_rows_kernel<2, false>;
         case 3: return star ? (const void*)adjoint_rows_kernel<3, true> : (const void*)adjoint_rows_kernel<3, false>;
         default: return nullptr;
@@ -584,8 +740,10 @@ int64_t adj_sqrt(int64_t T) { return (int64_t)std::ceil(std::sqrt((double)T)); }
 // states take at most 1 GiB: no checkpoint pass is needed then.  Otherwise
 // ceil(sqrt(T)), for radius 1 rounded up to whole launches of 8 steps (Heat 4096^2
 // x 128: 12 steps a segment 3.16 ms of forward launches, 16 steps 2.82 ms).
-int64_t adj_interval(int64_t T, int64_t asked, int R, size_t bytes) {
+// vary: states whose bits depend on the checkpoints (FP64 sums resolve them): sqrt(T) always.
+int64_t adj_interval(int64_t T, int64_t asked, int R, size_t bytes, bool vary) {
     if (asked > 0) return std::min<int64_t>(asked, T);
+    if (vary) return adj_sqrt(T);
     if ((double)(T + 3) * (double)bytes <= (double)(1ull << 30)) return T;
     const int64_t s = adj_sqrt(T);
     return std::min<int64_t>(R == 1 ? (s + 7) / 8 * 8 : s, T);
@@ -637,13 +795,23 @@ stencil_status_t adj_scratch(stencil_plan_t* plan, size_t grids, size_t grid_byt
 
 }  // namespace
 
-extern "C" {
+namespace {
 
-const char* stencil_adjoint_last_error(void) { return g_adj_error.c_str(); }
+// The plan in the form whose states' bits the FP64 sums are tied to, for one call.
+struct KeepSums {
+    stencil_plan_t* p;
+    const bool on;
+    KeepSums(stencil_plan_t* plan, bool wanted) : p(plan), on(wanted && plan_keep_sums(plan, true)) {}
+    ~KeepSums() {
+        if (on) plan_keep_sums(p, false);
+    }
+    KeepSums(const KeepSums&) = delete;
+    KeepSums& operator=(const KeepSums&) = delete;
+};
 
-stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const void* grad_uT, int64_t T,
-                                 void* grad_u0, double* grad_w, int64_t ckpt_interval,
-                                 stencil_stream_t stream) {
+// w32: the caller rounds grad_w to FP32, so its sums may be grouped freely.
+stencil_status_t adjoint_run(stencil_plan_t* plan, const void* u0, const void* grad_uT, int64_t T, void* grad_u0,
+                             double* grad_w, int64_t ckpt_interval, stencil_stream_t stream, bool w32) {
     if (!plan || !u0 || !grad_uT || !grad_u0) return afail(STENCIL_ERR_INVALID_ARG, "NULL argument");
     if (T < 0 || ckpt_interval < 0) return afail(STENCIL_ERR_INVALID_ARG, "T and ckpt_interval must be >= 0");
     stencil_plan_info_t info{};
@@ -664,15 +832,18 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
     // nx % 4 == 0, and the buffers below are then 16-byte aligned), else the
     // any-width one.
     const bool streamed = adjoint_stream_kernel_fn(R) != nullptr && nx % 4 == 0;
-    const int tiles_x = streamed ? (nx + kAdsCols - 1) / kAdsCols : (nx + kAdrCols - 1) / kAdrCols;
-    const int tile_rows = streamed ? kAdsWarps * kAdsRows : kAdrWarps * kAdrRows;
+    const bool rows = w32 && R > 1;
+    const int tile_cols = streamed ? kAdsCols : rows ? kAdrCols : kAdjTX;
+    const int tiles_x = (nx + tile_cols - 1) / tile_cols;
+    const int tile_rows = streamed ? kAdsWarps * kAdsRows : rows ? kAdrWarps * kAdrRows : kAdjTY;
     const int tiles = tiles_x * ((ny + tile_rows - 1) / tile_rows);
     if (T == 0) {
         if (grad_u0 != grad_uT) ACK(cudaMemcpyAsync(grad_u0, grad_uT, bytes, cudaMemcpyDeviceToDevice, st));
         if (grad_w) ACK(cudaMemsetAsync(grad_w, 0, sizeof(double) * D * D, st));
         return STENCIL_OK;
     }
-    int64_t sgm = adj_interval(T, ckpt_interval, R, bytes);
+    const KeepSums kept(plan, !w32);
+    int64_t sgm = adj_interval(T, ckpt_interval, R, bytes, !w32 && plan_states_vary(plan));
     int64_t nseg = (T + sgm - 1) / sgm;
     // Buffers: nseg checkpoints, sgm segment states, two adjoint grids.
     AdjScratch* sc = nullptr;
@@ -698,9 +869,11 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
     ACK(cudaMemcpyAsync(lam[0], grad_uT, bytes, cudaMemcpyDeviceToDevice, st));
     int cur = 0;
     // (a star's off-axis weights are zero: the lambda update skips them)
-    const void* kfn = streamed ? adjoint_stream_kernel_fn(R) : adjoint_rows_kernel_fn(R, adj_star(wf, R));
+    const void* kfn = streamed ? adjoint_stream_kernel_fn(R)
+                      : rows   ? adjoint_rows_kernel_fn(R, adj_star(wf, R))
+                               : adjoint_step_kernel_fn(R);
     if (!kfn) return afail(STENCIL_ERR_UNSUPPORTED, "no adjoint kernel for this radius");
-    const dim3 block = dim3(streamed ? kAdsWarps * 32 : kAdrWarps * 32);
+    const dim3 block = streamed ? dim3(kAdsWarps * 32) : rows ? dim3(kAdrWarps * 32) : dim3(32, 8);
     int vec = nx % 4 == 0;
     int periodic = info.boundary == STENCIL_BOUNDARY_PERIODIC;
     std::vector<float*> segp((size_t)sgm);
@@ -712,7 +885,7 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
         const float* state0 = ckpt + (size_t)j * n;
         if (len > 1) {
             for (int64_t t = 1; t < len; ++t) segp[t - 1] = seg + (size_t)t * n;
-            s = plan_run_states(plan, state0, segp.data(), len - 1, st);
+            s = plan_run_states(plan, state0, segp.data(), len - 1, w32, st);
             if (s != STENCIL_OK) return afail(s, std::string("segment recompute: ") + stencil_last_error());
         }
         for (int64_t t = len - 1; t >= 0; --t) {
@@ -745,16 +918,35 @@ stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const voi
     return STENCIL_OK;
 }
 
+}  // namespace
+
+extern "C" {
+
+const char* stencil_adjoint_last_error(void) { return g_adj_error.c_str(); }
+
+stencil_status_t stencil_adjoint(stencil_plan_t* plan, const void* u0, const void* grad_uT, int64_t T,
+                                 void* grad_u0, double* grad_w, int64_t ckpt_interval,
+                                 stencil_stream_t stream) {
+    return adjoint_run(plan, u0, grad_uT, T, grad_u0, grad_w, ckpt_interval, stream, false);
+}
+
+stencil_status_t stencil_adjoint_w32(stencil_plan_t* plan, const void* u0, const void* grad_uT, int64_t T,
+                                     void* grad_u0, double* grad_w, int64_t ckpt_interval,
+                                     stencil_stream_t stream) {
+    return adjoint_run(plan, u0, grad_uT, T, grad_u0, grad_w, ckpt_interval, stream, true);
+}
+
 int64_t stencil_adjoint_launches(const stencil_plan_t* plan, int64_t T, int64_t ckpt_interval) {
     if (!plan || T < 0 || ckpt_interval < 0) return -1;
     if (T == 0) return 0;
+    const KeepSums kept(const_cast<stencil_plan_t*>(plan), true);
     stencil_plan_info_t info{};
     const bool fused = stencil_plan_info(plan, &info) == STENCIL_OK && info.dtype == STENCIL_F32 &&
                        info.nx % 4 == 0;
-    const int64_t sgm = adj_interval(T, ckpt_interval, info.radius, (size_t)info.ny * (size_t)info.nx * sizeof(float));
+    const int64_t sgm = adj_interval(T, ckpt_interval, info.radius, (size_t)info.ny * (size_t)info.nx * sizeof(float), plan_states_vary(plan));
     const int64_t nseg = (T + sgm - 1) / sgm;
     int64_t L = (nseg - 1) * stencil_run_launches(plan, sgm);  // checkpoints
-    const bool resident = info.kernel == STENCIL_KERNEL_RESIDENT && info.ctas == 1 && info.threads != 1024 &&
+    const bool resident = info.kernel == STENCIL_KERNEL_RESIDENT && !plan_states_vary(plan) && info.ctas == 1 && info.threads != 1024 &&
                           !(info.boundary == STENCIL_BOUNDARY_PERIODIC && info.nx % 4 != 0);
     for (int64_t j = 0; j < nseg; ++j) {  // segment recompute: all-states launches of 8/4/2/1 steps
         int64_t m = std::min<int64_t>(sgm, T - j * sgm) - 1;

@@ -130,6 +130,10 @@ struct stencil_plan {
     // chip-resident register tiles (sweep_grid.cuh): usable, in use (kernel == RESIDENT then), scratch
     int grid_ok = 0, grid_on = 0;
     GridConfig grid;
+    // streaming plans: launches of up to tiles.k steps as register tiles: usable, in use
+    int tiles_ok = 0, tiles_on = 0;
+    int kept_kernel = 0, kept_grid = 0, kept_tiles = 0;  // what plan_keep_sums puts back
+    GridConfig tiles;
     void* grid_mem = nullptr;
     // streaming runs of a width that is not a multiple of 4 (zero rule): two grids of padded rows
     int64_t pad_ld = 0;
@@ -156,8 +160,11 @@ void plan_weights(const stencil_plan_t* p, float* w) {
 }
 void** plan_aux_slot(stencil_plan_t* p, int id) { return &p->aux[id]; }
 void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*)) { p->aux_free[id] = freer; }
-stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n,
-                                 cudaStream_t st);
+// Whether the bits of a run's states depend on how its steps are grouped into calls.
+bool plan_states_vary(const stencil_plan_t* p) {
+    return (p->kernel == STENCIL_KERNEL_RESIDENT && (!p->grid_on || p->grid.plain)) ||
+           (p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0);
+}
 }  // namespace gbst
 
 static size_t elem_size(int dtype) { return dtype == STENCIL_F32 ? 4 : 2; }
@@ -384,6 +391,7 @@ static stencil_status_t configure_stream(stencil_plan* p, int k, int threads, in
     if (strips * tiles_y > 0x7fffffffLL) return fail(STENCIL_ERR_UNSUPPORTED, "grid too large");
     p->kernel = STENCIL_KERNEL_STREAM;
     p->grid_on = 0;
+    p->tiles_on = 0;
     p->k = k;
     p->threads = nt;
     p->H = H;
@@ -582,8 +590,17 @@ static bool grid_candidate(stencil_plan* p) {
     }
     const int periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
     if (!grid_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, 0, 0, &p->grid)) return false;
+    p->grid.plain = resident_candidates(p) > 0;
     p->grid_ok = grid_fits(p->grid, p->R, p->star, p->sms);
     return p->grid_ok != 0;
+}
+
+// Whether a launch of nlev steps runs as register tiles.  Aligned launches of a
+// step or two (a run's remainder) are cheaper without the tiles' deep halo:
+// 2048^2, 1 step, 5-point star 15 us as tiles, 12 streaming, 13-point star 19 |
+// 15, 7x7 box 27 | 25; 2 steps 17 | 13, 23 | 17, but 42 | 48.
+static bool tiles_launch(const stencil_plan* p, int nlev, bool vec) {
+    return p->tiles_on && !(vec && nlev <= (p->star ? 2 : 1));
 }
 
 static void use_grid(stencil_plan* p) {
@@ -757,6 +774,11 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
     const size_t vec_bytes = 4 * p->elem;
     sp.vec = (p->nx % 4 == 0) && ((uintptr_t)src % vec_bytes == 0) &&
              ((uintptr_t)dst % vec_bytes == 0);
+    if (tiles_launch(p, nlev, sp.vec)) {
+        CK(launch_tiles(p->tiles, p->R, p->star, p->dtype, sp.periodic, src, dst, (int)p->ny, (int)p->nx, sp.vec, nlev,
+                        p->w, st));
+        return STENCIL_OK;
+    }
     if (p->warp_nc && nlev == kWarpDepth && sp.vec) return launch_warp(p, sp, st);
     dim3 grid((unsigned)(p->strips * p->tiles_y)), block((unsigned)p->threads);
     const void* fn = nullptr;
@@ -871,11 +893,13 @@ static std::vector<int> launch_depths(const stencil_plan* p, int64_t T) {
         for (int64_t t = 0; t < T; t += (1 << 30)) d.push_back((int)std::min<int64_t>(T - t, 1 << 30));
         return d;
     }
-    const int k = p->kernel == STENCIL_KERNEL_STREAM ? p->k : 1;
+    const int k = p->kernel != STENCIL_KERNEL_STREAM ? 1 : p->tiles_on ? p->tiles.k : p->k;
     for (int64_t t = 0; t < T / k; ++t) d.push_back(k);
     int rem = (int)(T % k);
     while (rem > 0) {
-        const int step = p->kernel == STENCIL_KERNEL_STREAM ? stream_depth_at_most(p->R, p->star, rem) : 1;
+        const int step = p->kernel != STENCIL_KERNEL_STREAM ? 1
+                         : p->tiles_on                      ? std::min(rem, p->tiles.k)
+                                                            : stream_depth_at_most(p->R, p->star, rem);
         d.push_back(step);
         rem -= step;
     }
@@ -955,12 +979,37 @@ static stencil_status_t launch_states(stencil_plan_t* p, const void* src, float*
 }
 
 namespace gbst {
-stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n,
+// The entry points that return sums over the grid in FP64 (weight gradients,
+// residuals) resolve the last bits of the states.  Register tiles give the bits of
+// the kernel they stand in for (cluster-resident: GridConfig::plain; else
+// streaming), except where the streaming kernel's depend on how steps are grouped:
+// periodic widths that are not a multiple of 4, and 16-bit storage.  For one such
+// call, on = true puts a plan of these kinds back on the streaming kernel (true: it
+// did, and on = false undoes it).
+bool plan_keep_sums(stencil_plan_t* p, bool on) {
+    if (!on) {
+        p->kernel = p->kept_kernel;
+        p->grid_on = p->kept_grid;
+        p->tiles_on = p->kept_tiles;
+        return false;
+    }
+    if (!(p->grid_on || p->tiles_on) || p->opt.autotune || (p->grid_on && p->grid.plain)) return false;
+    if (p->dtype == STENCIL_F32 && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0)) return false;
+    p->kept_kernel = p->kernel;
+    p->kept_grid = p->grid_on;
+    p->kept_tiles = p->tiles_on;
+    p->kernel = STENCIL_KERNEL_STREAM;
+    p->grid_on = p->tiles_on = 0;
+    return true;
+}
+
+stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
                                  cudaStream_t st) {
     // Chip-resident plans: every state in one launch (13-point star 1000 x 1022: a
     // single-step launch per state took 13 us each).  Not for periodic ragged widths,
-    // whose bits depend on how the steps are grouped.
-    bool strided = p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && p->dtype == STENCIL_F32 && n >= 1 &&
+    // whose bits depend on how the steps are grouped, and in the streaming kernel's
+    // summation order only (any_order: any will do).
+    bool strided = p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && (any_order || !p->grid.plain) && p->dtype == STENCIL_F32 && n >= 1 &&
                    n < (1 << 30) && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0);
     const int64_t stride = n > 1 ? outs[1] - outs[0] : 0;
     for (int64_t i = 1; i < n && strided; ++i) strided = outs[i] - outs[i - 1] == stride;
@@ -1006,7 +1055,7 @@ stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const
 stencil_status_t plan_run_last_two(stencil_plan_t* p, const void* in, void* g1, void* g2, void* g0, int64_t m,
                                    cudaStream_t st, const void** prev, const void** next) {
     if (p->dtype != STENCIL_F32 || m < 2 || (p->opt.autotune && !p->tuned)) return STENCIL_ERR_UNSUPPORTED;
-    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && m < (1 << 30) &&
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && !p->grid.plain && m < (1 << 30) &&
         !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0)) {
         const int vec = p->nx % 4 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)g1 % 16 == 0 && (uintptr_t)g2 % 16 == 0;
         const cudaError_t e = launch_grid(p->grid, p->R, p->star, p->dtype, p->boundary == STENCIL_BOUNDARY_PERIODIC, in,
@@ -1072,7 +1121,8 @@ static stencil_status_t time_launch(stencil_plan* p, const void* in, int reps, c
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     auto once = [&] {
-        return p->pad[0] ? launch_padded(p, p->pad[0], p->pad[1], p->k, false, st) : launch_once(p, in, p->ws, p->k, st);
+        return p->pad[0] ? launch_padded(p, p->pad[0], p->pad[1], p->k, false, st)
+                         : launch_once(p, in, p->ws, p->tiles_on ? p->tiles.k : p->k, st);
     };
     stencil_status_t s = once();  // warm-up
     if (s == STENCIL_OK) {
@@ -1146,13 +1196,15 @@ static stencil_status_t autotune_tc(stencil_plan* p, const void* in, cudaStream_
 }
 
 static stencil_status_t autotune(stencil_plan* p, const void* in, cudaStream_t st) {
-    const TuneKey key(p->ny, p->nx, p->R, p->star, p->dtype, p->boundary, p->device);
+    const TuneKey key(p->ny, p->nx, p->R + 32 * p->tiles_ok, p->star, p->dtype, p->boundary, p->device);
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            p->tma = it->second.second >> 16;
-            return configure_stream(p, it->second.first, it->second.second & 0xffff, p->opt.tile_rows);
+            p->tma = (it->second.second >> 16) & 1;
+            stencil_status_t s = configure_stream(p, it->second.first, it->second.second & 0xffff, p->opt.tile_rows);
+            if (s == STENCIL_OK) p->tiles_on = it->second.second >> 17;
+            return s;
         }
     }
     const int ths[3] = {64, 128, 256};
@@ -1199,8 +1251,17 @@ static stencil_status_t autotune(stencil_plan* p, const void* in, cudaStream_t s
     p->tma = btma;
     stencil_status_t s = configure_stream(p, bk, bt, p->opt.tile_rows);
     if (s != STENCIL_OK) return s;
+    if (p->tiles_ok) {
+        // the register tiles are this plan's default: they stay unless the best above is clearly faster
+        const int tk = p->tiles.k, reps = (int)std::max(1.0, std::min(64.0, 2e9 / (points * tk)));
+        float ms = 0.f;
+        p->tiles_on = 1;
+        s = time_launch(p, in, reps, st, &ms);
+        if (s != STENCIL_OK) return s;
+        p->tiles_on = ms / (float)(reps * tk) <= 1.02f * best;
+    }
     std::lock_guard<std::mutex> g(g_tune_mu);
-    g_tune_cache[key] = std::make_pair(bk, bt | (btma << 16));
+    g_tune_cache[key] = std::make_pair(bk, bt | (btma << 16) | (p->tiles_on << 17));
     return STENCIL_OK;
 }
 
@@ -1454,7 +1515,7 @@ stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t n
     }
     // Ragged widths under the zero rule: two grids of padded rows, the first of
     // which doubles as the workspace.
-    if (!p->ws && p->kernel == STENCIL_KERNEL_STREAM && pad_eligible(p)) {
+    if (!p->ws && p->kernel == STENCIL_KERNEL_STREAM && !p->tiles_on && pad_eligible(p)) {
         const int64_t ld = ceil_div(nx, kPadElems) * kPadElems;
         const size_t grid = ((size_t)ny * (size_t)ld * p->elem + 255) / 256 * 256;
         e = cudaMalloc(&p->ws, 2 * grid);
@@ -1550,7 +1611,16 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* p, stencil_plan_info_t*
     i.mma_n = p->umma_n;
     i.load = p->kernel == STENCIL_KERNEL_STREAM ? (p->tma ? STENCIL_LOAD_TMA : STENCIL_LOAD_CP_ASYNC) : 0;
     i.rank = p->kernel == STENCIL_KERNEL_LOWRANK ? p->lr_rank : 0;
-    if (p->kernel == STENCIL_KERNEL_STREAM && p->warp_nc) {
+    if (p->kernel == STENCIL_KERNEL_STREAM && p->tiles_on) {
+        i.tb_depth = p->tiles.k;
+        i.threads = 32 * p->tiles.warps;
+        i.halo_cols = p->tiles.H;
+        i.tile_cols = p->tiles.bx;
+        i.tile_rows = p->tiles.by;
+        i.ctas = p->tiles.strips * p->tiles.tiles_y;
+        i.smem_bytes = 0;
+    }
+    if (p->kernel == STENCIL_KERNEL_STREAM && p->warp_nc && !p->tiles_on) {
         i.threads = 32;
         i.halo_cols = kWarpDepth;
         i.tile_cols = p->warp_bx;

@@ -27,6 +27,7 @@ namespace gbst {
 void** plan_aux_slot(stencil_plan_t* p, int id);
 void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*));
 
+bool plan_keep_sums(stencil_plan_t* p, bool on);
 stencil_status_t plan_run_last_two(stencil_plan_t* p, const void* in, void* g1, void* g2, void* g0, int64_t m,
                                    cudaStream_t st, const void** prev, const void** next);
 
@@ -196,6 +197,14 @@ stencil_status_t stencil_run_residual(stencil_plan_t* plan, const void* in, void
     unsigned* finished = reinterpret_cast<unsigned*>(sc->partials + kResBlocks);
     RCK(cudaMemsetAsync(finished, 0, sizeof(unsigned), st));
     char* const G[3] = {sc->grids, sc->grids + sc->bytes, sc->count == 3 ? sc->grids + 2 * sc->bytes : nullptr};
+    // (residuals resolve the last bits of the states)
+    struct KeepSums {
+        stencil_plan_t* p;
+        const bool on;
+        ~KeepSums() {
+            if (on) plan_keep_sums(p, false);
+        }
+    } const kept{plan, T >= m && plan_keep_sums(plan, true)};
     const void* cur = in;
     int64_t t = 0, j = 0;
     while (t + m <= T) {

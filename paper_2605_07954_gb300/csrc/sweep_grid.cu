@@ -15,6 +15,10 @@ GridKernelRef get_grid_states_kernel_r1(int star, int rb);
 GridKernelRef get_grid_states_kernel_r2(int star, int rb);
 GridKernelRef get_grid_states_kernel_r3(int star, int rb);
 
+GridKernelRef get_grid_plain_kernel_r1(int star, int rb);
+GridKernelRef get_grid_plain_kernel_r2(int star, int rb);
+GridKernelRef get_grid_plain_kernel_r3(int star, int rb);
+
 static GridKernelRef grid_states_kernel(int R, int star, int rb) {
     switch (R) {
         case 1: return get_grid_states_kernel_r1(star, rb);
@@ -24,7 +28,13 @@ static GridKernelRef grid_states_kernel(int R, int star, int rb) {
     }
 }
 
-static GridKernelRef grid_kernel(int R, int star, int rb) {
+static GridKernelRef grid_kernel(int R, int star, int rb, int plain = 0) {
+    if (plain) switch (R) {
+            case 1: return get_grid_plain_kernel_r1(star, rb);
+            case 2: return get_grid_plain_kernel_r2(star, rb);
+            case 3: return get_grid_plain_kernel_r3(star, rb);
+            default: return {nullptr, 0};
+        }
     switch (R) {
         case 1: return get_grid_kernel_r1(star, rb);
         case 2: return get_grid_kernel_r2(star, rb);
@@ -78,9 +88,50 @@ bool grid_config(int ny, int nx, int R, int star, int periodic, int sms, int k, 
     return found;
 }
 
+constexpr double kTilesWave = 8000.0;  // launches of tiles: a wave's loads, stores, start and end
+
+bool tiles_config(int ny, int nx, int R, int star, int periodic, int sms, int kmin, GridConfig* out) {
+    const int taps = star ? 4 * R + 1 : (2 * R + 1) * (2 * R + 1);
+    bool found = false;
+    for (int rows : kGridRows) {
+        const GridKernelRef ref = grid_kernel(R, star, rows);
+        if (!ref.fn) continue;
+        for (int kk = kmin; kk <= kGridMaxK; ++kk) {
+            GridConfig c;
+            c.rb = rows;
+            c.k = kk;
+            c.Hy = R * kk;
+            c.H = up(R * kk, 4) * 4;
+            c.bx = kGridCols - 2 * c.H;
+            if (c.bx < 8) break;
+            const int ex = periodic ? 0 : 2 * c.H, ey = periodic ? 0 : 2 * c.Hy;
+            c.strips = std::max(1, up(nx - ex, c.bx));
+            const int max_warps = std::min(ref.max_threads / 32, (kGridMaxSmem / (R * 32 * 16) - 1) / 4);
+            const int by_max = max_warps * rows - 2 * c.Hy;
+            if (by_max < 1) break;
+            // the fewest tile rows, and up to three times as many (more CTAs per SM, fuller last waves)
+            const int fewest = std::max(1, up(ny - ey, by_max));
+            for (int ty = fewest; ty <= std::min(3 * fewest, fewest + 64); ++ty) {
+                c.by = std::max(1, up(ny - ey, ty));
+                c.tiles_y = std::max(1, up(ny - ey, c.by));
+                c.warps = up(std::min(c.by + 2 * c.Hy, periodic ? 1 << 30 : ny), rows);
+                if (c.warps > max_warps || c.warps < 4) continue;
+                const int per_sm = std::max(1, max_warps / c.warps);
+                const long long waves = ((long long)c.strips * c.tiles_y + (long long)sms * per_sm - 1) /
+                                        ((long long)sms * per_sm);
+                const double wave = kk * (kGridStep + up(per_sm * c.warps, 4) * rows * grid_row_cycles(taps, R)) + kTilesWave;
+                c.cycles = (double)waves * wave / kk;
+                if (!found || c.cycles < out->cycles) *out = c;
+                found = true;
+            }
+        }
+    }
+    return found;
+}
+
 bool grid_fits(const GridConfig& c, int R, int star, int sms) {
-    const GridKernelRef ref = grid_kernel(R, star, c.rb);
-    if (!ref.fn || c.strips * c.tiles_y > sms) return false;
+    const GridKernelRef ref = grid_kernel(R, star, c.rb, c.plain);
+    if (!ref.fn || (sms > 0 && c.strips * c.tiles_y > sms)) return false;
     const int smem = grid_smem_bytes(R, c.warps);
     int per_sm = 0;
     if (cudaFuncSetAttribute(ref.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kGridMaxSmem) != cudaSuccess ||
@@ -100,7 +151,7 @@ cudaError_t launch_grid(const GridConfig& c, int R, int star, int dtype, int per
                         int ny, int nx, int vec, int T, int k, void* scratch, unsigned* status, long long wait_ns,
                         int withhold, const Weights& w, cudaStream_t st, float* states,
                         long long state_stride, int state_first) {
-    const GridKernelRef ref = states ? grid_states_kernel(R, star, c.rb) : grid_kernel(R, star, c.rb);
+    const GridKernelRef ref = states ? grid_states_kernel(R, star, c.rb) : grid_kernel(R, star, c.rb, c.plain);
     if (!ref.fn) return cudaErrorInvalidValue;
     if (states) {  // (plain kernels: set when the plan is made, by grid_fits)
         const cudaError_t e =
@@ -140,6 +191,34 @@ cudaError_t launch_grid(const GridConfig& c, int R, int star, int dtype, int per
     void* args[] = {&p};
     return cudaLaunchCooperativeKernel(ref.fn, dim3((unsigned)(c.strips * c.tiles_y)), dim3((unsigned)(c.warps * 32)),
                                        args, (size_t)grid_smem_bytes(R, c.warps), st);
+}
+
+cudaError_t launch_tiles(const GridConfig& c, int R, int star, int dtype, int periodic, const void* in, void* out,
+                         int ny, int nx, int vec, int T, const Weights& w, cudaStream_t st) {
+    const GridKernelRef ref = grid_kernel(R, star, c.rb);
+    if (!ref.fn || T > c.k || in == out) return cudaErrorInvalidValue;
+    GridParams p{};
+    p.in = in;
+    p.out = out;
+    p.ny = ny;
+    p.nx = nx;
+    p.ld = nx;
+    p.T = T;
+    p.k = c.k;
+    p.Hy = c.Hy;
+    p.H = c.H;
+    p.bx = c.bx;
+    p.by = c.by;
+    p.strips = c.strips;
+    p.tiles_y = c.tiles_y;
+    p.periodic = periodic;
+    p.dtype = dtype;
+    p.vec = vec;
+    p.w = w;
+    for (int i = 0; i < kMaxTaps; ++i) p.w2.w2[i] = make_float2(w.w[i], w.w[i]);
+    void* args[] = {&p};
+    return cudaLaunchKernel(ref.fn, dim3((unsigned)(c.strips * c.tiles_y)), dim3((unsigned)(c.warps * 32)), args,
+                            (size_t)grid_smem_bytes(R, c.warps), st);
 }
 
 }  // namespace gbst

@@ -2,7 +2,9 @@
 // chip, all T steps of a run in one cooperative launch (sm_103a).
 //
 // The Jacobi update of Sec. II-C as the streaming kernel computes it (same
-// products in the same order, so the same bits for FP32 storage), for grids
+// products in the same order, so the same bits for FP32 storage; the PLAIN kernels
+// have the cluster-resident kernel's order and bits, for the grids that it would
+// take: FP64 residuals and gradients resolve the difference), for grids
 // that fit on the chip as one register tile per SM.  A CTA stages its tile with
 // a halo of Hy = R*k rows and H >= R*k columns per side (none at the grid's own
 // edges): warp w keeps staged rows [w*RB, w*RB+RB), each lane 4 adjacent columns
@@ -43,6 +45,11 @@
 // to hide latency: up to twice as slow at 1024^2), two or three CTAs per SM with
 // smaller tiles (3-25 % slower: more halo rows than they hide).
 //
+// One group of steps exchanges nothing, so a launch of at most k steps is also an
+// ordinary kernel over any number of tiles (launch_tiles): grids a little too
+// large for one tile per SM, and periodic ragged rows (the lines and both sides'
+// times stand at choose_tiles in plan.cu).
+//
 // Waits.  Tiles wait for one another, so the launch is cooperative (all CTAs
 // resident).  Each wait is bounded (globaltimer limit and an iteration cap): an
 // expired one records STENCIL_ERR_TIMEOUT, raises an abort flag that every
@@ -70,7 +77,7 @@ struct GridParams {
     const void* in;
     void* out;
     uint2* xbuf[2];   // exchange grids: ny rows of xld (value, epoch) pairs
-    int* ctl;         // control words
+    int* ctl;         // control words (null: a launch of at most k steps, which exchanges nothing)
     unsigned* status;
     long long wait_ns;
     int ny, nx, ld, xld;
@@ -150,7 +157,11 @@ __device__ __forceinline__ float grid_keep(float v, unsigned m) {
 // One step of a warp's RB rows in place.  `top` / `bot`: the R staged rows
 // above and below (32 chunks per row, as column pairs); MASK: points outside
 // the grid are forced to zero.
-template <int R, bool STAR, int RB, bool MASK, class WS>
+//
+// PLAIN: every output adds its products row by row with dx ascending, the
+// cluster-resident kernel's order, in place of the streaming kernel's (own chunk
+// first).
+template <int R, bool STAR, int RB, bool MASK, bool PLAIN, class WS>
 __device__ __forceinline__ void grid_step(const WS& ws, float2 (&u)[RB][2], const float4* top, const float4* bot,
                                           int lane, const GridEdges& ed) {
     constexpr int D = 2 * R + 1;
@@ -180,7 +191,53 @@ __device__ __forceinline__ void grid_step(const WS& ws, float2 (&u)[RB][2], cons
             Pa = u[i - R][0];
             Pb = u[i - R][1];
         }
-        if constexpr (R == 1) {
+        if constexpr (PLAIN) {
+            // q[d]: the output pairs' operands at column offset d - R
+            float2 q0[D], q1[D];
+            constexpr bool centre = STAR && halo_row;
+            if constexpr (R == 1) {
+                q0[1] = Pa;
+                q1[1] = Pb;
+                if constexpr (!centre) {
+                    q0[0] = make_float2(left(Pb.y), Pb.x);
+                    q0[2] = Pb;
+                    q1[0] = Pa;
+                    q1[2] = make_float2(Pa.y, right(Pa.x));
+                }
+            } else if constexpr (centre) {
+                q0[R] = Pa;
+                q1[R] = Pb;
+            } else {
+                float ext[4 + 2 * R];
+                ext[R + 0] = Pa.x;
+                ext[R + 1] = Pa.y;
+                ext[R + 2] = Pb.x;
+                ext[R + 3] = Pb.y;
+                ext[R - 1] = left(Pb.y);
+                ext[R - 2] = left(Pb.x);
+                if (R == 3) ext[0] = left(Pa.y);
+                ext[R + 4] = right(Pa.x);
+                ext[R + 5] = right(Pa.y);
+                if (R == 3) ext[R + 6] = right(Pb.x);
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    q0[d] = make_float2(ext[d], ext[d + 1]);
+                    q1[d] = make_float2(ext[d + 2], ext[d + 3]);
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < D; ++a) {  // weight row: output row i - a
+                if (i - a < 0 || i - a >= RB) continue;
+                const int slot = (i - a + R) % D;
+                if (a == 0) acc[slot][0] = acc[slot][1] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    if (STAR && a != R && d != R) continue;
+                    acc[slot][0] = __ffma2_rn(ws.w2(a * D + d), q0[d], acc[slot][0]);
+                    acc[slot][1] = __ffma2_rn(ws.w2(a * D + d), q1[d], acc[slot][1]);
+                }
+            }
+        } else if constexpr (R == 1) {
             own_products<R, STAR, 0, 2 * R>(ws, acc, Pa, Pb, i);
             if constexpr (!(STAR && halo_row)) {
                 ExtRow<R> ext;
@@ -341,7 +398,7 @@ static __device__ __noinline__ bool grid_wait_over(const GridParams& p, unsigned
 // STATES: every step's result is stored as well (a variant of its own: the branch
 // in the step loop cost the plain runs 6 %, 5-point star 512^2 x 100 steps 52.4 ->
 // 55.5 us).
-template <int R, bool STAR, int RB, bool STATES = false>
+template <int R, bool STAR, int RB, bool STATES = false, bool PLAIN = false>
 __global__ void __launch_bounds__(grid_max_threads(R, RB), 1)
     sweep_grid_kernel(const __grid_constant__ GridParams p) {
     extern __shared__ float4 grid_rows[];  // [parity][warp][first rows, last rows][R][32], then R zero rows
@@ -381,7 +438,8 @@ __global__ void __launch_bounds__(grid_max_threads(R, RB), 1)
 
     // The generation this launch counts from: read before any CTA can leave
     // (the last one to leave moves it on).
-    if (threadIdx.x == 0) s_base = *(volatile unsigned*)gen;
+    // (No control words: one group of steps, nothing to count.)
+    if (threadIdx.x == 0) s_base = p.ctl ? *(volatile unsigned*)gen : 0u;
     float4* const zero_rows = grid_rows + 4 * warps * R * 32;
     for (int i = threadIdx.x; i < R * 32; i += blockDim.x) zero_rows[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 
@@ -454,8 +512,8 @@ __global__ void __launch_bounds__(grid_max_threads(R, RB), 1)
             const float4* top = warp > 0 ? mine - R * 32 : zero_rows;
             const float4* bot = warp + 1 < warps ? mine + 2 * R * 32 : zero_rows;
             if (!idle) {
-                if (mask) grid_step<R, STAR, RB, true>(ws, u, top, bot, lane, ed);
-                else grid_step<R, STAR, RB, false>(ws, u, top, bot, lane, ed);
+                if (mask) grid_step<R, STAR, RB, true, PLAIN>(ws, u, top, bot, lane, ed);
+                else grid_step<R, STAR, RB, false, PLAIN>(ws, u, top, bot, lane, ed);
             }
             par ^= 1;
             if (STATES && t + s + 1 < p.T && t + s + 1 >= p.state_first && col_own) {
@@ -568,7 +626,7 @@ __global__ void __launch_bounds__(grid_max_threads(R, RB), 1)
     }
     // Leave: the last CTA moves the generation past this launch's epochs.
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && p.ctl) {
         const unsigned groups = (unsigned)((p.T + p.k - 1) / p.k);
         if (atomicAdd(leave, 1) == (int)gridDim.x - 1) {
             atomicExch(leave, 0);

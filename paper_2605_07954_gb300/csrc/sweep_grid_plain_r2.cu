@@ -1,0 +1,19 @@
+// sweep_grid_plain_r2.cu -- chip-resident register-tile kernels in the plain summation order: radius 2.
+#include "sweep_grid.cuh"
+
+namespace gbst {
+
+// Kernel with rb rows per warp ({nullptr, 0} if not instantiated).
+GridKernelRef get_grid_plain_kernel_r2(int star, int rb) {
+    switch (rb) {
+        case 4:
+            return {star ? (const void*)sweep_grid_kernel<2, true, 4, false, true> : (const void*)sweep_grid_kernel<2, false, 4, false, true>,
+                    grid_max_threads(2, 4)};
+        case 8:
+            return {star ? (const void*)sweep_grid_kernel<2, true, 8, false, true> : (const void*)sweep_grid_kernel<2, false, 8, false, true>,
+                    grid_max_threads(2, 8)};
+        default: return {nullptr, 0};
+    }
+}
+
+}  // namespace gbst
