@@ -595,6 +595,45 @@ static bool grid_candidate(stencil_plan* p) {
     return p->grid_ok != 0;
 }
 
+// Grids too large for one register tile per SM: the same tiles as launches of up
+// to tiles.k steps, two or three waves of them, in place of the streaming
+// kernel's launches.  Between the register tiles' limit and about 2048^2 the
+// streaming kernel has too few rows per tile: a launch is 15-20 us of pipeline
+// fill and halo rows.  48 steps in us, register tiles | streaming kernel, FP32,
+// zero rule, GB300:
+//   1600^2       5-point star 108 | 138  9-point box 152 | 188  9-point star 176 | 274
+//                5x5 box 324 | 519  13-point star 244 | 401  7x7 box 594 | 790
+//   2048^2       141 | 176  208 | 187  249 | 348  597 | 741  362 | 528  828 | 1140
+//   2304^2       176 | 175  275 | 224  323 | 348  619 | 741  463 | 561  1036 | 1235
+//   1024 x 4096  166 | 140  224 | 187  258 | 289  540 | 716  373 | 495  862 | 1137
+//   4096 x 1024  141 | 163  193 | 224  259 | 322  541 | 742  373 | 560  840 | 1441
+//   2001 x 2003  176 | 187  225 | 220  311 | 383  545 | 778  449 | 636  1037 | 1232
+// (BF16 alike; above 2400^2 the streaming kernel is the faster one: 3000^2 321 |
+// 212 ... 1629 | 1479).  So: up to 4.3 M points (boxes of radius 1: 2.8 M), and
+// for radius 1 no grids much wider than high, which the streaming kernel covers
+// with fewer halo rows.  Periodic rows that are not a multiple of 4 wide, which
+// the streaming kernel must load element by element through the wrap in every
+// launch, take the tiles at every size: 2001 x 2003 186 | 643 ... 1673 | 2742,
+// 4001 x 5003 719 | 1415 ... 4198 | 6094, 9001 x 8003 2611 | 4408 ... 14997 |
+// 18195; 16-bit boxes of radius 2 and 3 only up to 40 M points (4001 x 5003 2910 |
+// 3398, 9001 x 8003 10519 | 10209).
+static void choose_tiles(stencil_plan* p) {
+    if (p->ny > (1 << 20) || p->nx > (1 << 20)) return;
+    const int periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
+    const double points = (double)p->ny * (double)p->nx;
+    if (periodic && p->nx % 4 != 0) {
+        if (p->dtype != STENCIL_F32 && !p->star && p->R > 1 && points > 4e7) return;
+    } else {
+        if (points > (p->R == 1 && !p->star ? 2.8e6 : 4.3e6)) return;
+        if (p->R == 1 && p->nx > 1.5 * p->ny) return;
+    }
+    // 16-bit storage rounds once per launch: never more launches than the streaming kernel's
+    const int kmin = std::max(2, p->dtype == STENCIL_F32 ? 1 : p->k);
+    if (!tiles_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, kmin, &p->tiles)) return;
+    p->tiles_ok = p->tiles_on = grid_fits(p->tiles, p->R, p->star, 0);
+    if (p->tiles_on) p->warp_nc = 0;
+}
+
 // Whether a launch of nlev steps runs as register tiles.  Aligned launches of a
 // step or two (a run's remainder) are cheaper without the tiles' deep halo:
 // 2048^2, 1 step, 5-point star 15 us as tiles, 12 streaming, 13-point star 19 |
@@ -1485,6 +1524,7 @@ stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t n
         if (st == STENCIL_OK && may_grid && grid_candidate(p)) use_grid(p);
         if (st == STENCIL_OK && p->grid_on && o.autotune) resident_candidates(p);  // to be timed as well
         if (!p->grid_on) st = cluster_choice(st);
+        if (st == STENCIL_OK && may_grid && p->kernel == STENCIL_KERNEL_STREAM) choose_tiles(p);
     }
     if (st != STENCIL_OK) return bail(st);
 

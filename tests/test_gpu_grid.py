@@ -151,3 +151,62 @@ def test_expired_wait_reports_timeout_and_plan_recovers():
     ref = _reference_plan((512, 512), W)
     assert torch.equal(good.run(x, 60), ref.run(x, 60))
     good.status()
+
+
+# Grids beyond one tile per SM: launches of up to tb_depth steps over two or more
+# waves of tiles.  Just above that limit, two waves, tall and wide, ragged.
+TILE_SHAPES = [("heat5", (1600, 1600)), ("heat5", (4099, 1021)), ("box9", (1601, 1701)), ("star9", (2048, 2048)),
+               ("star9", (1024, 4099)), ("box25", (2001, 2003)), ("star13", (1801, 1804)), ("star13", (8190, 517)),
+               ("box49", (2048, 2048)), ("box49", (1701, 1601))]
+
+
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+@pytest.mark.parametrize("name,shape", TILE_SHAPES)
+def test_launches_of_tiles_same_bits(name, shape, boundary):
+    W = _weights(name)
+    x = torch.from_numpy(inputs.field(*shape)).cuda()
+    p = _plan(shape, W, grid=False, boundary=boundary)
+    q = _plan(shape, W, grid=False, boundary=boundary, kernel="stream")
+    i = p.info()
+    assert i["kernel"] == 2 and i["threads"] > 256 and i["tb_depth"] >= 2, i  # (the streaming kernel: at most 256)
+    k = i["tb_depth"]
+    for T in (1, 2, k, k + 1, 2 * k + 3):
+        y, z = p.run(x, T), q.run(x, T)
+        v = x.clone()
+        p.run(v, T, out=v)
+        if boundary == "periodic" and shape[1] % 4:
+            assert rel_l2(y.cpu().numpy(), z.cpu().numpy().astype(np.float64)) <= fp32_tol(T), T
+            assert rel_l2(v.cpu().numpy(), z.cpu().numpy().astype(np.float64)) <= fp32_tol(T), T
+        else:
+            assert torch.equal(y, z) and torch.equal(v, z), T
+        assert p.launches(T) == -(-T // k)
+    p.close()
+    q.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("name,shape", [("star13", (2048, 2048)), ("box9", (1601, 1701))])
+def test_launches_of_tiles_16_bit(dtype, name, shape):
+    """One rounding per launch, and no more launches than the streaming kernel's."""
+    W = _weights(name)
+    x = torch.from_numpy(inputs.field(*shape)).cuda().to(TDT[dtype])
+    p = _plan(shape, W, grid=False, dtype=dtype)
+    q = _plan(shape, W, grid=False, dtype=dtype, kernel="stream")
+    k = p.info()["tb_depth"]
+    assert p.info()["threads"] > 256 and k >= q.info()["tb_depth"]
+    y = p.run(x, k)
+    z = _plan(shape, W, grid=False, kernel="stream").run(x.float(), k)
+    assert torch.equal(y, z.to(TDT[dtype]))
+    y = p.run(x, 2 * k)
+    z = p.run(p.run(x, k), k)
+    assert torch.equal(y, z)
+
+
+def test_launches_of_tiles_autotuned():
+    """Autotuning times the tiles against the streaming kernel's variants; the bits are the same."""
+    shape, W = (1801, 1804), inputs.pattern_weights("star13")
+    x = torch.from_numpy(inputs.field(*shape)).cuda()
+    y = _plan(shape, W, grid=False, autotune=True).run(x, 23)
+    again = _plan(shape, W, grid=False, autotune=True)  # (the cached choice)
+    z = _plan(shape, W, grid=False, kernel="stream").run(x, 23)
+    assert torch.equal(y, z) and torch.equal(again.run(x, 23), z)
