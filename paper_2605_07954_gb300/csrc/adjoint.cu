@@ -69,7 +69,7 @@ stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const
 // longer than the staged-tile form's 8 products and 5 levels of lane sums.
 //
 // What bounds it: FMA issue, (13 or 49) + 49 FMAs per point for radius 3.  The
-// staged-tile form it replaces (one point per lane and row, both windows read
+// staged-tile form (one point per lane and row, both windows read
 // from shared memory) ran the 13-point star at 1000 x 1022 in 26.4 us a step:
 // now 14.4 (ncu).
 constexpr int kAdrWarps = 4;
@@ -832,7 +832,11 @@ stencil_status_t adjoint_run(stencil_plan_t* plan, const void* u0, const void* g
     // nx % 4 == 0, and the buffers below are then 16-byte aligned), else the
     // any-width one.
     const bool streamed = adjoint_stream_kernel_fn(R) != nullptr && nx % 4 == 0;
-    const bool rows = w32 && R > 1;
+    // (a star's off-axis weights are zero: adjoint_rows_kernel skips them in the lambda
+    // update.  Small boxes have too few of its 120 x 32 tiles: 7x7, 32 steps, 96 x 100
+    // 854 us staged, 920 by rows; 160^2 855 | 409, register-tile states included)
+    const bool star = adj_star(wf, R);
+    const bool rows = w32 && R > 1 && (star || n > 20000);
     const int tile_cols = streamed ? kAdsCols : rows ? kAdrCols : kAdjTX;
     const int tiles_x = (nx + tile_cols - 1) / tile_cols;
     const int tile_rows = streamed ? kAdsWarps * kAdsRows : rows ? kAdrWarps * kAdrRows : kAdjTY;
@@ -868,9 +872,8 @@ stencil_status_t adjoint_run(stencil_plan_t* plan, const void* u0, const void* g
     }
     ACK(cudaMemcpyAsync(lam[0], grad_uT, bytes, cudaMemcpyDeviceToDevice, st));
     int cur = 0;
-    // (a star's off-axis weights are zero: the lambda update skips them)
     const void* kfn = streamed ? adjoint_stream_kernel_fn(R)
-                      : rows   ? adjoint_rows_kernel_fn(R, adj_star(wf, R))
+                      : rows   ? adjoint_rows_kernel_fn(R, star)
                                : adjoint_step_kernel_fn(R);
     if (!kfn) return afail(STENCIL_ERR_UNSUPPORTED, "no adjoint kernel for this radius");
     const dim3 block = streamed ? dim3(kAdsWarps * 32) : rows ? dim3(kAdrWarps * 32) : dim3(32, 8);

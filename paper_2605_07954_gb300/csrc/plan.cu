@@ -590,7 +590,12 @@ static bool grid_candidate(stencil_plan* p) {
     }
     const int periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
     if (!grid_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, 0, 0, &p->grid)) return false;
+    // the cluster-resident kernel's bits where AUTO would otherwise take that kernel
     p->grid.plain = resident_candidates(p) > 0;
+    // (boxes of radius 2 and 3 of up to about 140^2 points, where each tile is mostly
+    // halo, stay with it: 96 x 100, 7x7 100 steps 129 us against 164, 5x5 16 steps 21
+    // against 22; at 160^2 it is 1.2 and 1.3 times as slow, at 400^2 2.4 and 2.6)
+    if (p->grid.plain && p->R >= 2 && !p->star && p->ny * p->nx <= 20000) return false;
     p->grid_ok = grid_fits(p->grid, p->R, p->star, p->sms);
     return p->grid_ok != 0;
 }
@@ -609,9 +614,10 @@ static bool grid_candidate(stencil_plan* p) {
 //   4096 x 1024  141 | 163  193 | 224  259 | 322  541 | 742  373 | 560  840 | 1441
 //   2001 x 2003  176 | 187  225 | 220  311 | 383  545 | 778  449 | 636  1037 | 1232
 // (BF16 alike; above 2400^2 the streaming kernel is the faster one: 3000^2 321 |
-// 212 ... 1629 | 1479).  So: up to 4.3 M points (boxes of radius 1: 2.8 M), and
-// for radius 1 no grids much wider than high, which the streaming kernel covers
-// with fewer halo rows.  Periodic rows that are not a multiple of 4 wide, which
+// 212 ... 1629 | 1479).  So: up to 4.3 M points (radius 1: 3.3 M for stars, whose
+// runs of a few launches gain nothing above: 1900 x 2000, 16 steps 54 | 46; 2.8 M
+// for boxes), and for radius 1 no grids much wider than high, which the streaming
+// kernel covers with fewer halo rows.  Periodic rows that are not a multiple of 4 wide, which
 // the streaming kernel must load element by element through the wrap in every
 // launch, take the tiles at every size: 2001 x 2003 186 | 643 ... 1673 | 2742,
 // 4001 x 5003 719 | 1415 ... 4198 | 6094, 9001 x 8003 2611 | 4408 ... 14997 |
@@ -624,7 +630,7 @@ static void choose_tiles(stencil_plan* p) {
     if (periodic && p->nx % 4 != 0) {
         if (p->dtype != STENCIL_F32 && !p->star && p->R > 1 && points > 4e7) return;
     } else {
-        if (points > (p->R == 1 && !p->star ? 2.8e6 : 4.3e6)) return;
+        if (points > (p->R > 1 ? 4.3e6 : p->star ? 3.3e6 : 2.8e6)) return;
         if (p->R == 1 && p->nx > 1.5 * p->ny) return;
     }
     // 16-bit storage rounds once per launch: never more launches than the streaming kernel's

@@ -233,8 +233,14 @@ __device__ __forceinline__ void grid_step(const WS& ws, float2 (&u)[RB][2], cons
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
                     if (STAR && a != R && d != R) continue;
-                    acc[slot][0] = __ffma2_rn(ws.w2(a * D + d), q0[d], acc[slot][0]);
-                    acc[slot][1] = __ffma2_rn(ws.w2(a * D + d), q1[d], acc[slot][1]);
+                    if (WS::pinned(a * D + d)) {
+                        acc[slot][0] = __ffma2_rn(ws.w2(a * D + d), q0[d], acc[slot][0]);
+                        acc[slot][1] = __ffma2_rn(ws.w2(a * D + d), q1[d], acc[slot][1]);
+                    } else {  // weights from the constant bank
+                        const float w = ws.p.w.w[a * D + d];
+                        acc[slot][0] = make_float2(fmaf(w, q0[d].x, acc[slot][0].x), fmaf(w, q0[d].y, acc[slot][0].y));
+                        acc[slot][1] = make_float2(fmaf(w, q1[d].x, acc[slot][1].x), fmaf(w, q1[d].y, acc[slot][1].y));
+                    }
                 }
             }
         } else if constexpr (R == 1) {

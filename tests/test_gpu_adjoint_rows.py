@@ -51,7 +51,9 @@ def test_gradients(oracle, name, boundary, shape, entry):
     assert np.linalg.norm(gu - ref_u) <= 1e-5 * np.linalg.norm(ref_u)
     assert np.linalg.norm(gw - ref_w) <= 1e-5 * np.linalg.norm(ref_w)
     # the states of the streaming kernels have the same bits, so the gradients have
-    if entry == "stencil_adjoint_w32" and not (boundary == "periodic" and shape[1] % 4):
+    # (small boxes: cluster-resident kernel)
+    tiles = name not in ("box25", "box49") or shape[0] * shape[1] > 20000
+    if entry == "stencil_adjoint_w32" and tiles and not (boundary == "periodic" and shape[1] % 4):
         su, sw = _grads(u0, W, T, gT, boundary, entry, kernel="stream")
         assert np.array_equal(gu, su) and np.array_equal(gw, sw)
     assert rel_l2(gu, ref_u) <= 1e-5
