@@ -595,6 +595,9 @@ static bool grid_candidate(stencil_plan* p) {
     // (boxes of radius 2 and 3 of up to about 140^2 points, where each tile is mostly
     // halo, stay with it: 96 x 100, 7x7 100 steps 129 us against 164, 5x5 16 steps 21
     // against 22; at 160^2 it is 1.2 and 1.3 times as slow, at 400^2 2.4 and 2.6)
+    // 16-bit storage: the streaming kernel rounds once per launch, which adds up over a
+    // long run; grids that it takes keep its roundings
+    if (p->dtype != STENCIL_F32 && !p->grid.plain) return false;
     if (p->grid.plain && p->R >= 2 && !p->star && p->ny * p->nx <= 20000) return false;
     p->grid_ok = grid_fits(p->grid, p->R, p->star, p->sms);
     return p->grid_ok != 0;
@@ -613,7 +616,7 @@ static bool grid_candidate(stencil_plan* p) {
 //   1024 x 4096  166 | 140  224 | 187  258 | 289  540 | 716  373 | 495  862 | 1137
 //   4096 x 1024  141 | 163  193 | 224  259 | 322  541 | 742  373 | 560  840 | 1441
 //   2001 x 2003  176 | 187  225 | 220  311 | 383  545 | 778  449 | 636  1037 | 1232
-// (BF16 alike; above 2400^2 the streaming kernel is the faster one: 3000^2 321 |
+// (above 2400^2 the streaming kernel is the faster one: 3000^2 321 |
 // 212 ... 1629 | 1479).  So: up to 4.3 M points (radius 1: 3.3 M for stars, whose
 // runs of a few launches gain nothing above: 1900 x 2000, 16 steps 54 | 46; 2.8 M
 // for boxes), and for radius 1 no grids much wider than high, which the streaming
@@ -621,21 +624,17 @@ static bool grid_candidate(stencil_plan* p) {
 // the streaming kernel must load element by element through the wrap in every
 // launch, take the tiles at every size: 2001 x 2003 186 | 643 ... 1673 | 2742,
 // 4001 x 5003 719 | 1415 ... 4198 | 6094, 9001 x 8003 2611 | 4408 ... 14997 |
-// 18195; 16-bit boxes of radius 2 and 3 only up to 40 M points (4001 x 5003 2910 |
-// 3398, 9001 x 8003 10519 | 10209).
+// 18195.
 static void choose_tiles(stencil_plan* p) {
-    if (p->ny > (1 << 20) || p->nx > (1 << 20)) return;
+    // (16-bit storage rounds once per launch, so its results depend on the depth)
+    if (p->dtype != STENCIL_F32 || p->ny > (1 << 20) || p->nx > (1 << 20)) return;
     const int periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
     const double points = (double)p->ny * (double)p->nx;
-    if (periodic && p->nx % 4 != 0) {
-        if (p->dtype != STENCIL_F32 && !p->star && p->R > 1 && points > 4e7) return;
-    } else {
+    if (!(periodic && p->nx % 4 != 0)) {
         if (points > (p->R > 1 ? 4.3e6 : p->star ? 3.3e6 : 2.8e6)) return;
         if (p->R == 1 && p->nx > 1.5 * p->ny) return;
     }
-    // 16-bit storage rounds once per launch: never more launches than the streaming kernel's
-    const int kmin = std::max(2, p->dtype == STENCIL_F32 ? 1 : p->k);
-    if (!tiles_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, kmin, &p->tiles)) return;
+    if (!tiles_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, 2, &p->tiles)) return;
     p->tiles_ok = p->tiles_on = grid_fits(p->tiles, p->R, p->star, 0);
     if (p->tiles_on) p->warp_nc = 0;
 }
@@ -854,9 +853,10 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
 // rows cannot be padded: a wrapped chunk would read the padding.)  Measured on
 // GB300, 64 steps, us padded | element-wise: 4001 x 5003 5-point star FP32 540 |
 // 809, BF16 519 | 849; 9-point box 706 | 871, 683 | 1030; 13-point star 1622 |
-// 2242, 1567 | 2241; 5x5 box BF16 2353 | 2512; 7x7 box BF16 3568 | 3724.  The
-// FP32 boxes of radius 2 and 3 are bound by arithmetic either way and keep the
-// dense grids (5x5 1600 x 1701 830 | 777, 7x7 4001 x 5003 3512 | 3233).
+// 2242, 1567 | 2241; 5x5 box BF16 2353 | 2512.  The FP32 boxes of radius 2 and the
+// 7x7 boxes are bound by arithmetic either way and keep the dense grids (5x5 FP32
+// 1600 x 1701 830 | 777; 7x7 FP32 4001 x 5003 3512 | 3233; 7x7 BF16 4001 x 5003 3568 |
+// 3724, but 3001 x 2053, 400 steps, 13145 | 11525).
 
 constexpr int kPadElems = 16;  // pitch granularity
 
@@ -1028,9 +1028,8 @@ namespace gbst {
 // residuals) resolve the last bits of the states.  Register tiles give the bits of
 // the kernel they stand in for (cluster-resident: GridConfig::plain; else
 // streaming), except where the streaming kernel's depend on how steps are grouped:
-// periodic widths that are not a multiple of 4, and 16-bit storage.  For one such
-// call, on = true puts a plan of these kinds back on the streaming kernel (true: it
-// did, and on = false undoes it).
+// periodic widths that are not a multiple of 4.  For one such call, on = true puts
+// such a plan back on the streaming kernel (true: it did, and on = false undoes it).
 bool plan_keep_sums(stencil_plan_t* p, bool on) {
     if (!on) {
         p->kernel = p->kept_kernel;
@@ -1039,7 +1038,7 @@ bool plan_keep_sums(stencil_plan_t* p, bool on) {
         return false;
     }
     if (!(p->grid_on || p->tiles_on) || p->opt.autotune || (p->grid_on && p->grid.plain)) return false;
-    if (p->dtype == STENCIL_F32 && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0)) return false;
+    if (!(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0)) return false;
     p->kept_kernel = p->kernel;
     p->kept_grid = p->grid_on;
     p->kept_tiles = p->tiles_on;

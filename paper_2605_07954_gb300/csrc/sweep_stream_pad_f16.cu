@@ -35,8 +35,6 @@ StreamKernelRef get_stream_pad_kernel_f16(int R, int star, int k) {
         case 201: return pad_ref<2, false, 1>();
         case 202: return pad_ref<2, false, 2>();
         case 204: return pad_ref<2, false, 4>();
-        case 301: return pad_ref<3, false, 1>();
-        case 302: return pad_ref<3, false, 2>();
         default: return {nullptr, 0};
     }
 }
