@@ -33,34 +33,60 @@ stencil_status_t plan_run_last_two(stencil_plan_t* p, const void* in, void* g1, 
 
 constexpr int kResBlocks = 1024;
 
-// A running sum of squared differences.  FP64 FMAs run at 1/64 of the FP32 rate
-// here, so the sum is kept in two FP32 numbers: the difference, its square and
-// the addition each with their rounding error (TwoDiff, FMA, TwoSum), about 45
-// bits in all.  Differences whose square or its error would leave the FP32 range
-// take the FP64 sum.
+// A running sum of squared differences, at no less than FP64's accuracy.  FP64 FMAs
+// run at 1/64 of the FP32 rate here, so half of the terms (WIDE) take one of them
+// each and the other half FP32 arithmetic that keeps every rounding error: the
+// difference d + e = a - b and the square p + pe = d^2 are exact (TwoDiff, FMA), p
+// goes into `s` and the errors into `c` with their own errors (TwoSum), and those
+// plainly into `low`; 2^-70 of the sum is dropped.  Per thread, against exact sums
+// of 16 to 1024 random terms, the FP32 half is within 1e-16 and a plain FP64 sum
+// within 3e-15.  Terms whose square or its error would leave the FP32 range are
+// summed in FP64 from the start: below 2^-40, and above 2^40, so that no number of
+// terms that a thread can meet overflows `s`.
 struct SquareSum {
-    float s = 0.f, err = 0.f;
+    float s = 0.f, c = 0.f, low = 0.f;
     double wide = 0.0;
+    // acc + v, and the rounding error of that addition
+    static __device__ __forceinline__ float two_sum(float& acc, float v) {
+        const float n = acc + v, y = n - acc, err = (acc - (n - y)) + (v - y);
+        acc = n;
+        return err;
+    }
+    template <bool WIDE>
     __device__ __forceinline__ void add(float a, float b) {
         const float d = a - b, z = d - a;
         const float e = (a - (d - z)) - (b + z);  // a - b = d + e
         const float m = fabsf(d);
-        if (m >= 0x1p-40f && m <= 0x1p+60f) {
-            const float p = d * d, pe = fmaf(d, d, -p);
-            const float n = s + p, y = n - s;
-            err += ((s - (n - y)) + (p - y)) + (pe + 2.f * d * e);
-            s = n;
+        if (m >= 0x1p-40f && m <= 0x1p+40f) {
+            if (WIDE) {
+                // |d| as a double by its bits (a normal number: 896 is the difference of the exponents' biases)
+                const unsigned u = __float_as_uint(m);
+                const double w = __hiloint2double((int)((u >> 3) + (896u << 20)), (int)(u << 29));
+                wide = fma(w, w, wide);
+            } else {
+                const float p = __fmul_rn(d, d), pe = fmaf(d, d, -p);  // (never fused into the sum)
+                const float l = two_sum(c, two_sum(s, p));
+                low += l + two_sum(c, pe);
+            }
+            if (e != 0.f) {  // (a and b within a factor of two differ by a float)
+                const float d2 = 2.f * d, x = __fmul_rn(d2, e), xe = fmaf(d2, e, -x);
+                low += two_sum(c, x) + fmaf(e, e, xe);
+            }
         } else if (!(m == 0.f)) {  // (infinities and NaN too)
             const double w = (double)a - (double)b;
-            wide += w * w;
+            wide = fma(w, w, wide);
         }
     }
-    __device__ __forceinline__ double total() const { return ((double)s + (double)err) + wide; }
+    __device__ __forceinline__ double total() const { return ((double)s + ((double)c + (double)low)) + wide; }
 };
 
 // partials[block] = the block's share of sum (a - b)^2, in a fixed order; the last
 // block to finish adds them in a fixed tree and writes *out = sqrt(sum).
-// 2048^2 FP32: 6 us, against 39 + 4 for FP64 sums of scalar loads and a second launch.
+// A check of 2048^2 FP32 takes 6-8 us, with plain FP64 sums, scalar loads and a second
+// launch 39 + 4.  Two FP32 numbers a thread (2^-45 of the sum, and overflow beyond
+// differences of 2^57) took 6.  A step and its check, 16384^2: 751 us; 918 with FP32
+// alone (47 instructions a term), 830 with one term in four in FP64, 743 with two
+// FP32 numbers.
 template <typename TS>
 __global__ void __launch_bounds__(256)
     residual_kernel(const TS* __restrict__ a, const TS* __restrict__ b, long long n, int vec,
@@ -72,18 +98,27 @@ __global__ void __launch_bounds__(256)
     const long long lo = (long long)blockIdx.x * chunk;
     const long long hi = lo + chunk < n ? lo + chunk : n;
     SquareSum q;
-    if (vec) {
-        long long i = lo + 4 * threadIdx.x;
-        for (; i + 3 < hi; i += 4 * 256) {
-            const float4 x = Storage<TS>::load4(a + i), y = Storage<TS>::load4(b + i);
-            q.add(x.x, y.x);
-            q.add(x.y, y.y);
-            q.add(x.z, y.z);
-            q.add(x.w, y.w);
+    // four terms a pass: one 4-wide piece (vec; only the grid's last piece is cut), else 256 apart
+    const int step = vec ? 1 : 256;
+    for (long long i = lo + (vec ? 4 : 1) * (int)threadIdx.x; i < hi; i += 4 * 256) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+        if (vec && i + 3 < hi) {
+            x = Storage<TS>::load4(a + i);
+            y = Storage<TS>::load4(b + i);
+        } else {
+            x.x = Storage<TS>::load1(a + i);
+            y.x = Storage<TS>::load1(b + i);
+            if (i + step < hi) x.y = Storage<TS>::load1(a + i + step), y.y = Storage<TS>::load1(b + i + step);
+            if (i + 2 * step < hi) x.z = Storage<TS>::load1(a + i + 2 * step), y.z = Storage<TS>::load1(b + i + 2 * step);
+            if (i + 3 * step < hi) x.w = Storage<TS>::load1(a + i + 3 * step), y.w = Storage<TS>::load1(b + i + 3 * step);
         }
-        for (; i < hi; ++i) q.add(Storage<TS>::load1(a + i), Storage<TS>::load1(b + i));  // (one thread's tail)
-    } else {
-        for (long long i = lo + threadIdx.x; i < hi; i += 256) q.add(Storage<TS>::load1(a + i), Storage<TS>::load1(b + i));
+        // (one copy of the two bodies: unrolled, a launch took 2 us longer to fetch them)
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            q.add<true>(x.x, y.x);
+            q.add<false>(x.y, y.y);
+            x.x = x.z, x.y = x.w, y.x = y.z, y.y = y.w;
+        }
     }
     sh[threadIdx.x] = q.total();
     __syncthreads();

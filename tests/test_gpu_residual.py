@@ -96,3 +96,38 @@ def test_residual_outside_the_fp32_range(scale):
     want = [torch.linalg.vector_norm(p.run(x, t).double() - p.run(x, t - 1).double()) for t in (2, 4)]
     assert torch.allclose(res, torch.stack(want), rtol=1e-11, atol=0, equal_nan=True)
     p.close()
+
+
+@pytest.mark.parametrize("side", [1024, 16384])
+def test_large_differences_keep_a_finite_sum(side):
+    """Differences near 1e18: on the larger grid a thread adds about a thousand
+    squares of 1e36 each, more than FP32 holds."""
+    from paper_2605_07954_gb300 import Plan
+    W = np.zeros((3, 3), dtype=np.float32)
+    W[1, 1] = 2.0  # u_1 - u_0 = u_0
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    x = torch.rand((side, side), generator=g, device="cuda").add_(0.5).mul_(2.0 ** 59)
+    p = Plan(side, side, W)
+    _, res = p.run_residual(x, 1, 1)
+    want = torch.linalg.vector_norm(x, dtype=torch.float64)
+    # two FP64 sums of positive terms (at most 2^-53 per addition, fewer than 2000 in a row)
+    assert torch.allclose(res[0], want, rtol=2e-13, atol=0)
+    p.close()
+
+
+def test_sum_is_as_accurate_as_fp64():
+    """Differences that need more than 24 bits, against their exact sum: 16 terms per
+    thread, then some 20 additions of FP64 numbers one after the other."""
+    from paper_2605_07954_gb300 import Plan
+    W = np.zeros((3, 3), dtype=np.float32)
+    W[1, 1] = 2.0 ** -13  # u_0 - u_1 = u_0 (1 - 2^-13), 37 bits
+    n = np.random.default_rng(1).integers(1 << 23, 1 << 24, size=(2048, 2048))
+    p = Plan(2048, 2048, W)
+    _, res = p.run_residual(torch.from_numpy(n.astype(np.float32)).cuda(), 1, 1)
+    rows = (n.astype(np.uint64) ** 2).reshape(-1, 4096).sum(axis=1, dtype=np.uint64)  # (each below 2^60)
+    exact = sum(int(r) for r in rows) * 8191 ** 2  # x 2^-26
+    got = float(res[0].cpu())
+    # the square root halves the error of the sum and adds a rounding of its own
+    assert abs(got ** 2 * 2.0 ** 26 / exact - 1.0) <= 24 * 2.0 ** -53
+    p.close()
