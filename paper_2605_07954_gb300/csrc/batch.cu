@@ -260,6 +260,7 @@ __global__ void __launch_bounds__(32, batch_warp_min_blocks(K))
             }
         }
         if (__any_sync(0xffffffffu, it < 0)) break;
+        __syncwarp();  // (a vote orders no memory) every lane's reads follow all the acquires above
         StreamParams p;
         p.in = g.buf[item.z & 1];
         p.out = g.buf[(item.z + 1) & 1];

@@ -199,3 +199,32 @@ def test_periodic_grids_of_many_tiles(name):
         for i, g in enumerate(grids):
             assert torch.equal(g["out"], _single(g["x"], W, 24, "periodic")), i
     b.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+def test_one_warp_tiles_read_what_their_neighbours_wrote(dtype):
+    """Many low one-warp tiles, each block of steps reading rows that up to eight
+    other SMs wrote in the block before: every run has the bits of a streaming
+    plan that rounds after the same 8 steps (16-bit rows are read through L1)."""
+    from paper_2605_07954_gb300 import Batch, Plan
+    td = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}[dtype]
+    grids, want = [], []
+    for i, (ny, nx, kind) in enumerate([(1200, 1000, "box9"), (1500, 340, "heat5r"), (900, 2048, "heat5r"),
+                                        (333, 777, "box9")]):
+        W = inputs.batch_grid_weights(kind, i)
+        x = torch.from_numpy(inputs.field(ny, nx, stream=40 + i)).cuda().to(td)
+        grids.append(dict(x=x, out=torch.empty_like(x), weights=W, T=160))
+        p = Plan(ny, nx, W, dtype=dtype, kernel="stream", tb_depth=8, threads=128)
+        want.append(p.run(x, 160))
+        torch.cuda.synchronize()
+        p.close()
+    b = Batch(grids, dtype=dtype, tb_depth=8, tile_rows=12)
+    assert b.info()["threads"] == 32
+    for _ in range(10):
+        for g in grids:
+            g["out"].zero_()
+        b.run()
+        torch.cuda.synchronize()
+        b.status()
+        assert all(torch.equal(g["out"], w) for g, w in zip(grids, want))
+    b.close()
