@@ -188,7 +188,8 @@ class _PlanCache:
         if plan is None:
             plan = Plan(ny, nx, W, boundary=boundary)
             while len(self.plans) >= self.size:
-                self.plans.pop(next(iter(self.plans))).close()
+                # (not closed here: a backward pass may still hold it; its last owner frees it)
+                self.plans.pop(next(iter(self.plans)))
         else:
             plan.set_weights(W)
         self.plans[key] = plan  # most recently used last
