@@ -9,6 +9,7 @@ current stream.  ``_capi`` holds the raw C entry points under their C names;
 from __future__ import annotations
 
 import ctypes
+import threading
 
 import numpy as np
 
@@ -49,6 +50,7 @@ class Plan:
         self.shape = (int(ny), int(nx))
         self.dtype = dtype
         self.weights = w
+        self.lock = threading.Lock()  # for threads that set the weights and enqueue a run with them
         opt = _capi.stencil_options_t(COMPUTES[compute], KERNELS[kernel], int(tb_depth),
                                       int(threads), int(tile_rows), int(bool(autotune)), int(mma_n),
                                       int(timeout_ms), int(debug_withhold), LOADS[load], int(rank))
@@ -170,30 +172,41 @@ def _adjoint(plan, u0, grad_uT, T, ckpt_interval, entry):
 
 
 class _PlanCache:
-    """Plans for StencilFn, reused across calls: keyed by (device, shape,
-    radius, footprint class, boundary); a hit only replaces the weights
-    (stencil_plan_set_weights), so the workspace, the tuned configuration and
-    the adjoint's checkpoint scratch are allocated once, not per iteration.
-    At most `size` plans are kept (least recently used dropped first)."""
+    """Plans for StencilFn, reused across calls: keyed by (device, stream, shape,
+    radius, footprint class, boundary), so the workspace, the tuned configuration
+    and the adjoint's scratch are allocated once, not per iteration.  A plan serves
+    one stream at a time (its launches share the workspace and the exchange grids),
+    so each stream has its own; calls that are being captured into a graph, where
+    nothing can be allocated, take over another stream's plan if they have none.
+    At most `size` plans are kept per stream and 4 * `size` in all (least recently
+    used dropped first).  The caller sets the weights, under the plan's lock."""
 
     def __init__(self, size: int = 8):
         self.size = size
         self.plans = {}
+        self.lock = threading.Lock()
 
-    def get(self, device: int, ny: int, nx: int, W: np.ndarray, boundary: str) -> Plan:
+    def get(self, device: int, ny: int, nx: int, W: np.ndarray, boundary: str, stream: int = 0,
+            capturing: bool = False) -> Plan:
         r = W.shape[0] // 2
         star = bool(np.all(W[np.arange(W.shape[0]) != r][:, np.arange(W.shape[1]) != r] == 0))
-        key = (device, ny, nx, r, star, boundary)
-        plan = self.plans.pop(key, None)
-        if plan is None:
-            plan = Plan(ny, nx, W, boundary=boundary)
-            while len(self.plans) >= self.size:
+        what = (ny, nx, r, star, boundary)
+        key = (device, stream) + what
+        with self.lock:
+            plan = self.plans.pop(key, None)
+            if plan is None and capturing:
+                other = next((k for k in reversed(self.plans) if k[0] == device and k[2:] == what), None)
+                plan = self.plans.pop(other, None)
+            if plan is None:
+                plan = Plan(ny, nx, W, boundary=boundary)
                 # (not closed here: a backward pass may still hold it; its last owner frees it)
-                self.plans.pop(next(iter(self.plans)))
-        else:
-            plan.set_weights(W)
-        self.plans[key] = plan  # most recently used last
-        return plan
+                mine = [k for k in self.plans if k[:2] == key[:2]]
+                if len(mine) >= self.size:
+                    self.plans.pop(mine[0])
+                while len(self.plans) >= 4 * self.size:
+                    self.plans.pop(next(iter(self.plans)))
+            self.plans[key] = plan  # most recently used last
+            return plan
 
 
 _PLANS = _PlanCache()
@@ -208,17 +221,23 @@ def _stencil_fn():
         apply(u0, weights, T, boundary="zero", ckpt_interval=0): u0 a CUDA FP32
         tensor; weights a (2r+1, 2r+1) tensor on any device (its values are read
         at forward time).  The weight gradient has the weights' dtype and device.
-        Plans come from a small per-process cache (see _PlanCache), so repeated
-        calls with new weights allocate nothing new.  The backward pass uses the
+        Plans come from a small per-process cache (see _PlanCache), one per stream
+        and shape, so repeated calls with new weights allocate nothing new, and
+        calls on several streams or threads run side by side.  The backward pass uses the
         weights of its own forward call, read back from the saved copy.
         """
 
         @staticmethod
         def forward(ctx, u0, weights, T, boundary="zero", ckpt_interval=0):
             W = np.ascontiguousarray(weights.detach().to("cpu", torch.float32).numpy())
-            plan = _PLANS.get(u0.device.index if u0.is_cuda else -1, u0.shape[0], u0.shape[1], W, boundary)
+            on_gpu = u0.is_cuda
+            plan = _PLANS.get(u0.device.index if on_gpu else -1, u0.shape[0], u0.shape[1], W, boundary,
+                              _current_stream_handle() if on_gpu else 0,
+                              on_gpu and torch.cuda.is_current_stream_capturing())
             u0c = u0.detach().contiguous()
-            y = plan.run(u0c, int(T))
+            with plan.lock:
+                plan.set_weights(W)
+                y = plan.run(u0c, int(T))
             ctx.save_for_backward(u0c)
             ctx.plan, ctx.W, ctx.T, ctx.ckpt = plan, W, int(T), int(ckpt_interval)
             ctx.wdtype, ctx.wdevice = weights.dtype, weights.device
@@ -227,10 +246,11 @@ def _stencil_fn():
         @staticmethod
         def backward(ctx, grad_y):
             (u0,) = ctx.saved_tensors
-            # another forward call may have changed the cached plan's weights
-            ctx.plan.set_weights(ctx.W)
             entry = "stencil_adjoint" if ctx.wdtype == torch.float64 else "stencil_adjoint_w32"
-            g_u0, g_w = _adjoint(ctx.plan, u0, grad_y.contiguous(), ctx.T, ctx.ckpt, entry)
+            with ctx.plan.lock:
+                # another forward call may have changed the cached plan's weights
+                ctx.plan.set_weights(ctx.W)
+                g_u0, g_w = _adjoint(ctx.plan, u0, grad_y.contiguous(), ctx.T, ctx.ckpt, entry)
             return g_u0, g_w.to(ctx.wdevice, ctx.wdtype), None, None, None
 
     return StencilFn

@@ -36,3 +36,29 @@ def test_a_dropped_plan_stays_usable_for_its_holders(cache):
     assert len(cache.plans) == 3 and held not in cache.plans.values()
     gc.collect()
     assert not held.closed
+
+
+def test_every_stream_has_its_own_plans(cache):
+    """A plan's launches share its workspace and exchange grids, so two streams never share a plan."""
+    a = cache.get(0, 10, 10, W3, "zero", stream=1)
+    b = cache.get(0, 10, 10, W3, "zero", stream=2)
+    assert a is not b
+    assert cache.get(0, 10, 10, W3, "zero", stream=1) is a
+    assert cache.get(0, 10, 10, W3, "periodic", stream=2) is not b
+    # one stream's many shapes do not push out another's
+    for n in range(20, 30):
+        cache.get(0, n, n, W3, "zero", stream=2)
+    assert cache.get(0, 10, 10, W3, "zero", stream=1) is a
+    assert len(cache.plans) == 1 + 3
+    # and many streams are bounded as well
+    for s in range(3, 40):
+        cache.get(0, 10, 10, W3, "zero", stream=s)
+    assert len(cache.plans) == 4 * 3
+
+
+def test_a_captured_call_allocates_nothing(cache):
+    """A call under capture takes over the plan that a warm-up on another stream made."""
+    a = cache.get(0, 10, 10, W3, "zero", stream=1)
+    assert cache.get(0, 10, 10, W3, "zero", stream=9, capturing=True) is a
+    assert cache.get(0, 10, 10, W3, "zero", stream=9) is a
+    assert cache.get(0, 10, 10, W3, "zero", stream=1) is not a
