@@ -46,6 +46,7 @@ namespace gbst {
 void plan_weights(const stencil_plan_t* p, float* w);
 void** plan_aux_slot(stencil_plan_t* p, int id);
 void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*));
+void plan_set_stream(stencil_plan_t* p, cudaStream_t st);
 bool plan_keep_sums(stencil_plan_t* p, bool on);
 bool plan_states_vary(const stencil_plan_t* p);
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
@@ -824,6 +825,7 @@ stencil_status_t adjoint_run(stencil_plan_t* plan, const void* u0, const void* g
     const size_t n = (size_t)ny * (size_t)nx;
     const size_t bytes = n * sizeof(float);
     cudaStream_t st = (cudaStream_t)stream;
+    plan_set_stream(plan, st);
     Weights wf{};
     plan_weights(plan, wf.w);
     Weights wadj = wf;  // the step kernels index W directly; the flip is in their loops

@@ -159,6 +159,8 @@ void plan_weights(const stencil_plan_t* p, float* w) {
     for (int i = 0; i < kMaxTaps; ++i) w[i] = p->w.w[i];
 }
 void** plan_aux_slot(stencil_plan_t* p, int id) { return &p->aux[id]; }
+// The stream whose work stencil_plan_status waits for.
+void plan_set_stream(stencil_plan_t* p, cudaStream_t st) { p->last_stream = st; }
 void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*)) { p->aux_free[id] = freer; }
 // Whether the bits of a run's states depend on how its steps are grouped into calls.
 bool plan_states_vary(const stencil_plan_t* p) {

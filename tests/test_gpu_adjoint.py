@@ -216,3 +216,22 @@ def test_fullsize_heat_4096_T512_window(oracle):
     rhs = float(torch.dot(x.double().flatten(), ATy.double().flatten()))
     assert abs(lhs - rhs) <= 1e-5 * abs(lhs)
     p.close()
+
+
+@pytest.mark.parametrize("entry", ["stencil_adjoint", "stencil_adjoint_w32"])
+def test_status_waits_for_the_adjoint(entry):
+    """A wait that runs out in the recomputed states is reported by a status call right
+    after the adjoint, with no other synchronisation: the plan's first call, on a stream
+    that does not wait for the default one."""
+    from paper_2605_07954_gb300 import Plan, StencilError, _adjoint
+    W = inputs.heat_weights(0.2)
+    x = torch.from_numpy(inputs.field(1000, 1000)).cuda()
+    p = Plan(1000, 1000, W, timeout_ms=100, debug_withhold=1)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        _adjoint(p, x, x, 40, 0, entry)
+        with pytest.raises(StencilError, match="TIMEOUT"):
+            p.status()
+        p.status()  # (the word was cleared, by the time the launch had ended)
+    p.close()
