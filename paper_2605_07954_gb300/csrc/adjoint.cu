@@ -117,6 +117,9 @@ __global__ void __launch_bounds__(kAdrWarps * 32, 2)
     const int yb = ((int)blockIdx.x / tiles_x) * (kAdrWarps * kAdrRows) + warp * kAdrRows;
     const bool per = periodic != 0;
     const bool own = lane >= 1 && lane <= 30 && c < nx;
+    bool live[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) live[e] = c + e < nx;
     float win[D][E];
     float g[2][D * D];
 #pragma unroll
@@ -172,7 +175,8 @@ __global__ void __launch_bounds__(kAdrWarps * 32, 2)
                     for (int e = 0; e < 4; ++e) {
                         const float l = win[R - dy][R + e - dx];
                         if (!STAR || dy == 0 || dx == 0) acc[e] = fmaf(w.w[t], l, acc[e]);
-                        g[j][t] = fmaf(uu[e], l, g[j][t]);
+                        // (a column beyond the grid has no term, not a zero one: lambda may be infinite)
+                        if (live[e]) g[j][t] = fmaf(uu[e], l, g[j][t]);
                     }
                 }
             if (own) {
@@ -188,9 +192,10 @@ __global__ void __launch_bounds__(kAdrWarps * 32, 2)
         }
     }
     // Fixed order: thread (tap, half) adds the 64 sums of two warps, sum and rounding
-    // error apart.
+    // error apart; where that leaves the FP32 range, once more in FP64.  (Lanes that own
+    // no columns have multiplied zeros by neighbours' lambdas, which may be infinite.)
 #pragma unroll
-    for (int k = 0; k < D * D; ++k) sums[k][threadIdx.x] = g[0][k] + g[1][k];
+    for (int k = 0; k < D * D; ++k) sums[k][threadIdx.x] = own ? g[0][k] + g[1][k] : 0.f;
     __syncthreads();
     for (int t = threadIdx.x; t < 2 * D * D; t += kAdrWarps * 32) {
         const int k = t % (D * D), h = t / (D * D);
@@ -200,7 +205,11 @@ __global__ void __launch_bounds__(kAdrWarps * 32, 2)
             err += (s - (n - z)) + (v - z);
             s = n;
         }
-        const double d = (double)s + (double)err;
+        double d = (double)s + (double)err;
+        if (!(fabs(d) <= 3.5e38)) {
+            d = 0.0;
+            for (int i = 0; i < 64; ++i) d += (double)sums[k][64 * h + i];
+        }
         if (h) half[k] = d;
         else partials[(size_t)blockIdx.x * D * D + k] += d;
     }

@@ -82,3 +82,31 @@ def test_fp64_sums_keep_their_bits(name, shape, boundary):
     assert np.array_equal(np.asarray(ra.cpu() if hasattr(ra, "cpu") else ra),
                           np.asarray(rb.cpu() if hasattr(rb, "cpu") else rb))
     assert p.info() == info and torch.equal(p.run(x, 9), y)
+
+
+@pytest.mark.parametrize("name", ["star9", "star13", "box49"])
+@pytest.mark.parametrize("boundary,nx", [("zero", 361), ("periodic", 361), ("periodic", 364)])
+@pytest.mark.parametrize("col", [117, 119, 120, 122, 239, 240, 355, 360])
+def test_an_infinite_lambda_gives_infinite_sums(name, boundary, nx, col):
+    """One infinite lambda times positive u: every tap's sum is infinite, not NaN, next
+    to the columns where a warp's strip ends and beside the grid's last column too."""
+    if boundary == "zero" and col + 3 >= nx:
+        col = nx - 4  # (nearer the edge the term u~ = 0 beyond it is 0 x inf)
+    W = _weights(name)
+    u0 = inputs.field(200, nx) + np.float32(0.5)
+    gT = np.zeros((200, nx), dtype=np.float32)
+    gT[100, col] = np.inf
+    for entry in ("stencil_adjoint_w32", "stencil_adjoint"):
+        _, gw = _grads(u0, W, 1, gT, boundary, entry)
+        assert np.all(np.isposinf(gw)), entry
+
+
+@pytest.mark.parametrize("name", ["star9", "star13", "box49"])
+def test_sums_beyond_fp32_stay_finite(name):
+    """Lambdas of 1e36: the sums of 128 lanes leave the FP32 range, their FP64 sum does not."""
+    W = _weights(name)
+    u0 = inputs.field(200, 362) + np.float32(0.5)
+    gT = np.full((200, 362), 1e36, dtype=np.float32)
+    _, gw = _grads(u0, W, 1, gT, "periodic", "stencil_adjoint_w32")
+    _, ref = _grads(u0, W, 1, gT, "periodic", "stencil_adjoint")
+    assert np.all(np.isfinite(gw)) and rel_l2(gw / 1e36, ref / 1e36) <= 1e-5
