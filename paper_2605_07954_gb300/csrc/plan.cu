@@ -779,6 +779,8 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
             cudaGetLastError();
             p->grid_on = p->grid_ok = 0;
             p->kernel = STENCIL_KERNEL_STREAM;
+            const int C = p->grid.plain ? resident_candidates(p) : 0;  // (the kernel the tiles stood in for)
+            if (C > 0) use_resident(p, C);
             return fail(STENCIL_ERR_UNSUPPORTED, "the chip-resident tiles do not fit at once");
         }
         CK(e);
@@ -1320,11 +1322,13 @@ static const int kTuneGrid = 1 << 20;
 
 static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaStream_t st) {
     // (plans that asked for the cluster-resident kernel have no chip-resident candidate)
-    const TuneKey key(p->ny, p->nx, p->R + 16 * p->grid_ok, p->star, p->dtype, p->boundary, p->device);
+    auto tune_key = [&] {
+        return TuneKey(p->ny, p->nx, p->R + 16 * p->grid_ok, p->star, p->dtype, p->boundary, p->device);
+    };
     int decision = -1;
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
-        auto it = g_res_tune_cache.find(key);
+        auto it = g_res_tune_cache.find(tune_key());
         if (it != g_res_tune_cache.end()) decision = it->second;
     }
     if (decision < 0) {
@@ -1360,7 +1364,8 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
         if (p->grid_ok) {
             use_grid(p);
             stencil_status_t s = try_resident(kTuneGrid);
-            if (s != STENCIL_OK) return s;
+            // (a partition too small for the tiles, which launch_once then rules out: the others are left)
+            if (s != STENCIL_OK && !(s == STENCIL_ERR_UNSUPPORTED && !p->grid_ok)) return s;
         }
         for (int lg = 0; (1 << lg) <= resident_max_cluster(); ++lg) {
             if (!((p->res_ok >> lg) & 1)) continue;
@@ -1383,7 +1388,7 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
         if (s != STENCIL_OK) return s;
         if (ms / (float)(sreps * p->k) < best) decision = 0;
         std::lock_guard<std::mutex> g(g_tune_mu);
-        g_res_tune_cache[key] = decision;
+        g_res_tune_cache[tune_key()] = decision;  // (for the candidates that there were)
     }
     if (decision == kTuneGrid) {
         use_grid(p);
@@ -1754,9 +1759,10 @@ stencil_status_t stencil_run(stencil_plan_t* p, const void* in, void* out, int64
     if (p->kernel == STENCIL_KERNEL_RESIDENT) {
         // one launch reads all of its input before it writes any output
         for (size_t i = 0; i < depths.size(); ++i) {
+            const bool tiles = p->grid_on;
             stencil_status_t s = launch_once(p, src, out, depths[i], st);
-            if (s == STENCIL_ERR_UNSUPPORTED && p->kernel == STENCIL_KERNEL_STREAM) {
-                // (nothing was launched: the streaming kernel takes the run)
+            if (s == STENCIL_ERR_UNSUPPORTED && tiles && !p->grid_on) {
+                // (nothing was launched: the kernel that launch_once put in its place takes the run)
                 return stencil_run(p, src == p->ws ? in : src, out, T - (int64_t)i * (1 << 30), stream);
             }
             if (s != STENCIL_OK) return s;
