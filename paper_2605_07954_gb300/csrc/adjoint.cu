@@ -49,6 +49,8 @@ void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*));
 void plan_set_stream(stencil_plan_t* p, cudaStream_t st);
 bool plan_keep_sums(stencil_plan_t* p, bool on);
 bool plan_states_vary(const stencil_plan_t* p);
+bool plan_states_one_launch(const stencil_plan_t* p, bool any_order);
+int64_t plan_sum_launches(const stencil_plan_t* p, int64_t T);
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
                                  cudaStream_t st);
 
@@ -953,23 +955,23 @@ stencil_status_t stencil_adjoint_w32(stencil_plan_t* plan, const void* u0, const
 int64_t stencil_adjoint_launches(const stencil_plan_t* plan, int64_t T, int64_t ckpt_interval) {
     if (!plan || T < 0 || ckpt_interval < 0) return -1;
     if (T == 0) return 0;
-    const KeepSums kept(const_cast<stencil_plan_t*>(plan), true);
     stencil_plan_info_t info{};
     const bool fused = stencil_plan_info(plan, &info) == STENCIL_OK && info.dtype == STENCIL_F32 &&
                        info.nx % 4 == 0;
-    const int64_t sgm = adj_interval(T, ckpt_interval, info.radius, (size_t)info.ny * (size_t)info.nx * sizeof(float), plan_states_vary(plan));
+    const int64_t sgm = adj_interval(T, ckpt_interval, info.radius,
+                                     (size_t)info.ny * (size_t)info.nx * sizeof(float), plan_states_vary(plan));
     const int64_t nseg = (T + sgm - 1) / sgm;
-    int64_t L = (nseg - 1) * stencil_run_launches(plan, sgm);  // checkpoints
-    const bool resident = info.kernel == STENCIL_KERNEL_RESIDENT && !plan_states_vary(plan) && info.ctas == 1 && info.threads != 1024 &&
-                          !(info.boundary == STENCIL_BOUNDARY_PERIODIC && info.nx % 4 != 0);
+    int64_t L = (nseg - 1) * plan_sum_launches(plan, sgm);  // checkpoints
+    const bool one = plan_states_one_launch(plan, false);
+    const int64_t step = fused ? 0 : plan_sum_launches(plan, 1);
     for (int64_t j = 0; j < nseg; ++j) {  // segment recompute: all-states launches of 8/4/2/1 steps
         int64_t m = std::min<int64_t>(sgm, T - j * sgm) - 1;
-        if (resident) {  // (register tiles: one launch)
+        if (one) {  // (register tiles)
             L += m > 0;
             continue;
         }
         if (!fused) {
-            L += m * stencil_run_launches(plan, 1);
+            L += m * step;
             continue;
         }
         const int top = info.radius == 3 && !info.shape ? 2 : (info.radius == 1 ? 8 : 4);

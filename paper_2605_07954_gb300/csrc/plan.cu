@@ -1051,14 +1051,25 @@ bool plan_keep_sums(stencil_plan_t* p, bool on) {
     return true;
 }
 
+// stencil_run_launches(p, T) in the form that plan_keep_sums gives the plan for such a call.
+int64_t plan_sum_launches(const stencil_plan_t* p, int64_t T) {
+    stencil_plan q = *p;  // (the caller's plan stays as it is: another thread may be running it)
+    plan_keep_sums(&q, true);
+    return stencil_run_launches(&q, T);
+}
+
+// Chip-resident plans: every state in one launch (13-point star 1000 x 1022: a
+// single-step launch per state took 13 us each).  Not for periodic ragged widths,
+// whose bits depend on how the steps are grouped, and in the streaming kernel's
+// summation order only (any_order: any will do).
+bool plan_states_one_launch(const stencil_plan_t* p, bool any_order) {
+    return p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && (any_order || !p->grid.plain) &&
+           p->dtype == STENCIL_F32 && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0);
+}
+
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
                                  cudaStream_t st) {
-    // Chip-resident plans: every state in one launch (13-point star 1000 x 1022: a
-    // single-step launch per state took 13 us each).  Not for periodic ragged widths,
-    // whose bits depend on how the steps are grouped, and in the streaming kernel's
-    // summation order only (any_order: any will do).
-    bool strided = p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && (any_order || !p->grid.plain) && p->dtype == STENCIL_F32 && n >= 1 &&
-                   n < (1 << 30) && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0);
+    bool strided = plan_states_one_launch(p, any_order) && n >= 1 && n < (1 << 30);
     const int64_t stride = n > 1 ? outs[1] - outs[0] : 0;
     for (int64_t i = 1; i < n && strided; ++i) strided = outs[i] - outs[i - 1] == stride;
     if (strided) {

@@ -235,3 +235,33 @@ def test_status_waits_for_the_adjoint(entry):
             p.status()
         p.status()  # (the word was cleared, by the time the launch had ended)
     p.close()
+
+
+def test_counting_launches_leaves_the_plan_alone():
+    """stencil_adjoint_launches only asks: runs of the plan in another thread meanwhile
+    keep their kernel (and, on periodic ragged widths, their bits)."""
+    import threading
+    from paper_2605_07954_gb300 import Plan, _capi
+    W = inputs.heat_weights(0.2)
+    x = torch.from_numpy(inputs.field(999, 1001)).cuda()
+    p = Plan(999, 1001, W, boundary="periodic")
+    want = p.run(x, 8)
+    count = _capi.load().stencil_adjoint_launches
+    n = count(p.handle, 400, 0)
+    assert n == count(Plan(999, 1001, W, boundary="periodic", kernel="stream").handle, 400, 0)
+    # one launch for the states, one per reverse step, one reduction
+    assert count(Plan(1000, 1000, W).handle, 32, 0) == 1 + 32 + 1
+    done = threading.Event()
+
+    def ask():
+        while not done.is_set():
+            count(p.handle, 400_000, 2)
+
+    t = threading.Thread(target=ask)
+    t.start()
+    try:
+        for _ in range(200):
+            assert torch.equal(p.run(x, 8), want)
+    finally:
+        done.set()
+        t.join()
