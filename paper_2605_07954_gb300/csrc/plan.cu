@@ -66,7 +66,7 @@ int resident_threads();
 int resident_max_cluster();
 int resident_config(int ny, int nx, int radius, int periodic, int C, int kb, int max_smem, int* rp_out);
 cudaError_t launch_resident(const void* fn, int C, int smem, const ResidentParams& prm, cudaStream_t st);
-bool resident_cluster_fits(const void* fn, int C, int smem);
+bool resident_cluster_fits(const void* fn, int C, int smem, int max_smem);
 struct TcParams {  // must match box49_tc.cu
     const void* in;
     void* out;
@@ -543,7 +543,7 @@ static int resident_candidates(stencil_plan* p, int kb = 1) {
         int rp = 0;
         const int smem = resident_config((int)p->ny, (int)p->nx, p->R, periodic, C, kb, max_smem, &rp);
         if (smem < 0) continue;
-        if (!resident_cluster_fits(fn, C, smem)) continue;
+        if (!resident_cluster_fits(fn, C, smem, max_smem)) continue;
         int lg = 0;
         while ((1 << lg) < C) ++lg;
         p->res_ok |= 1 << lg;
@@ -561,7 +561,8 @@ static stencil_status_t use_resident(stencil_plan* p, int C, int kb = 1) {
     int rp = 0;
     const int smem = resident_config((int)p->ny, (int)p->nx, p->R, periodic, C, kb, p->res_max_smem, &rp);
     if (smem < 0) return fail(STENCIL_ERR_UNSUPPORTED, "grid does not fit the cluster-resident kernel");
-    CK(cudaFuncSetAttribute(p->res_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // (the kernel's limit, which all plans share: the largest any of them may need)
+    CK(cudaFuncSetAttribute(p->res_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->res_max_smem));
     if (C > 8) CK(cudaFuncSetAttribute(p->res_fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     p->kernel = STENCIL_KERNEL_RESIDENT;
     p->grid_on = 0;

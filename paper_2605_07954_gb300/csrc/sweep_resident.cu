@@ -292,9 +292,10 @@ cudaError_t launch_resident(const void* fn, int C, int smem, const ResidentParam
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-// Whether a cluster of C CTAs with `smem` bytes each can be scheduled.
-bool resident_cluster_fits(const void* fn, int C, int smem) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+// Whether a cluster of C CTAs with `smem` bytes each can be scheduled.  (The kernel's
+// shared-memory limit is set to `max_smem`, whatever `smem` is: plans share it.)
+bool resident_cluster_fits(const void* fn, int C, int smem, int max_smem) {
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }

@@ -163,3 +163,17 @@ def test_blocked_exchange_depths(oracle, name, kb, boundary):
     a, _, _ = _run(u0, W, 3 * kb + 1, boundary, kernel="resident", tb_depth=kb)
     b, _, _ = _run(u0, W, 3 * kb + 1, boundary, kernel="resident")
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("big,small", [((600, 600), (64, 64)), ((200, 1500), (100, 100))])
+def test_a_smaller_plan_leaves_a_larger_one_usable(big, small):
+    """All plans of one footprint share a kernel, and so its shared-memory limit."""
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights("heat5")
+    x = torch.from_numpy(inputs.field(*big)).cuda()
+    p = Plan(*big, W, kernel="resident")
+    y = p.run(x, 9)
+    others = [Plan(*small, W, kernel="resident"), Plan(*small, W), Plan(*small, W, autotune=True)]
+    for q in others:
+        q.run(torch.from_numpy(inputs.field(*small)).cuda(), 9)
+        assert torch.equal(p.run(x, 9), y)
