@@ -124,7 +124,9 @@ stencil_status_t launch_depth(const Geometry& g, const StreamParams& base, int R
     StreamKernelRef r = kernel_for(R, star, depth, dtype, sp.vec);
     if (!r.fn) return nfail(STENCIL_ERR_UNSUPPORTED, "no streaming kernel for this depth");
     const int smem = stream_smem_bytes(R, depth, elem, sp.vec != 0, false, g.nt);
-    NCK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // (the largest CTA's, as plans set it: the limit is the kernel's, not the launch's)
+    NCK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             stream_smem_bytes(R, depth, elem, sp.vec != 0, false, kStreamMaxThreads)));
     void* args[] = {&sp};
     NCK(cudaLaunchKernel(r.fn, dim3((unsigned)(g.strips * g.tiles_y)), dim3((unsigned)g.nt), args,
                          (size_t)smem, st));
@@ -201,7 +203,8 @@ stencil_status_t stencil_run_noalloc(int64_t ny, int64_t nx, int radius, const f
         StreamKernelRef r = kernel_for(radius, star, k, dtype, vec);
         if (!r.fn) return nfail(STENCIL_ERR_UNSUPPORTED, "no streaming kernel for this shape");
         const int smem = stream_smem_bytes(radius, k, elem, vec != 0, false, g.nt);
-        NCK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        NCK(cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 stream_smem_bytes(radius, k, elem, vec != 0, false, kStreamMaxThreads)));
         NCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.fn, g.nt, smem));
     }
     if (per_sm < 1) return nfail(STENCIL_ERR_UNSUPPORTED, "streaming kernel does not fit on an SM");

@@ -146,3 +146,15 @@ def test_noalloc_rejects_grids_beyond_the_scratch(lib):
                                  0, 0, x.data_ptr(), x.data_ptr(), 1, None)
     assert st == 2  # STENCIL_ERR_UNSUPPORTED
     assert "exceeds" in lib.stencil_noalloc_last_error().decode()
+
+
+@pytest.mark.parametrize("name", ["heat5", "box9", "star13", "box49"])
+def test_noalloc_leaves_plans_usable(lib, name):
+    """A narrow no-alloc sweep runs the kernels of plans with wide CTAs, whose shared-memory limit they share."""
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights(name)
+    x = torch.from_numpy(inputs.field(300, 1200)).cuda()
+    p = Plan(300, 1200, W, kernel="stream", threads=256)
+    y = p.run(x, 17)
+    _noalloc(lib, torch.from_numpy(inputs.field(40, 12)).cuda(), W, 17)
+    assert torch.equal(p.run(x, 17), y)
