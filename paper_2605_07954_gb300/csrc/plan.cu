@@ -310,6 +310,13 @@ static StreamKernelRef pad_kernel(const stencil_plan* p, int k) {
 // 4096^2 (64-row tiles, NC = 4; NC = 8: 389) 397 | 473, 3500^2 (47 rows) 317 |
 // 338, 3000^2 (34 rows) 312 | 281; 9-point box 16384^2 6712 | 6901, 8192^2 1796 |
 // 1827, 4096^2 561 | 576, 3500^2 439 | 445, 3000^2 476 | 363.
+// NC = 8 needs widths that are a multiple of 8: where the right edge cuts a lane's
+// chunk, the checks of those tiles set the time of the whole wave.  5-point star,
+// NC = 8 | NC = 4 | CTA-wide: 8191 x 8188 1459 | 1260 | 1272, 6600 x 7012 1062 | 901 |
+// 933, 16383^2 5668 | 5122 | 5468; BF16 8191^2 1428 | 1263 | 1375, 12000 x 9001 2154 |
+// 1909 | 2108; periodic 8192 x 8188 1444 | 1307 | 1372.  16-bit storage gains as FP32
+// does: BF16 4096^2 359 | 439 (star), 544 | 569 (box), 8192^2 955 | 1208, 1746 | 1799,
+// periodic 1012 | 1225, 1768 | 1801, 4001 x 5003 459 | 528, 671 | 692.
 static bool pad_eligible(const stencil_plan* p);
 constexpr int kWarpDepth = 8;
 constexpr int kWarpMinRows = 44;      // NC = 4
@@ -337,6 +344,7 @@ static void configure_warp(stencil_plan* p, int threads_asked) {
         o.load != STENCIL_LOAD_AUTO || threads_asked != default_threads(p->R, p->star))
         return;
     for (int nc = p->star ? 8 : 4; nc >= 4; nc -= 4) {
+        if (nc == 8 && p->nx % 8 != 0) continue;
         const WarpTiles t = warp_tiles(p, nc);
         if (t.by < (nc == 8 ? kWarpMinRowsWide : kWarpMinRows)) continue;
         p->warp_nc = nc;

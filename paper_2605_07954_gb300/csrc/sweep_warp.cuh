@@ -252,7 +252,7 @@ __device__ __forceinline__ void warp_tile(const StreamParams& p, const WarpWeigh
 __host__ __device__ constexpr int warp_min_blocks(int NC) { return NC == 8 ? 8 : 16; }
 
 // A launch of one-warp CTAs over a whole grid: p.strips x tile rows, edge tiles first.
-// (ALL kernels take widths that are a multiple of NC.)
+// (ALL and NC = 8 kernels take widths that are a multiple of NC.)
 template <bool STAR, int K, typename TS, int NC, bool ALL = false>
 __global__ void __launch_bounds__(32, warp_min_blocks(NC)) sweep_warp_kernel(const __grid_constant__ StreamParams p) {
     __shared__ __align__(16) char ring[warp_ring_bytes<TS, NC>()];
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(32, warp_min_blocks(NC)) sweep_warp_kernel(con
     const bool interior = y0 - K >= 0 && ylast + warp_rows_after(K) <= ny && x0 - p.H >= 0 && x0 - p.H + 32 * NC <= nx;
     const WarpWeights<STAR> ws([&](int i) { return p.w.w[i]; });
     if (interior) warp_tile<STAR, K, TS, NC, false, false, ALL>(p, ws, ring, lane, x0, y0);
-    else if (ALL || nx % NC == 0) warp_tile<STAR, K, TS, NC, true, false, ALL>(p, ws, ring, lane, x0, y0);
+    else if (ALL || NC == 8 || nx % NC == 0) warp_tile<STAR, K, TS, NC, true, false, ALL>(p, ws, ring, lane, x0, y0);
     else warp_tile<STAR, K, TS, NC, true, true, ALL>(p, ws, ring, lane, x0, y0);
 }
 

@@ -44,3 +44,20 @@ def test_same_bits_as_cta_wide_kernel(name, dtype, shape, boundary):
             assert torch.equal(z, y), T
     p.close()
     q.close()
+
+
+@pytest.mark.parametrize("nx,columns", [(8192, 8), (8188, 4), (8191, 4), (8190, 4)])
+def test_wide_chunks_only_where_no_chunk_is_cut(nx, columns):
+    """8 columns a lane for the 5-point star on widths that are a multiple of 8, else 4
+    (tiles of at most 240 and 112 columns); the bits of the CTA-wide kernel either way."""
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights("heat5")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(6)
+    x = torch.rand((8190, nx), generator=g, device="cuda")
+    p, q = Plan(8190, nx, W), Plan(8190, nx, W, threads=128)
+    i = p.info()
+    assert i["threads"] == 32 and (112 < i["tile_cols"] <= 240) == (columns == 8), i
+    assert torch.equal(p.run(x, 17), q.run(x, 17))
+    p.close()
+    q.close()
