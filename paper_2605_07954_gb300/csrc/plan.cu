@@ -36,7 +36,7 @@ StreamKernelRef get_stream_pad_kernel_f32(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_bf16(int R, int star, int k);
 StreamKernelRef get_stream_pad_kernel_f16(int R, int star, int k);
 const void* get_warp_kernel(int star, int dtype, int nc);
-const void* get_warp_states_kernel(int star);
+const void* get_warp_states_kernel();
 StreamKernelRef get_stream_tma_kernel_r1(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r2(int star, int k);
 StreamKernelRef get_stream_tma_kernel_r3(int star, int k);
@@ -975,9 +975,11 @@ static std::vector<int> launch_depths(const stencil_plan* p, int64_t T) {
 
 // One all-states launch of d steps: level l+1 to outs[l] (null: not stored, but the last must be).
 static stencil_status_t launch_states(stencil_plan_t* p, const void* src, float* const* outs, int d, cudaStream_t st) {
-    if (d == kWarpDepth && p->R == 1) {
-        // one-warp tiles where they have enough rows (4096^2 5-point star: 123 us
-        // per launch, 153 CTA-wide)
+    if (d == kWarpDepth && p->R == 1 && p->star) {
+        // one-warp tiles for the 5-point star where they have enough rows (4096^2: 123 us
+        // per launch, 153 CTA-wide).  Not the 9-point box, whose levels' stores spill
+        // there: gradients of 18 steps with 8 states a segment, one-warp | CTA-wide, us:
+        // 4096^2 1188 | 1141, 7567 x 3036 1722 | 1614, 8192^2 4267 | 4178.
         const WarpTiles t = warp_tiles(p, 4);
         if (t.by >= kWarpMinRows) {
             StreamParams sp = stream_params(p, d);
@@ -990,7 +992,7 @@ static stencil_status_t launch_states(stencil_plan_t* p, const void* src, float*
             sp.vec = 1;
             for (int l = 0; l < d - 1; ++l) sp.lvl_out[l] = outs[l];
             void* args[] = {&sp};
-            CK(cudaLaunchKernel(get_warp_states_kernel(p->star), dim3((unsigned)(t.strips * t.tiles)), dim3(32), args, 0,
+            CK(cudaLaunchKernel(get_warp_states_kernel(), dim3((unsigned)(t.strips * t.tiles)), dim3(32), args, 0,
                                 st));
             return STENCIL_OK;
         }

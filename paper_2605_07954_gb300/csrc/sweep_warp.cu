@@ -19,10 +19,7 @@ const void* get_warp_kernel(int star, int dtype, int nc) {
     }
 }
 
-// The same, storing every level (FP32, 4 columns per lane, nx % 4 == 0).
-const void* get_warp_states_kernel(int star) {
-    return star ? (const void*)sweep_warp_kernel<true, 8, float, 4, true>
-                : (const void*)sweep_warp_kernel<false, 8, float, 4, true>;
-}
+// The 5-point star's, storing every level (FP32, 4 columns per lane, nx % 4 == 0).
+const void* get_warp_states_kernel() { return (const void*)sweep_warp_kernel<true, 8, float, 4, true>; }
 
 }  // namespace gbst

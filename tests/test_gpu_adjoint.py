@@ -265,3 +265,19 @@ def test_counting_launches_leaves_the_plan_alone():
     finally:
         done.set()
         t.join()
+
+
+@pytest.mark.parametrize("name", ["heat5", "box9"])
+@pytest.mark.parametrize("shape,boundary", [((4096, 4096), "zero"), ((6000, 3036), "periodic")])
+def test_eight_states_a_launch_have_the_bits_of_four(name, shape, boundary):
+    """Large radius-1 grids: launches that store eight states (one-warp tiles for the star,
+    the CTA-wide kernel for the box) against launches of four and two."""
+    from paper_2605_07954_gb300 import Plan, adjoint
+    W = inputs.pattern_weights(name)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(8)
+    x, gT = (torch.rand(shape, generator=g, device="cuda") for _ in range(2))
+    p = Plan(*shape, W, boundary=boundary)
+    a, b = adjoint(p, x, gT, 18, 9), adjoint(p, x, gT, 18, 7)
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+    p.close()
