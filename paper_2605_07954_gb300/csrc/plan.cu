@@ -602,7 +602,8 @@ static bool grid_candidate(stencil_plan* p) {
     const int periodic = p->boundary == STENCIL_BOUNDARY_PERIODIC;
     if (!grid_config((int)p->ny, (int)p->nx, p->R, p->star, periodic, p->sms, 0, 0, &p->grid)) return false;
     // the cluster-resident kernel's bits where AUTO would otherwise take that kernel
-    p->grid.plain = resident_candidates(p) > 0;
+    const int C = resident_candidates(p);
+    p->grid.plain = C > 0;
     // (boxes of radius 2 and 3 of up to about 140^2 points, where each tile is mostly
     // halo, stay with it: 96 x 100, 7x7 100 steps 129 us against 164, 5x5 16 steps 21
     // against 22; at 160^2 it is 1.2 and 1.3 times as slow, at 400^2 2.4 and 2.6)
@@ -611,6 +612,7 @@ static bool grid_candidate(stencil_plan* p) {
     if (p->dtype != STENCIL_F32 && !p->grid.plain) return false;
     if (p->grid.plain && p->R >= 2 && !p->star && p->ny * p->nx <= 20000) return false;
     p->grid_ok = grid_fits(p->grid, p->R, p->star, p->sms);
+    if (p->grid_ok && C > 0 && use_resident(p, C) != STENCIL_OK) p->res_c = 0;  // (for cluster_run)
     return p->grid_ok != 0;
 }
 
@@ -661,6 +663,41 @@ static bool tiles_launch(const stencil_plan* p, int nlev, bool vec) {
 static void use_grid(stencil_plan* p) {
     p->kernel = STENCIL_KERNEL_RESIDENT;
     p->grid_on = 1;
+}
+
+// Register-tile plans in the cluster-resident kernel's order keep that kernel
+// configured: the bits are the same, so each run takes the faster of the two.
+//
+// One step: the cooperative launch and its end cost ~2 us more than the cluster's, and
+// in place, where a tile may not write before its neighbours have read, the tiles copy
+// the input first (two steps: they exchange after the first).  In us, alone and among
+// others, register tiles | cluster: 5-point star 64^2 16.4 / 6.3 | 14.8 / 5.2, 9-point
+// box 140 x 141 17.7 / 8.2 | 14.4 / 6.3, 13-point star 300 x 110 17.7 / 8.3 | 16.6 / 6.5,
+// 200^2 even; in place, among others, 5-point star 200 x 201 12.1 | 6.9, 256^2 10.4 |
+// 8.3, 300^2 11.4 | 9.4, 7x7 box 300^2 12.4 | 12.4; two steps in place 260 x 161 10.4 |
+// 8.4, 300 x 201 10.4 | 9.2, 200^2 8.8 | 8.3.
+//
+// Periodic ragged widths: the tiles read their halos element by element through the
+// wrap, twice the cost of an exchange, and the more of a tile is halo the worse.
+// 100 steps, register tiles | cluster: 13-point star 60 x 61 192 | 131, 300 x 110
+// 238 | 183, 250 x 251 245 | 216, 300 x 301 290 | 342; 7x7 box 300 x 110 390 | 211,
+// 300 x 201 387 | 271, 300 x 301 395 | 462; 5x5 box 300 x 110 267 | 164, 250 x 251
+// 215 | 193; 9-point star 141^2 152 | 138, 200 x 201 183 | 190; 9-point box 100 x 99
+// 132 | 118, 200 x 201 143 | 197; 5-point star always fewer as tiles, but for short
+// runs: 2 steps 300 x 110 19.7 / 10.3 | 17.9 / 8.4, 3 steps 141^2 18.8 / 10.4 | 19.4 /
+// 8.4, 1 step 250 x 251 20.5 / 10.4 | 18.6 / 9.0.  Flat grids give the cluster's CTAs
+// few rows each: 50 x 403, 13-point star, 100 steps 171 | 221.
+static bool cluster_run(const stencil_plan* p, int64_t T, bool in_place) {
+    if (!p->grid.plain || p->res_c == 0) return false;
+    const int64_t points = p->ny * p->nx;
+    const bool ragged = p->nx % 4 != 0;
+    if (in_place && (T == 1 || (T == 2 && ragged)) && points <= (T == 1 ? 90000 : 60000)) return true;
+    if (ragged && p->boundary == STENCIL_BOUNDARY_PERIODIC) {
+        if (p->nx > 4 * p->ny) return false;
+        const int64_t any = p->R == 1 ? (p->star ? 0 : 15000) : p->R == 2 && p->star ? 36000 : 65000;
+        return points <= std::max<int64_t>(any, T == 1 ? 65000 : T == 2 ? 36000 : T == 3 ? 20000 : 0);
+    }
+    return T == 1 && points <= (ragged ? 60000 : p->R == 1 ? 36000 : 20000);
 }
 
 static stencil_status_t configure_naive(stencil_plan* p) {
@@ -772,7 +809,7 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
         }
         return STENCIL_OK;
     }
-    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on) {
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && !cluster_run(p, nlev, src == dst)) {
         const size_t vec_bytes = 4 * p->elem;
         const int vec = p->nx % 4 == 0 && (uintptr_t)src % vec_bytes == 0 && (uintptr_t)dst % vec_bytes == 0;
         // In place, a tile may only write once its neighbours have read: at least
@@ -1413,6 +1450,13 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
         g_res_tune_cache[tune_key()] = decision;  // (for the candidates that there were)
     }
     if (decision == kTuneGrid) {
+        if (p->grid.plain) {  // (for cluster_run: the default configuration, not the last one timed)
+            const int C = resident_candidates(p);
+            if (C > 0) {
+                stencil_status_t s = use_resident(p, C);
+                if (s != STENCIL_OK) return s;
+            }
+        }
         use_grid(p);
         return STENCIL_OK;
     }
@@ -1772,7 +1816,7 @@ stencil_status_t stencil_run(stencil_plan_t* p, const void* in, void* out, int64
     }
     std::vector<int> depths = launch_depths(p, T);
     const void* src = in;
-    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && in == out && T == 1) {
+    if (p->kernel == STENCIL_KERNEL_RESIDENT && p->grid_on && in == out && T == 1 && !cluster_run(p, T, true)) {
         // a single step in place has no exchange that orders the reads before the writes
         CK(cudaMemcpyAsync(p->ws, in, bytes, cudaMemcpyDeviceToDevice, st));
         src = p->ws;

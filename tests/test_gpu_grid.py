@@ -203,3 +203,36 @@ def test_launches_of_tiles_autotuned():
     again = _plan(shape, W, grid=False, autotune=True)  # (the cached choice)
     z = _plan(shape, W, grid=False, kernel="stream").run(x, 23)
     assert torch.equal(y, z) and torch.equal(again.run(x, 23), z)
+
+
+# Either side of the lines up to which short runs, and runs of periodic ragged widths,
+# take the cluster-resident kernel from a register-tile plan.
+CLUSTER_SHAPES = [(140, 141), (141, 142), (180, 200), (181, 200), (100, 200), (101, 200), (60, 249), (250, 251),
+                  (255, 257), (50, 201), (50, 199)]
+
+
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+@pytest.mark.parametrize("name", ["heat5", "box9", "star9", "box25", "star13", "box49"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_runs_in_one_cluster_have_the_same_bits(name, boundary, dtype):
+    """One plan's runs of different lengths may take either kernel: the cluster-resident
+    kernel's bits every time, in place as well."""
+    W = _weights(name)
+    for shape in CLUSTER_SHAPES:
+        x = torch.from_numpy(inputs.field(*shape)).cuda().to(TDT[dtype])
+        p = _plan(shape, W, grid=False, boundary=boundary, dtype=dtype)
+        a = _plan(shape, W, grid=False, boundary=boundary, dtype=dtype, autotune=True)
+        q = _plan(shape, W, grid=False, boundary=boundary, dtype=dtype, kernel="resident")
+        for T in (1, 2, 1, 3, 4, 25, 1):
+            want = q.run(x, T)
+            z = x.clone()
+            p.run(z, T, out=z)
+            assert torch.equal(p.run(x, T), want) and torch.equal(z, want), (shape, T)
+        assert torch.equal(p.run(p.run(x, 1), 1), q.run(q.run(x, 1), 1))
+        for T in (1, 2, 25):
+            y = a.run(x, T)
+            if a.info()["kernel"] == 6:  # (autotuning may keep the streaming kernel, whose bits differ)
+                assert torch.equal(y, q.run(x, T)), (shape, T)
+        p.status()
+        for plan in (p, a, q):
+            plan.close()
