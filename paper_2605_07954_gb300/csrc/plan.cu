@@ -652,12 +652,28 @@ static void choose_tiles(stencil_plan* p) {
     if (p->tiles_on) p->warp_nc = 0;
 }
 
-// Whether a launch of nlev steps runs as register tiles.  Aligned launches of a
-// step or two (a run's remainder) are cheaper without the tiles' deep halo:
-// 2048^2, 1 step, 5-point star 15 us as tiles, 12 streaming, 13-point star 19 |
-// 15, 7x7 box 27 | 25; 2 steps 17 | 13, 23 | 17, but 42 | 48.
-static bool tiles_launch(const stencil_plan* p, int nlev, bool vec) {
-    return p->tiles_on && !(vec && nlev <= (p->star ? 2 : 1));
+// Whether a launch of nlev steps runs as register tiles.  Launches of a step or two
+// (a short run, or a run's remainder), and for the 5-point star every depth below 8
+// that the streaming kernel has as one launch, are cheaper without the tiles' deep
+// halo.  Zero rule, among others, us as tiles | streaming: 5-point star 1600^2 3 steps
+// 16.5 | 14.4, 4 17.5 | 16.6, 5 (4 + 1) 18.6 | 28.5, 6 20.7 | 18.6, 8 22.7 | 22.7; 1833 x
+// 1459 1 step 18.4 | 14.6, 2 19.2 | 14.5, 3 20.7 | 16.5, 6 26.0 | 22.7, 8 28.9 | 34.7;
+// 9-point box 1833 x 1459 1 14.5 | 13.6, 2 16.6 | 14.5, 3 18.6 | 18.6, 4 20.7 | 22.7;
+// 9-point star 1 18.6 | 16.5, 2 21.3 | 22.6; 5x5 box 1800 x 2047 1 24.6 | 17.3, 2 29.7 |
+// 23.7, 3 35.5 | 42.3 (1833 x 1459 2 22.7 | 22.9); 13-point star 1833 x 1459 1 20.0 |
+// 16.5, 2 22.7 | 20.6, 3 26.4 | 33.5; 7x7 box 1 27.5 | 26.7, 2 37.2 | 44.5.  Aligned
+// 2048^2: 1 step, 13-point star 19 | 15, 7x7 box 27 | 25; 2 steps 23 | 17, 42 | 48.
+// (Element-wise launches of the 9-point box and of radius 2 gain as whole runs only:
+// behind launches of tiles, 1833 x 1459, 8 + 1 steps, 9-point box 43.1 | 45.2, 5x5 box
+// 4 + 1 51.3 | 53.4.)  Periodic ragged launches stay tiles (see choose_tiles).
+static bool tiles_launch(const stencil_plan* p, int nlev, bool vec, bool whole_run) {
+    if (!p->tiles_on) return false;
+    // (a full launch of a long run, or no streaming launch of that depth in the plan)
+    if ((nlev > 2 && nlev == p->tiles.k) || nlev > p->k || stream_depth_at_most(p->R, p->star, nlev) != nlev) return true;
+    if (vec) return nlev > (p->R == 1 && p->star ? 6 : p->star ? 2 : 1);
+    if (p->boundary == STENCIL_BOUNDARY_PERIODIC) return true;
+    if ((p->R == 2 || (p->R == 1 && !p->star)) && !whole_run) return true;
+    return nlev > (p->R == 1 ? (p->star ? 6 : 2) : p->R == 2 ? (p->star ? 1 : 2) : p->star ? 2 : 1);
 }
 
 static void use_grid(stencil_plan* p) {
@@ -868,7 +884,7 @@ static stencil_status_t launch_once(stencil_plan* p, const void* src, void* dst,
     const size_t vec_bytes = 4 * p->elem;
     sp.vec = (p->nx % 4 == 0) && ((uintptr_t)src % vec_bytes == 0) &&
              ((uintptr_t)dst % vec_bytes == 0);
-    if (tiles_launch(p, nlev, sp.vec)) {
+    if (tiles_launch(p, nlev, sp.vec, first && last)) {
         CK(launch_tiles(p->tiles, p->R, p->star, p->dtype, sp.periodic, src, dst, (int)p->ny, (int)p->nx, sp.vec, nlev,
                         p->w, st));
         return STENCIL_OK;

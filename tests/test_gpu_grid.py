@@ -236,3 +236,31 @@ def test_runs_in_one_cluster_have_the_same_bits(name, boundary, dtype):
         p.status()
         for plan in (p, a, q):
             plan.close()
+
+
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+@pytest.mark.parametrize("name,shape", [("heat5", (1833, 1459)), ("heat5", (1600, 1600)), ("box9", (1601, 1701)),
+                                        ("star9", (2047, 1801)), ("box25", (1800, 2047)), ("star13", (1801, 1804)),
+                                        ("star13", (1800, 2047)), ("box49", (1701, 1601))])
+def test_short_launches_of_tile_plans_have_the_same_bits(name, shape, boundary):
+    """Runs of up to a few steps, and the remainders of longer ones, stream: every count
+    from 1 to one past a launch of tiles, in and out of place."""
+    W = _weights(name)
+    x = torch.from_numpy(inputs.field(*shape)).cuda()
+    p = _plan(shape, W, grid=False, boundary=boundary)
+    q = _plan(shape, W, grid=False, boundary=boundary, kernel="stream")
+    k = p.info()["tb_depth"]
+    want = x
+    for T in range(1, min(k, 12) + 2):
+        z = x.clone()
+        p.run(z, T, out=z)
+        y = p.run(x, T)
+        if boundary == "periodic" and shape[1] % 4:
+            want = q.run(x, T).double()
+            for v in (y, z):
+                assert float((v.double() - want).norm() / want.norm()) <= fp32_tol(T), T
+        else:
+            want = q.run(want, 1)
+            assert torch.equal(y, want) and torch.equal(z, want), T
+    p.close()
+    q.close()
