@@ -1480,6 +1480,26 @@ static stencil_status_t autotune_resident(stencil_plan* p, const void* in, cudaS
     return autotune(p, in, st);
 }
 
+// Clear device memory before returning, without touching the caller's streams:
+// a first run on any stream must see it cleared.
+// (One stream per device, kept for the life of the process: creating one per
+// plan cost more than the rest of the call.)
+static cudaError_t zero_now(int device, void* ptr, size_t bytes) {
+    static std::mutex mu;
+    static std::map<int, cudaStream_t> streams;
+    std::lock_guard<std::mutex> g(mu);
+    cudaStream_t& st = streams[device];
+    cudaError_t e = cudaSuccess;
+    if (!st) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ptr, 0, bytes, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e;
+}
+
+namespace gbst {
+cudaError_t plan_zero_now(const stencil_plan_t* p, void* ptr, size_t bytes) { return zero_now(p->device, ptr, bytes); }
+}  // namespace gbst
+
 extern "C" {
 
 const char* stencil_status_string(stencil_status_t s) {
@@ -1498,22 +1518,6 @@ const char* stencil_status_string(stencil_status_t s) {
 const char* stencil_last_error(void) { return g_last_error.c_str(); }
 
 int stencil_version(void) { return 100; }
-
-// Clear device memory before returning, without touching the caller's streams:
-// a first run on any stream must see it cleared.
-// (One stream per device, kept for the life of the process: creating one per
-// plan cost more than the rest of the call.)
-static cudaError_t zero_now(int device, void* ptr, size_t bytes) {
-    static std::mutex mu;
-    static std::map<int, cudaStream_t> streams;
-    std::lock_guard<std::mutex> g(mu);
-    cudaStream_t& st = streams[device];
-    cudaError_t e = cudaSuccess;
-    if (!st) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ptr, 0, bytes, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return e;
-}
 
 stencil_status_t stencil_plan_create(stencil_plan_t** out, int64_t ny, int64_t nx, int radius,
                                      const float* weights, int dtype, int boundary,

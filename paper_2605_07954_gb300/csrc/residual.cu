@@ -27,11 +27,13 @@ namespace gbst {
 void** plan_aux_slot(stencil_plan_t* p, int id);
 void plan_set_aux_free(stencil_plan_t* p, int id, void (*freer)(void*));
 
+cudaError_t plan_zero_now(const stencil_plan_t* p, void* ptr, size_t bytes);
 bool plan_keep_sums(stencil_plan_t* p, bool on);
 stencil_status_t plan_run_last_two(stencil_plan_t* p, const void* in, void* g1, void* g2, void* g0, int64_t m,
                                    cudaStream_t st, const void** prev, const void** next);
 
-constexpr int kResBlocks = 1024;
+constexpr int kResBlocks = 1024;   // CTAs of a norm at most,
+constexpr int kResBlockTerms = 1024;  // one for so many points (a term each for its threads' first pass)
 
 // A running sum of squared differences, at no less than FP64's accuracy.  FP64 FMAs
 // run at 1/64 of the FP32 rate here, so half of the terms (WIDE) take one of them
@@ -228,9 +230,16 @@ stencil_status_t stencil_run_residual(stencil_plan_t* plan, const void* in, void
             sc->partials = nullptr;
             return rfail(STENCIL_ERR_OOM, "cudaMalloc of the residual scratch failed");
         }
+        // the count of finished blocks starts at 0; every norm leaves it there
+        const cudaError_t e = plan_zero_now(plan, sc->partials + kResBlocks, sizeof(unsigned));
+        if (e != cudaSuccess) {
+            cudaFree(sc->partials);
+            sc->partials = nullptr;
+            return rfail(STENCIL_ERR_CUDA, std::string("clearing the residual scratch: ") + cudaGetErrorString(e));
+        }
     }
     unsigned* finished = reinterpret_cast<unsigned*>(sc->partials + kResBlocks);
-    RCK(cudaMemsetAsync(finished, 0, sizeof(unsigned), st));
+    const unsigned blocks = (unsigned)std::min<long long>(kResBlocks, (n + kResBlockTerms - 1) / kResBlockTerms);
     char* const G[3] = {sc->grids, sc->grids + sc->bytes, sc->count == 3 ? sc->grids + 2 * sc->bytes : nullptr};
     // (residuals resolve the last bits of the states)
     struct KeepSums {
@@ -268,15 +277,15 @@ stencil_status_t stencil_run_residual(stencil_plan_t* plan, const void* in, void
         if (s != STENCIL_OK) return rfail(s, std::string("run: ") + stencil_last_error());
         const int vec = ((uintptr_t)prev | (uintptr_t)next) % (4 * elem) == 0;
         if (info.dtype == STENCIL_F32)
-            residual_kernel<float><<<kResBlocks, 256, 0, st>>>(static_cast<const float*>(prev),
+            residual_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(prev),
                                                                static_cast<const float*>(next), n, vec, sc->partials,
                                                                finished, residuals + j);
         else if (info.dtype == STENCIL_BF16)
-            residual_kernel<__nv_bfloat16><<<kResBlocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(prev),
+            residual_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(prev),
                                                                        static_cast<const __nv_bfloat16*>(next), n, vec,
                                                                        sc->partials, finished, residuals + j);
         else
-            residual_kernel<__half><<<kResBlocks, 256, 0, st>>>(static_cast<const __half*>(prev),
+            residual_kernel<__half><<<blocks, 256, 0, st>>>(static_cast<const __half*>(prev),
                                                                 static_cast<const __half*>(next), n, vec, sc->partials,
                                                                 finished, residuals + j);
         RCK(cudaGetLastError());
