@@ -32,8 +32,16 @@ bool plan_keep_sums(stencil_plan_t* p, bool on);
 stencil_status_t plan_run_last_two(stencil_plan_t* p, const void* in, void* g1, void* g2, void* g0, int64_t m,
                                    cudaStream_t st, const void** prev, const void** next);
 
-constexpr int kResBlocks = 1024;   // CTAs of a norm at most,
-constexpr int kResBlockTerms = 1024;  // one for so many points (a term each for its threads' first pass)
+constexpr int kResBlocks = 1024;  // CTAs of a norm at most
+
+// CTAs of a norm over n points: the last one to finish counts ~3 ns for each, a pass
+// over 1024 points of a CTA takes ~0.7 us unless other CTAs hide it.  Steps with a
+// check each, 9-point box, 608 | 1024 CTAs, us: 1000^2 20.7 | 23.9, 2048^2 28.9 | 30.9,
+// 4096^2 66.2 | 62.2, 8192^2 230 | 210.
+static unsigned residual_blocks(long long n) {
+    const long long many = (n + 8191) / 8192, few = std::min(608LL, (n + 1023) / 1024);
+    return (unsigned)std::min<long long>(kResBlocks, std::max(many, few));
+}
 
 // A running sum of squared differences, at no less than FP64's accuracy.  FP64 FMAs
 // run at 1/64 of the FP32 rate here, so half of the terms (WIDE) take one of them
@@ -239,7 +247,7 @@ stencil_status_t stencil_run_residual(stencil_plan_t* plan, const void* in, void
         }
     }
     unsigned* finished = reinterpret_cast<unsigned*>(sc->partials + kResBlocks);
-    const unsigned blocks = (unsigned)std::min<long long>(kResBlocks, (n + kResBlockTerms - 1) / kResBlockTerms);
+    const unsigned blocks = residual_blocks(n);
     char* const G[3] = {sc->grids, sc->grids + sc->bytes, sc->count == 3 ? sc->grids + 2 * sc->bytes : nullptr};
     // (residuals resolve the last bits of the states)
     struct KeepSums {
