@@ -110,3 +110,15 @@ def test_sums_beyond_fp32_stay_finite(name):
     _, gw = _grads(u0, W, 1, gT, "periodic", "stencil_adjoint_w32")
     _, ref = _grads(u0, W, 1, gT, "periodic", "stencil_adjoint")
     assert np.all(np.isfinite(gw)) and rel_l2(gw / 1e36, ref / 1e36) <= 1e-5
+
+
+@pytest.mark.parametrize("entry", ["stencil_adjoint", "stencil_adjoint_w32"])
+@pytest.mark.parametrize("T", [1, 2, 3])
+@pytest.mark.parametrize("name,shape", [("heat5", (945, 1700)), ("star13", (1000, 1022)), ("box25", (900, 1000))])
+def test_few_steps(name, shape, T, entry):
+    """One or two recomputed states: the gradients of a streaming plan, bit for bit."""
+    W = _weights(name)
+    u0 = inputs.field(*shape)
+    gT = (inputs.field(*shape, stream=inputs.STREAM_TARGET) - 0.5).astype(np.float32)
+    for a, b in zip(_grads(u0, W, T, gT, "zero", entry), _grads(u0, W, T, gT, "zero", entry, kernel="stream")):
+        assert np.array_equal(a, b)
