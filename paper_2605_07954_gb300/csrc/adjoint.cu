@@ -50,6 +50,7 @@ void plan_set_stream(stencil_plan_t* p, cudaStream_t st);
 bool plan_keep_sums(stencil_plan_t* p, bool on);
 bool plan_states_vary(const stencil_plan_t* p);
 bool plan_states_one_launch(const stencil_plan_t* p, bool any_order);
+int plan_states_depth(const stencil_plan_t* p);
 int64_t plan_sum_launches(const stencil_plan_t* p, int64_t T);
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
                                  cudaStream_t st);
@@ -974,7 +975,7 @@ int64_t stencil_adjoint_launches(const stencil_plan_t* plan, int64_t T, int64_t 
             L += m * step;
             continue;
         }
-        const int top = info.radius == 3 && !info.shape ? 2 : (info.radius == 1 ? 8 : 4);
+        const int top = plan_states_depth(plan);
         for (int d = top; d >= 1 && m > 0; d /= 2)
             while (m >= d) {
                 m -= d;

@@ -1131,6 +1131,14 @@ bool plan_states_one_launch(const stencil_plan_t* p, bool any_order) {
            p->dtype == STENCIL_F32 && !(p->boundary == STENCIL_BOUNDARY_PERIODIC && p->nx % 4 != 0);
 }
 
+// Most states of one all-states launch.  The 5-point star's CTA-wide kernel stores eight
+// levels at a higher cost than twice four (gradients of 33 steps, 8 | 4 levels, us: 1032 x
+// 2712 725 | 628, 2048^2 799 | 674, 1500 x 4000 1008 | 883), its one-warp tiles do not.
+int plan_states_depth(const stencil_plan_t* p) {
+    if (p->R == 1) return p->star && warp_tiles(p, 4).by < kWarpMinRows ? 4 : 8;
+    return p->R == 3 && !p->star ? 2 : 4;
+}
+
 stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const* outs, int64_t n, bool any_order,
                                  cudaStream_t st) {
     bool fused = p->dtype == STENCIL_F32 && p->nx % 4 == 0 && (uintptr_t)in % 16 == 0;
@@ -1161,7 +1169,7 @@ stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const
     }
     const void* src = in;
     for (int64_t i = 0; i < n;) {
-        int d = 8;
+        int d = plan_states_depth(p);
         for (; d > 1; d /= 2)
             if (d <= n - i && get_stream_states_kernel(p->R, p->star, d).fn) break;
         stencil_status_t s = launch_states(p, src, outs + i, d, st);

@@ -268,10 +268,10 @@ def test_counting_launches_leaves_the_plan_alone():
 
 
 @pytest.mark.parametrize("name", ["heat5", "box9"])
-@pytest.mark.parametrize("shape,boundary", [((4096, 4096), "zero"), ((6000, 3036), "periodic")])
+@pytest.mark.parametrize("shape,boundary", [((4096, 4096), "zero"), ((6000, 3036), "periodic"), ((1352, 2088), "zero")])
 def test_eight_states_a_launch_have_the_bits_of_four(name, shape, boundary):
-    """Large radius-1 grids: launches that store eight states (one-warp tiles for the star,
-    the CTA-wide kernel for the box) against launches of four and two."""
+    """Radius-1 grids: launches that store up to eight states (one-warp tiles for the star
+    where they have the rows, the CTA-wide kernel for the box) against launches of four and two."""
     from paper_2605_07954_gb300 import Plan, adjoint
     W = inputs.pattern_weights(name)
     g = torch.Generator(device="cuda")
