@@ -847,10 +847,16 @@ stencil_status_t adjoint_run(stencil_plan_t* plan, const void* u0, const void* g
     // any-width one.
     const bool streamed = adjoint_stream_kernel_fn(R) != nullptr && nx % 4 == 0;
     // (a star's off-axis weights are zero: adjoint_rows_kernel skips them in the lambda
-    // update.  Small boxes have too few of its 120 x 32 tiles: 7x7, 32 steps, 96 x 100
-    // 854 us staged, 920 by rows; 160^2 855 | 409, register-tile states included)
+    // update.)  Small grids have too few of its 120 x 32 tiles to hide their latency, and
+    // periodic ragged rows load element by element.  A step's time less the staged
+    // kernel's, us: radius 3 256^2 +2, 256 x 259 +4 (periodic +8), 500^2 +2, 600^2 -4, 600 x
+    // 603 -2 (periodic +2), 800 x 803 periodic -3, 1000^2 -14; radius 2 400^2 0, 500 x 503 +2
+    // (periodic +6), 800^2 -1 to -3, 800 x 803 -1 (periodic +2), 1000^2 -4, 1000 x 1003
+    // periodic 0.
     const bool star = adj_star(wf, R);
-    const bool rows = w32 && R > 1 && (star || n > 20000);
+    const bool wrapped = nx % 4 != 0 && info.boundary == STENCIL_BOUNDARY_PERIODIC;
+    const size_t rows_from = R == 3 ? (wrapped ? 450000 : 300000) : (wrapped ? 1000000 : 500000);
+    const bool rows = w32 && R > 1 && n >= rows_from;
     const int tile_cols = streamed ? kAdsCols : rows ? kAdrCols : kAdjTX;
     const int tiles_x = (nx + tile_cols - 1) / tile_cols;
     const int tile_rows = streamed ? kAdsWarps * kAdsRows : rows ? kAdrWarps * kAdrRows : kAdjTY;

@@ -88,14 +88,14 @@ def test_fp64_sums_keep_their_bits(name, shape, boundary):
 @pytest.mark.parametrize("boundary,nx", [("zero", 361), ("periodic", 361), ("periodic", 364)])
 @pytest.mark.parametrize("col", [117, 119, 120, 122, 239, 240, 355, 360])
 def test_an_infinite_lambda_gives_infinite_sums(name, boundary, nx, col):
-    """One infinite lambda times positive u: every tap's sum is infinite, not NaN, next
+    """(Grids large enough for the kernel in registers.)  One infinite lambda times positive u: every tap's sum is infinite, not NaN, next
     to the columns where a warp's strip ends and beside the grid's last column too."""
     if boundary == "zero" and col + 3 >= nx:
         col = nx - 4  # (nearer the edge the term u~ = 0 beyond it is 0 x inf)
     W = _weights(name)
-    u0 = inputs.field(200, nx) + np.float32(0.5)
-    gT = np.zeros((200, nx), dtype=np.float32)
-    gT[100, col] = np.inf
+    u0 = inputs.field(2800, nx) + np.float32(0.5)
+    gT = np.zeros((2800, nx), dtype=np.float32)
+    gT[1400, col] = np.inf
     for entry in ("stencil_adjoint_w32", "stencil_adjoint"):
         _, gw = _grads(u0, W, 1, gT, boundary, entry)
         assert np.all(np.isposinf(gw)), entry
@@ -105,8 +105,8 @@ def test_an_infinite_lambda_gives_infinite_sums(name, boundary, nx, col):
 def test_sums_beyond_fp32_stay_finite(name):
     """Lambdas of 1e36: the sums of 128 lanes leave the FP32 range, their FP64 sum does not."""
     W = _weights(name)
-    u0 = inputs.field(200, 362) + np.float32(0.5)
-    gT = np.full((200, 362), 1e36, dtype=np.float32)
+    u0 = inputs.field(2800, 362) + np.float32(0.5)
+    gT = np.full((2800, 362), 1e36, dtype=np.float32)
     _, gw = _grads(u0, W, 1, gT, "periodic", "stencil_adjoint_w32")
     _, ref = _grads(u0, W, 1, gT, "periodic", "stencil_adjoint")
     assert np.all(np.isfinite(gw)) and rel_l2(gw / 1e36, ref / 1e36) <= 1e-5
@@ -122,3 +122,20 @@ def test_few_steps(name, shape, T, entry):
     gT = (inputs.field(*shape, stream=inputs.STREAM_TARGET) - 0.5).astype(np.float32)
     for a, b in zip(_grads(u0, W, T, gT, "zero", entry), _grads(u0, W, T, gT, "zero", entry, kernel="stream")):
         assert np.array_equal(a, b)
+
+
+# Either side of the sizes from which the reverse step keeps its rows in registers, and
+# widths that cut its strips of 120 columns and its chunks of 4.
+@pytest.mark.parametrize("name", ["star9", "box25", "star13", "box49"])
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+@pytest.mark.parametrize("shape", [(600, 499), (600, 500), (600, 501), (901, 499), (902, 499), (1000, 501), (1253, 364),
+                                   (2779, 361), (8400, 120), (8500, 121)])
+def test_gradients_of_larger_grids(oracle, name, boundary, shape):
+    W = _weights(name)
+    u0 = inputs.field(*shape)
+    T = 2
+    gT = (inputs.field(*shape, stream=inputs.STREAM_TARGET) - 0.5).astype(np.float32)
+    ref_u, ref_w = oracle.adjoint_f64(u0, W, T, gT.astype(np.float64), boundary)
+    gu, gw = _grads(u0, W, T, gT, boundary, "stencil_adjoint_w32")
+    assert np.linalg.norm(gu - ref_u) <= 1e-5 * np.linalg.norm(ref_u)
+    assert np.linalg.norm(gw - ref_w) <= 1e-5 * np.linalg.norm(ref_w)
