@@ -103,13 +103,16 @@ class Plan:
 
     def run(self, x, T: int, out=None):
         """u_T from u_0 = x (device tensor); enqueued on torch's current stream."""
+        return self._run(x, T, out, None)
+
+    def _run(self, x, T, out, stream):
         torch = self._check_tensor(x)
         if out is None:
             out = torch.empty_like(x)
         else:
             self._check_tensor(out)
         check(_capi.load().stencil_run(self._h, x.data_ptr(), out.data_ptr(), int(T),
-                                       _current_stream_handle()), "stencil_run")
+                                       _current_stream_handle() if stream is None else stream), "stencil_run")
         return out
 
     def run_residual(self, x, T: int, m: int, out=None):
@@ -187,14 +190,14 @@ class _PlanCache:
         self.lock = threading.Lock()
 
     def get(self, device: int, ny: int, nx: int, W: np.ndarray, boundary: str, stream: int = 0,
-            capturing: bool = False) -> Plan:
+            capturing=lambda: False) -> Plan:
         r = W.shape[0] // 2
         star = bool(np.all(W[np.arange(W.shape[0]) != r][:, np.arange(W.shape[1]) != r] == 0))
         what = (ny, nx, r, star, boundary)
         key = (device, stream) + what
         with self.lock:
             plan = self.plans.pop(key, None)
-            if plan is None and capturing:
+            if plan is None and capturing():
                 other = next((k for k in reversed(self.plans) if k[0] == device and k[2:] == what), None)
                 plan = self.plans.pop(other, None)
             if plan is None:
@@ -216,28 +219,31 @@ def _stencil_fn():
     import torch
 
     class StencilFn(torch.autograd.Function):
-        """u_T = A^T u0 with gradients for u0 and the weights (sqrt(T) checkpointing).
+        """u_T = A^T u0 with gradients for u0 and the weights.
 
         apply(u0, weights, T, boundary="zero", ckpt_interval=0): u0 a CUDA FP32
         tensor; weights a (2r+1, 2r+1) tensor on any device (its values are read
         at forward time).  The weight gradient has the weights' dtype and device.
         Plans come from a small per-process cache (see _PlanCache), one per stream
         and shape, so repeated calls with new weights allocate nothing new, and
-        calls on several streams or threads run side by side.  The backward pass uses the
-        weights of its own forward call, read back from the saved copy.
+        calls on several streams or threads run side by side.  A plan's backward
+        scratch lies outside torch's allocator: all T states while they take at most
+        1 GiB, else about 2 sqrt(T) grids; ckpt_interval = s makes it T/s + s grids.
+        The backward pass uses the weights of its own forward call, read back from
+        the saved copy.
         """
 
         @staticmethod
         def forward(ctx, u0, weights, T, boundary="zero", ckpt_interval=0):
             W = np.ascontiguousarray(weights.detach().to("cpu", torch.float32).numpy())
             on_gpu = u0.is_cuda
-            plan = _PLANS.get(u0.device.index if on_gpu else -1, u0.shape[0], u0.shape[1], W, boundary,
-                              _current_stream_handle() if on_gpu else 0,
-                              on_gpu and torch.cuda.is_current_stream_capturing())
+            stream = _current_stream_handle() if on_gpu else 0
+            plan = _PLANS.get(u0.device.index if on_gpu else -1, u0.shape[0], u0.shape[1], W, boundary, stream,
+                              lambda: on_gpu and torch.cuda.is_current_stream_capturing())
             u0c = u0.detach().contiguous()
             with plan.lock:
                 plan.set_weights(W)
-                y = plan.run(u0c, int(T))
+                y = plan._run(u0c, int(T), None, stream)
             ctx.save_for_backward(u0c)
             ctx.plan, ctx.W, ctx.T, ctx.ckpt = plan, W, int(T), int(ckpt_interval)
             ctx.wdtype, ctx.wdevice = weights.dtype, weights.device

@@ -59,6 +59,6 @@ def test_every_stream_has_its_own_plans(cache):
 def test_a_captured_call_allocates_nothing(cache):
     """A call under capture takes over the plan that a warm-up on another stream made."""
     a = cache.get(0, 10, 10, W3, "zero", stream=1)
-    assert cache.get(0, 10, 10, W3, "zero", stream=9, capturing=True) is a
+    assert cache.get(0, 10, 10, W3, "zero", stream=9, capturing=lambda: True) is a
     assert cache.get(0, 10, 10, W3, "zero", stream=9) is a
     assert cache.get(0, 10, 10, W3, "zero", stream=1) is not a
