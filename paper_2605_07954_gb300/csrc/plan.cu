@@ -693,6 +693,9 @@ static void use_grid(stencil_plan* p) {
 // 8.3, 300^2 11.4 | 9.4, 7x7 box 300^2 12.4 | 12.4; two steps in place 260 x 161 10.4 |
 // 8.4, 300 x 201 10.4 | 9.2, 200^2 8.8 | 8.3.
 //
+// 7x7 boxes on narrow grids, of which a strip holds little but halo, 100 steps: 256 x 96
+// 159 | 154, 400 x 64 160 | 154, 700 x 40 191 | 163, 200 x 128 155 | 158, 800 x 64 188 | 214.
+//
 // Periodic ragged widths: the tiles read their halos element by element through the
 // wrap, twice the cost of an exchange, and the more of a tile is halo the worse.
 // 100 steps, register tiles | cluster: 13-point star 60 x 61 192 | 131, 300 x 110
@@ -713,6 +716,7 @@ static bool cluster_run(const stencil_plan* p, int64_t T, bool in_place) {
         const int64_t any = p->R == 1 ? (p->star ? 0 : 15000) : p->R == 2 && p->star ? 36000 : 65000;
         return points <= std::max<int64_t>(any, T == 1 ? 65000 : T == 2 ? 36000 : T == 3 ? 20000 : 0);
     }
+    if (p->R == 3 && !p->star && points <= 28000 && p->nx <= 112) return true;
     return T == 1 && points <= (ragged ? 60000 : p->R == 1 ? 36000 : 20000);
 }
 

@@ -208,7 +208,7 @@ def test_launches_of_tiles_autotuned():
 # Either side of the lines up to which short runs, and runs of periodic ragged widths,
 # take the cluster-resident kernel from a register-tile plan.
 CLUSTER_SHAPES = [(140, 141), (141, 142), (180, 200), (181, 200), (100, 200), (101, 200), (60, 249), (250, 251),
-                  (255, 257), (50, 201), (50, 199)]
+                  (255, 257), (50, 201), (50, 199), (250, 112), (251, 112)]
 
 
 @pytest.mark.parametrize("boundary", ["zero", "periodic"])
