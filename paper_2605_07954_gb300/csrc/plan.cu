@@ -319,7 +319,8 @@ static StreamKernelRef pad_kernel(const stencil_plan* p, int k) {
 // periodic 1012 | 1225, 1768 | 1801, 4001 x 5003 459 | 528, 671 | 692.
 static bool pad_eligible(const stencil_plan* p);
 constexpr int kWarpDepth = 8;
-constexpr int kWarpMinRows = 44;      // NC = 4
+constexpr int kWarpMinRows = 44;      // NC = 4, 5-point star
+constexpr int kWarpMinRowsBox = 52;   // 9-point box (7000 x 1901, 49 rows, 544 | 526; 5200 x 2600, 52 rows, 486 | 491)
 constexpr int kWarpMinRowsWide = 128;  // NC = 8: fewer warps, so taller tiles before it pays
 
 struct WarpTiles {
@@ -329,10 +330,19 @@ struct WarpTiles {
 // One wave of one-warp tiles with nc columns per lane.
 static WarpTiles warp_tiles(const stencil_plan* p, int nc) {
     const int64_t bx_max = 32 * nc - 2 * kWarpDepth;
-    const int64_t bx = ceil_div(ceil_div(p->nx, ceil_div(p->nx, bx_max)), nc) * nc;
+    int64_t bx = ceil_div(ceil_div(p->nx, ceil_div(p->nx, bx_max)), nc) * nc;
+    // (a last strip narrower than the halo columns does the same to the strip beside it as
+    // a low last tile row, below: 9-point box, 64 steps, 8192 x 8180, 4 columns left over,
+    // 2246 us, 8192 x 8184 1805; 5-point star 1457, 8192 x 8188 1255)
+    while (bx > nc && bx < p->nx && p->nx % bx != 0 && p->nx % bx < kWarpDepth) bx -= nc;
     const int64_t strips = ceil_div(p->nx, bx);
     const int64_t warps = (int64_t)p->sms * (nc == 8 ? 8 : 16);
-    const int64_t by = ceil_div(p->ny, std::max<int64_t>(1, warps / strips));
+    int64_t by = ceil_div(p->ny, std::max<int64_t>(1, warps / strips));
+    // A last tile row of fewer rows than a tile loads beyond its own puts the whole row of
+    // tiles above it on the path that checks for the grid's edge, and those set the time
+    // of the wave: 9-point box, 64 steps, 7192 x 2000 613 us with 10 rows left over, 7193 x
+    // 2000 509 with 11.
+    while (by < p->ny && p->ny % by != 0 && p->ny % by < kWarpDepth + 3) ++by;
     return {(int)bx, (int)by, (int)strips, (int)ceil_div(p->ny, by)};
 }
 
@@ -346,7 +356,7 @@ static void configure_warp(stencil_plan* p, int threads_asked) {
     for (int nc = p->star ? 8 : 4; nc >= 4; nc -= 4) {
         if (nc == 8 && p->nx % 8 != 0) continue;
         const WarpTiles t = warp_tiles(p, nc);
-        if (t.by < (nc == 8 ? kWarpMinRowsWide : kWarpMinRows)) continue;
+        if (t.by < (nc == 8 ? kWarpMinRowsWide : p->star ? kWarpMinRows : kWarpMinRowsBox)) continue;
         p->warp_nc = nc;
         p->warp_bx = t.bx;
         p->warp_by = t.by;

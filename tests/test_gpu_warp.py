@@ -61,3 +61,24 @@ def test_wide_chunks_only_where_no_chunk_is_cut(nx, columns):
     assert torch.equal(p.run(x, 17), q.run(x, 17))
     p.close()
     q.close()
+
+
+@pytest.mark.parametrize("name", ["heat5", "box9"])
+@pytest.mark.parametrize("ny,nx", [(7192, 2000), (7050, 2000), (7186, 2001), (4100, 4096), (4096, 4372),
+                                   (8192, 8180), (8000, 2020), (8000, 1801)])
+def test_the_last_tiles_are_large_enough(name, ny, nx):
+    """Tile sizes that would leave a last row of tiles lower than the 11 rows, or a last
+    strip narrower than the 8 columns, that the tiles beside them read beyond their own
+    are changed; the bits are the CTA-wide kernel's."""
+    from paper_2605_07954_gb300 import Plan
+    W = inputs.pattern_weights(name)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    x = torch.rand((ny, nx), generator=g, device="cuda")
+    p, q = Plan(ny, nx, W), Plan(ny, nx, W, threads=128 if name == "heat5" else 64)
+    i = p.info()
+    assert i["threads"] == 32 and (ny % i["tile_rows"] == 0 or ny % i["tile_rows"] >= 11), i
+    assert nx % i["tile_cols"] == 0 or nx % i["tile_cols"] >= 8, i
+    assert torch.equal(p.run(x, 17), q.run(x, 17))
+    p.close()
+    q.close()
