@@ -116,7 +116,12 @@ typedef enum {
  * the one-cluster form; tb_depth then sets its steps per halo exchange
  * (default 1).  stencil_plan_info reports tb_depth = 0 for RESIDENT (one launch
  * per run), ctas = the cluster size (1 for register tiles, whose CTAs are not
- * clustered) and tile_rows = the height of a slab or tile. */
+ * clustered) and tile_rows = the height of a slab or tile.  Register-tile plans of
+ * grids that fit one cluster run short runs, and runs of small periodic grids whose
+ * width is not a multiple of 4, in one cluster all the same (same bits).
+ * Register tiles use every SM.  Programs that keep eight or more small plans (up to
+ * about 512 x 512) busy on streams of their own get up to twice the throughput from
+ * kernel = RESIDENT, at most 16 SMs a plan, or from a batch (stencil_batch_create). */
 typedef struct {
     int compute;      /* stencil_compute_t                                          */
     int kernel;       /* stencil_kernel_t                                           */
@@ -208,7 +213,9 @@ stencil_status_t stencil_plan_info(const stencil_plan_t* plan, stencil_plan_info
  *             read.  in == out is allowed.  Other partial overlap is an error
  *             the library cannot detect.
  *   T         >= 0.  T == 0 copies in to out.
- * Launches ceil(T/k) kernels (k = tb_depth, +1 if in == out and that count is odd).
+ * Launches ceil(T/k) kernels (k = tb_depth, +1 if in == out and that count is odd);
+ * RESIDENT plans one; streaming plans of the zero rule whose width is not a multiple
+ * of 4 one more, which pads the rows, when that makes two or more.
  */
 stencil_status_t stencil_run(stencil_plan_t* plan, const void* in, void* out, int64_t T,
                              stencil_stream_t stream);
@@ -244,8 +251,8 @@ stencil_status_t stencil_plan_status(stencil_plan_t* plan);
 /*
  * T steps with a convergence check every m steps (the paper's periodic
  * convergence checks, Sec. IV).  After every m-th step t (t = m, 2m, ... <= T)
- * residuals[t/m - 1] = || u_t - u_{t-1} ||_2 over the whole grid (FP64,
- * deterministic).  Same operation, arguments and result bits as stencil_run
+ * residuals[t/m - 1] = || u_t - u_{t-1} ||_2 over the whole grid (summed with at
+ * least FP64's accuracy and range, deterministic).  Same operation, arguments and result bits as stencil_run
  * (periodic grids with nx % 4 != 0: the same values up to rounding, since
  * their results depend on the launch depths at the rounding level).
  *   residuals  DEVICE, floor(T/m) doubles, written.
@@ -278,6 +285,7 @@ const char* stencil_residual_last_error(void);
  *                  T + 3 grids take at most 1 GiB, else about sqrt(T) (always sqrt(T)
  *                  for grids small enough for the cluster-resident kernel).  The result
  *                  does not depend on it (same bits).
+ *                  Set it to bound the scratch (next paragraph).
  * States are recomputed from checkpoints, not stored: the plan allocates and
  * keeps (ceil(T/s) + s + 2) grids of scratch, s = ckpt_interval.  The weight
  * gradient is reduced deterministically (fixed order, FP64 partials).

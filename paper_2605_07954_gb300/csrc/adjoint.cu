@@ -23,8 +23,8 @@
 // sums the partials over tiles in a fixed order.  The gradient is deterministic.
 // adjoint_stream_kernel is that step for radius 1 and widths a multiple of 4;
 // for everything else adjoint_step_kernel, or, where the caller rounds the weight
-// gradient to FP32 (stencil_adjoint_w32) and the radius is 2 or 3, the faster
-// adjoint_rows_kernel.
+// gradient to FP32 (stencil_adjoint_w32), the radius is 2 or 3 and the grid has enough
+// tiles for it (adjoint_run), the faster adjoint_rows_kernel.
 //
 // The FP64 weight gradient of stencil_adjoint is tied to the bits of the states, so
 // where those depend on how steps are grouped they come from the streaming kernel
@@ -72,7 +72,8 @@ stencil_status_t plan_run_states(stencil_plan_t* p, const void* in, float* const
 // (TwoSum) before they go into its FP64 partial; that keeps the FP32 part no
 // longer than the staged-tile form's 8 products and 5 levels of lane sums.
 //
-// What bounds it: FMA issue, (13 or 49) + 49 FMAs per point for radius 3.  The
+// What bounds it: latency; two warps a scheduler have (13 or 49) + 49 FMAs per point
+// for radius 3 to issue (13-point star 1000 x 1022: issue 39 %, FMA pipe 23 %).  The
 // staged-tile form (one point per lane and row, both windows read
 // from shared memory) ran the 13-point star at 1000 x 1022 in 26.4 us a step:
 // now 14.4 (ncu).

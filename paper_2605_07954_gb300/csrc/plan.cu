@@ -600,7 +600,10 @@ static stencil_status_t use_resident(stencil_plan* p, int C, int kb = 1) {
 // 111 | 322, 212 | 371; 13-point star 97 | 658, 211 | 658, 1400^2 423 | 725; 7x7
 // box 183 | 1478, 433 | 1379, 1400^2 743 | 1575; 4 steps 11-38 | 16-67.  Against
 // the cluster-resident kernel: 512^2 5-point star, 100 steps, 52 | 219 (FP32);
-// 130 x 517 13-point star, 20 steps, 24 | 74.  A plan the caller steers (kernel,
+// 130 x 517 13-point star, 20 steps, 24 | 74.  (Shorter runs and periodic ragged widths:
+// cluster_run below.)  That is one run at a time: tiles use every SM, so eight or more
+// small plans on streams of their own ran up to twice as fast in one cluster each (9-point
+// box 256^2, 100 steps, us per run with 1, 4, 8 plans: 55 | 116, 36 | 30, 36 | 19).  A plan the caller steers (kernel,
 // tb_depth, threads, tile_rows or load set) keeps what it asked for.
 static bool grid_candidate(stencil_plan* p) {
     if (p->compute != STENCIL_COMPUTE_FP32 || p->ny > (1 << 20) || p->nx > (1 << 20)) return false;

@@ -32,9 +32,10 @@
 // zero rows, and only tiles whose edge cuts a lane's chunk or a warp's rows mask
 // what they compute.
 //
-// What bounds it.  The instruction issue of k steps (for the 5-point star about
-// 120 warp instructions per warp and step for 80 cycles of FMA pipe) plus one
-// exchange of ~1.5 us per group; the cost model in sweep_grid.cu weighs the two.
+// What bounds it.  Latency: one CTA barrier per step for two to five warps a scheduler
+// and one exchange of ~1.5 us per group (5-point star 1024^2: about 120 warp
+// instructions per warp and step, 154 with the exchanges, issue 44 %, FMA pipe 31 %;
+// 13-point star 512^2 41 %, 28 %); the cost model in sweep_grid.cu weighs the two.
 // The cluster-resident kernel runs such grids on at most 16 SMs at ~0.7 us of
 // cluster barrier per step, the streaming kernel at 15-20 us of launch, pipeline
 // fill and drain per k steps.  Measured (FP32, GB300): 5-point star 1024^2, 1000
